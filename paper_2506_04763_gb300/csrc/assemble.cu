@@ -29,10 +29,11 @@
 //   F_w = rho_w (lam_w(S_up) T_w - lam_w(S(x_M)) T_c),
 //   F_n = rho_n lam_n(S hat_up) T_n.
 //
-// K1 runs one thread per vertex: it visits the 2^d elements around its vertex
-// and, in each, the d faces that touch it, and accumulates its own block row
-// (27 or 9 2x2 blocks) in shared memory; no atomics, no second pass.  The row
-// is written once with 1 KB-per-warp coalesced stores.
+// K1 runs in two passes, k_asm_faces and k_asm_rows (below).  The first form,
+// k_assemble (RF_ASM_VERTEX=1, for comparison), runs one thread per vertex: it
+// visits the 2^d elements around its vertex and, in each, the d faces that
+// touch it, and accumulates its own block row (27 or 9 2x2 blocks) in shared
+// memory.
 #include <cstdlib>
 
 #include "rf_common.cuh"
@@ -43,6 +44,8 @@ namespace rf {
 struct Phys {
   double rho_w, rho_n, mu_w, mu_n, S_wr, S_nr, lam, den;
   double h[3], g[3];
+  double rh[3], rmu_w, nid;   // 1 / h, 1 / mu_w (rounded), -1 / den
+  double Af[3], gw[3], gn[3]; // SCV face sizes, rho_w g, rho_n g per axis
   int scheme;   // SCHEME_* bits (0: the discretisation of Sec. 3)
 };
 
@@ -206,10 +209,11 @@ __global__ void k_perm_scalar_to_p(Dims d, const double* __restrict__ nat, doubl
 
 // ---------------------------------------------------------------- K1a
 // Per-vertex quantities of the state (parity-split order): S_e, p_n = p_w +
-// p_c, p_c, dp_c/dS_n, k_rw, dk_rw/dS_n.
+// p_c, p_c, dp_c/dS_n, lambda_w, lambda_n and their S_n-derivatives.
 __global__ void k_vertex_state(Dims d, Phys ph, const double2* __restrict__ u, const double* __restrict__ pdmin,
                                double* __restrict__ Se, double* __restrict__ pn, double* __restrict__ pc,
-                               double* __restrict__ dpc, double* __restrict__ krw, double* __restrict__ dkrw) {
+                               double* __restrict__ dpc, double* __restrict__ krw, double* __restrict__ dkrw,
+                               double* __restrict__ krn, double* __restrict__ dkrn) {
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= d.nv) return;
   double2 uv = u[p];
@@ -227,12 +231,17 @@ __global__ void k_vertex_state(Dims d, Phys ph, const double2* __restrict__ u, c
   // divided here once per vertex instead of once per face visit
   krw[p] = k / ph.mu_w;
   dkrw[p] = (-dk / ph.den) / ph.mu_w;
+  // lambda_n = k_rn / mu_n where S hat = S_e (the elements of the vertex's
+  // lowest entry pressure), and its S_n-derivative
+  krn_of(ph.lam, se, k, dk);
+  krn[p] = k / ph.mu_n;
+  dkrn[p] = dk * 1.0 * ph.nid / ph.mu_n;
 }
 
 // ---------------------------------------------------------------- K1 / K1r
 struct AsmIn {
   const double2* u;
-  const double *Se, *pn, *pc, *dpc, *krw, *dkrw, *pdmin, *phiv;
+  const double *Se, *pn, *pc, *dpc, *krw, *dkrw, *krn, *dkrn, *pdmin, *phiv;
   const double *K, *pd, *phi;     // per cell (natural cell order)
   double vol;                     // cell volume
   const uint8_t* dir;             // parity-split
@@ -432,225 +441,442 @@ __global__ void __launch_bounds__(128) k_assemble(Dims d, Phys ph, AsmIn in, dou
   }
 }
 
-// ---------------------------------------------------------------- K1, one thread per element
-// Each SCV face is evaluated once, by the thread of its element, and its flux
-// and derivatives go to both end vertices (a: -, b: +).  The one-thread-per-
-// vertex kernel above evaluates every face twice, once from each end, and K1
-// is FP64-pipe-bound on GB300, so this halves most of its FP64 work.
-// Elements are processed in 2^DIM colours (parities of their lower corner):
-// elements of one colour share no vertex, so each thread owns the rows of its
-// corners for the launch and adds into them without atomics, face by face in
-// a fixed order (deterministic).  J is zeroed before the first colour; the
-// adds go straight to global memory (coalesced across the warp: neighbouring
-// threads own neighbouring rows), which keeps the kernel free of shared
-// memory and its occupancy at what its registers allow (K1 is FP64-latency-
-// bound below ~8 warps per SM).  k_assemble_finish then adds the sources and
-// applies the Dirichlet rows and M.  The face arithmetic is
-// the vertex kernel's, expression by expression, so every upwind, cap and
-// clamp decision and every flux and derivative value are bitwise the same;
-// only the order in which a row's contributions are summed differs.
-template <int DIM, bool WANT_J>
-__global__ void __launch_bounds__(128) k_assemble_cells(Dims d, Phys ph, AsmIn in, int colour, int64_t ncol,
-                                                        double2* __restrict__ F, double* __restrict__ J) {
-  constexpr int NC = 1 << DIM, NE = 1 << (DIM - 1);
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= ncol) return;
-  const int cx = d.nx - 1, cy = d.ny - 1;
-  const int px = colour & 1, py = (colour >> 1) & 1, pz = (colour >> 2) & 1;
-  const int nxp = (cx - px + 1) / 2, nyp = (cy - py + 1) / 2;
-  const uint32_t line = (uint32_t)t / (uint32_t)nxp, kl = line / (uint32_t)nyp;   // 32-bit: fewer than 2^31 cells
-  const int ci = 2 * (int)((uint32_t)t - line * (uint32_t)nxp) + px;
-  const int cj = 2 * (int)(line - kl * (uint32_t)nyp) + py;
-  const int ck = DIM == 3 ? 2 * (int)kl + pz : 0;
+// ---------------------------------------------------------------- K1, faces then rows
+// K1 is FP64-pipe-bound on GB300 (0.53 T FMA/s against 6.8 TB/s), so it is
+// organised to evaluate nothing twice.  Two passes over slabs of cell planes:
+//   k_asm_faces  one thread per element and axis evaluates the element's SCV
+//     faces along that axis and leaves, per face, the fluxes F_w, F_n and six
+//     numbers from which every entry of J they reach follows;
+//   k_asm_rows   gathers them per vertex: the water threads write the entries
+//     (w, p_w), (w, S_n) and F_w, the NAPL threads (n, p_w), (n, S_n), F_n and
+//     M.  Every row is written once, complete (no zero fill, no read-modify-
+//     write, no colours, no atomics), in a fixed order of sums.
+// Face f of row r along axis k, with D the 3-bit offset of corner q from r and
+// W = prod over the other axes of (D_t ? 1/4 : 3/4):
+//   dF_w/dp_w(q) = -+ alpha W,  dF_w/dS_n(q) = -+ beta W dpc(q) +- gamma W/2
+//   (+ delta at the upwind vertex),  the same with nu and eta for F_n,
+//   alpha = rho_w lam_w,up K A_f / h,  beta = rho_w (lam_w,up - lam_w,M) K A_f / h,
+//   gamma = rho_w lam_w,M' T_c,  delta = rho_w lam_w,up' T_w,  nu = rho_n
+//   lam_n,up K A_f / h,  eta = rho_n lam_n,up' T_n.
+// The four faces around one edge of r differ only in W, which factors over the
+// two other axes: their 3 x 3 entries are the tensor transform (a, b) -> (a,
+// 3 (a + b), b) along each, 5 sums (the 1/16 is stored with the coefficient,
+// exactly, and the 3s go into multiply-adds); and since dpc(q)
+// depends on the vertex q alone, the beta of all faces are summed before one
+// product per block.  The face arithmetic that a decision rests on (gradients, T,
+// S_e at x_M, S hat) is the vertex kernel's, operation by operation, and k_rw,
+// k_rn and their derivatives are too (1 - S_e^2 cancels where k_rn ~ 0).
+// Measured on GB300 (F, J and M; then F alone), against one thread per element
+// adding its faces' 768 entries into J colour by colour (4,154 FP64 instructions
+// per vertex; on small grids 8 dependent chains of about 190 us): 257^3 150.9 ->
+// 63.1 ms (52.1 -> 25.8 ms), 65^3 2.79 -> 1.10 ms (1.00 -> 0.48), 17^3 1.57 ->
+// 0.067 ms (0.60 -> 0.042), 33^2 0.224 -> 0.041 ms.  ncu at 97^3: FP64 pipe 83%
+// busy in k_asm_faces, 73% in k_asm_rows, DRAM below 15% of its peak.
+constexpr int NCO = 8;   // numbers per face with J: F_w, F_n, alpha, beta, gamma, delta, nu, eta
+constexpr int NCO_F = 2; // without
+
+// A slab: cell planes [c0, c1) along axis ax (z in 3D, y in 2D; y in 3D too
+// where z planes are too large for the workspace) in face workspace W, plane c
+// in ring slot c % ring (the plane below the slab stays for the slab's first
+// vertex plane).  Number m of face f (axis * 2^(d-1) + position) of in-plane
+// cell q lies at W[(f * NCO + m) * ws + slot * pc + q], its axis' upwind bits
+// (2 per position: water, NAPL from the lower vertex) at U[axis * ws + ...].
+// Cells are parity-split along x as vertices are.
+struct Slab {
+  double* W;
+  uint8_t* U;
+  int ws, pc, ring, c0, c1, ax;
+};
+
+// x / h given rh = 1 / h rounded to nearest: one Newton step on x * rh, the
+// correctly rounded quotient for every h when no step under- or overflows
+// (Markstein, IBM J. Res. Dev. 34 (1990); Brisebarre, Muller, Raina, IEEE
+// Trans. Comput. 53 (2004)); 3 FP64 instructions where the general division
+// has about 10.  Outside [2^-959, 2^957] it divides; zero needs no step.
+__device__ __forceinline__ double div_by(double x, double h, double rh) {
+  const uint32_t e = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
+  const double q = __dmul_rn(x, rh);
+  const double y = __fma_rn(__fma_rn(-q, h, x), rh, q);
+  if (e - 64u < 1917u) return y;
+  if ((((uint32_t)__double2hiint(x) << 1) | (uint32_t)__double2loint(x)) == 0u) return y;
+  return __ddiv_rn(x, h);
+}
+
+// a + w x, product and sum rounded separately; a power-of-two weight's product
+// is exact, so one fused operation rounds alike
+__device__ __forceinline__ double add_term(double a, double w, double x, bool pow2) {
+  return pow2 ? __fma_rn(w, x, a) : __dadd_rn(a, __dmul_rn(w, x));
+}
+
+// x >= 0 (-0 included) from the bits: comparisons of doubles issue on the FP64
+// pipe.  (A NaN flux makes F and J NaN whichever side it takes.)
+__device__ __forceinline__ bool not_below(double x) {
+  const int hi = __double2hiint(x);
+  return hi >= 0 || (((uint32_t)hi << 1) | (uint32_t)__double2loint(x)) == 0u;
+}
+
+template <int DIM, int K, bool WANT_J, bool DARCY>
+__device__ __forceinline__ void faces_of_axis(const Dims& d, const Phys& ph, const AsmIn& in, const Slab& sl, int t) {
+  constexpr int NC = 1 << DIM, NE = 1 << (DIM - 1), CO = WANT_J ? NCO : NCO_F;
+  constexpr int O1 = K == 0 ? 1 : 0, O2 = K == 2 ? 1 : 2;   // the other axes, in order
+  const int cx = d.nx - 1, cy = d.ny - 1, EC = (cx + 1) / 2;
+  const int pl = (int)((uint32_t)t / (uint32_t)sl.pc), q0 = t - pl * sl.pc;
+  const int line = (int)((uint32_t)q0 / (uint32_t)cx), pos = q0 - line * cx, plane = sl.c0 + pl;
+  const int ci = pos < EC ? 2 * pos : 2 * (pos - EC) + 1;
+  const int cj = DIM == 2 || sl.ax == 1 ? plane : line;
+  const int ck = DIM == 2 ? 0 : sl.ax == 1 ? line : plane;
   const int64_t cell = ci + (int64_t)cx * (cj + (int64_t)cy * ck);
   const double Kc = in.K[cell], pdc = in.pd[cell];
   const double* law = in.law ? law_row(in.kr_tab, in.law[cell]) : nullptr;
-  const double neg_inv_den = -1.0 / ph.den;
-  const bool darcy = (ph.scheme & SCHEME_DARCY_UPWIND) != 0;
-  double gtab[DIM][DIM];   // +-w / h_k by the number of 1/4 factors (see k_assemble)
-#pragma unroll
-  for (int kk = 0; kk < DIM; ++kk)
-#pragma unroll
-    for (int m = 0; m < DIM; ++m) {
-      double w = 1.0;
-#pragma unroll
-      for (int tt = 0; tt < DIM - 1; ++tt) w = w * (tt < m ? 0.25 : 0.75);
-      gtab[kk][m] = w / ph.h[kk];
-    }
-  int64_t vq[NC];
-  double se[NC], pnq[NC], pcq[NC], dpcq[NC], pwq[NC], Fl[NC][2];
+  const double h = ph.h[K], rh = ph.rh[K];
+  const double KA = __dmul_rn(Kc, ph.Af[K]);
+  int vq[NC];
+  double se[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
-    vq[q] = pidx(d, ci + (q & 1), cj + ((q >> 1) & 1), DIM == 3 ? ck + ((q >> 2) & 1) : 0);
+    vq[q] = (int)pidx(d, ci + (q & 1), cj + ((q >> 1) & 1), DIM == 3 ? ck + ((q >> 2) & 1) : 0);
     se[q] = in.Se[vq[q]];
-    pnq[q] = in.pn[vq[q]];
-    pcq[q] = in.pc[vq[q]];
-    dpcq[q] = in.dpc[vq[q]];
-    pwq[q] = darcy ? in.u[vq[q]].x : 0.0;
-    Fl[q][0] = 0.0;
-    Fl[q][1] = 0.0;
   }
+  double dn[NE], dc[NE], dw[NE];
 #pragma unroll
-  for (int kk = 0; kk < DIM; ++kk) {
-    int oth[2], no = 0;
+  for (int e = 0; e < NE; ++e) {
+    const int a = (e & 1) << O1 | (DIM == 3 ? (e >> 1) << O2 : 0), b = a | 1 << K;
+    dn[e] = __dsub_rn(in.pn[vq[b]], in.pn[vq[a]]);
+    dc[e] = __dsub_rn(in.pc[vq[b]], in.pc[vq[a]]);
+    if (DARCY) dw[e] = __dsub_rn(in.u[vq[b]].x, in.u[vq[a]].x);
+  }
+  const double gw = ph.gw[K], gn = ph.gn[K];
+  const double kah = div_by(KA, h, rh) * (DIM == 3 ? 0.0625 : 0.25);
+  const double gsc = ph.rho_w * ph.nid * (DIM == 3 ? 0.03125 : 0.125);
+  const int wi = (int)((uint32_t)plane % (uint32_t)sl.ring) * sl.pc + q0;
+  uint32_t up = 0;
 #pragma unroll
-    for (int m = 0; m < DIM; ++m)
-      if (m != kk) oth[no++] = m;
-    double Af = 1.0;
+  for (int e = 0; e < NE; ++e) {
+    const int a = (e & 1) << O1 | (DIM == 3 ? (e >> 1) << O2 : 0), b = a | 1 << K;
+    double gpn = 0.0, gpc = 0.0, gpw = 0.0, SeM = 0.0;
 #pragma unroll
-    for (int tt = 0; tt < DIM - 1; ++tt) Af = __dmul_rn(Af, __dmul_rn(ph.h[oth[tt]], 0.5));
-    const double KA = __dmul_rn(Kc, Af);
+    for (int e2 = 0; e2 < NE; ++e2) {
+      double w = 1.0;
 #pragma unroll
-    for (int e = 0; e < NE; ++e) {
-      int o[2] = {0, 0};
+      for (int m = 0; m < DIM - 1; ++m) w = w * ((((e ^ e2) >> m) & 1) ? 0.25 : 0.75);
+      const bool pow2 = (e ^ e2) == NE - 1;
+      gpn = e2 ? add_term(gpn, w, dn[e2], pow2) : __dmul_rn(w, dn[0]);
+      gpc = e2 ? add_term(gpc, w, dc[e2], pow2) : __dmul_rn(w, dc[0]);
+      if (DARCY) gpw = e2 ? add_term(gpw, w, dw[e2], pow2) : __dmul_rn(w, dw[0]);
+    }
+    gpn = div_by(gpn, h, rh);
+    gpc = div_by(gpc, h, rh);
+    if (DARCY) gpw = div_by(gpw, h, rh);
 #pragma unroll
-      for (int tt = 0; tt < DIM - 1; ++tt) o[tt] = (e >> tt) & 1;
-      int a = 0;
-#pragma unroll
-      for (int tt = 0; tt < DIM - 1; ++tt) a |= o[tt] << oth[tt];
-      const int b = a | (1 << kk);
-      double gpn = 0.0, gpc = 0.0, gpw = 0.0;
-#pragma unroll
-      for (int e2 = 0; e2 < NE; ++e2) {
-        int o2[2] = {e2 & 1, (e2 >> 1) & 1};
-        double w = 1.0;
-        int a2 = 0;
-#pragma unroll
-        for (int tt = 0; tt < DIM - 1; ++tt) {
-          w = w * (o2[tt] == o[tt] ? 0.75 : 0.25);
-          a2 |= o2[tt] << oth[tt];
-        }
-        const int b2 = a2 | (1 << kk);
-        gpn = __dadd_rn(gpn, __dmul_rn(w, __dsub_rn(pnq[b2], pnq[a2])));
-        gpc = __dadd_rn(gpc, __dmul_rn(w, __dsub_rn(pcq[b2], pcq[a2])));
-        if (darcy) gpw = __dadd_rn(gpw, __dmul_rn(w, __dsub_rn(pwq[b2], pwq[a2])));
-      }
-      gpn = __ddiv_rn(gpn, ph.h[kk]);
-      gpc = __ddiv_rn(gpc, ph.h[kk]);
-      gpw = __ddiv_rn(gpw, ph.h[kk]);
-      double wM[NC], SeM = 0.0;
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        double w = 0.5;
-#pragma unroll
-        for (int tt = 0; tt < DIM - 1; ++tt) w = w * ((((q >> oth[tt]) & 1) == o[tt]) ? 0.75 : 0.25);
-        wM[q] = w;
-        SeM = __dadd_rn(SeM, __dmul_rn(w, se[q]));
-      }
-      const double Tw = __dmul_rn(-KA, __dsub_rn(gpn, __dmul_rn(ph.rho_w, ph.g[kk])));
-      const double Tn = __dmul_rn(-KA, __dsub_rn(gpn, __dmul_rn(ph.rho_n, ph.g[kk])));
-      const double Tc = __dmul_rn(-KA, gpc);
-      const double Tpw = __dmul_rn(-KA, __dsub_rn(gpw, __dmul_rn(ph.rho_w, ph.g[kk])));
-      const bool wa = darcy ? Tpw >= 0.0 : Tw >= 0.0, na = Tn >= 0.0;
-      const int qw = wa ? a : b, qn = na ? a : b;
-      const int64_t vw = wa ? vq[a] : vq[b], vn = na ? vq[a] : vq[b];   // selects, not indexing
-      double lw_up, dlw_up;   // k_rw / mu_w of the upwind vertex (with this element's law) and its S_n-derivative
-      if (!law) {
-        lw_up = in.krw[vw];
-        dlw_up = in.dkrw[vw];
-      } else {
-        double k, dk;
-        krw_law(ph.lam, law, wa ? se[a] : se[b], k, dk);
-        lw_up = k / ph.mu_w;
-        dlw_up = (-dk / ph.den) / ph.mu_w;
-      }
-      double kM, dkM;
+    for (int q = 0; q < NC; ++q) {
+      double w = 0.5;
+      w = w * ((((q >> O1) & 1) == (e & 1)) ? 0.75 : 0.25);
+      if (DIM == 3) w = w * ((((q >> O2) & 1) == (e >> 1)) ? 0.75 : 0.25);
+      SeM = q ? add_term(SeM, w, se[q], w == (DIM == 3 ? 0.03125 : 0.125)) : __dmul_rn(w, se[0]);
+    }
+    const double Tw = __dmul_rn(-KA, __dsub_rn(gpn, gw));
+    const double Tn = __dmul_rn(-KA, __dsub_rn(gpn, gn));
+    const double Tc = __dmul_rn(-KA, gpc);
+    const double Tpw = DARCY ? __dmul_rn(-KA, __dsub_rn(gpw, gw)) : 0.0;
+    const bool wa = not_below(DARCY ? Tpw : Tw), na = not_below(Tn);
+    const int vw = wa ? vq[a] : vq[b], vn = na ? vq[a] : vq[b];   // selects, not indexing
+    double lw_up, dlw_up = 0.0;   // k_rw / mu_w of the upwind vertex (with this element's law), its S_n-derivative
+    if (!law) {
+      lw_up = in.krw[vw];
+      if (WANT_J) dlw_up = in.dkrw[vw];
+    } else {
+      double k, dk;
+      krw_law(ph.lam, law, wa ? se[a] : se[b], k, dk);
+      lw_up = k / ph.mu_w;
+      dlw_up = (-dk / ph.den) / ph.mu_w;
+    }
+    double kM, dkM;
+    if (!law && ph.lam == 2.0 && (uint32_t)__double2hiint(SeM) - 1u < 0x3fefffffu) {   // inside (0, 1): no clamps
+      const double s2 = SeM * SeM;
+      kM = s2 * s2;
+      dkM = 4.0 * s2 * SeM;
+    } else {
       krw_law(ph.lam, law, SeM, kM, dkM);
-      const double lwM = kM / ph.mu_w;
+    }
+    const double lwM = div_by(kM, ph.mu_w, ph.rmu_w);
+    // lambda_n of S hat at the upwind vertex: the vertex's own where S hat = S_e
+    double ln_up, dln_up = 0.0;
+    const double pdm = in.pdmin[vn];
+    if (!law && __double_as_longlong(pdc) == __double_as_longlong(pdm)) {
+      ln_up = in.krn[vn];
+      if (WANT_J) dln_up = in.dkrn[vn];
+    } else {
       double sh, dsh, kn, dkn;
-      shat_of(ph.lam, na ? se[a] : se[b], pdc, in.pdmin[vn], sh, dsh);
+      shat_of(ph.lam, na ? se[a] : se[b], pdc, pdm, sh, dsh);
       krn_law(ph.lam, law, sh, kn, dkn);
-      const double ln_up = kn / ph.mu_n;
-      const double Fw = darcy ? ph.rho_w * (lw_up * Tpw) : ph.rho_w * (lw_up * Tw - lwM * Tc);
-      const double Fn = ph.rho_n * (ln_up * Tn);
-      Fl[a][0] -= Fw;
-      Fl[a][1] -= Fn;
-      Fl[b][0] += Fw;
-      Fl[b][1] += Fn;
-      if (WANT_J) {
-        const double dlwM_dSeM = dkM / ph.mu_w;
-        const double dln_up = dkn * dsh * neg_inv_den / ph.mu_n;
-#pragma unroll
-        for (int q = 0; q < NC; ++q) {
-          int nq = 0;
-#pragma unroll
-          for (int tt = 0; tt < DIM - 1; ++tt) nq += (((q >> oth[tt]) & 1) == o[tt]) ? 0 : 1;
-          const double gq = ((q >> kk) & 1) ? gtab[kk][nq] : -gtab[kk][nq];
-          const double dT = -KA * gq;
-          const double dlwM = wM[q] * dlwM_dSeM * neg_inv_den;
-          const double d0 = ph.rho_w * lw_up * dT;
-          const double d1 = darcy ? ph.rho_w * (q == qw ? dlw_up * Tpw : 0.0)
-                                  : ph.rho_w * ((q == qw ? dlw_up * Tw : 0.0) + lw_up * dT * dpcq[q] - dlwM * Tc -
-                                                lwM * dT * dpcq[q]);
-          const double d2 = ph.rho_n * ln_up * dT;
-          const double d3 = ph.rho_n * ((q == qn ? dln_up * Tn : 0.0) + ln_up * dT * dpcq[q]);
-          const int bia = blk_of(DIM, (q & 1) - (a & 1), ((q >> 1) & 1) - ((a >> 1) & 1),
-                                 DIM == 3 ? ((q >> 2) & 1) - ((a >> 2) & 1) : 0);
-          const int bib = blk_of(DIM, (q & 1) - (b & 1), ((q >> 1) & 1) - ((b >> 1) & 1),
-                                 DIM == 3 ? ((q >> 2) & 1) - ((b >> 2) & 1) : 0);
-          double2* ja = reinterpret_cast<double2*>(J + ((int64_t)bia * d.nv + vq[a]) * 4);
-          double2* jb = reinterpret_cast<double2*>(J + ((int64_t)bib * d.nv + vq[b]) * 4);
-          double2 a0 = ja[0], a1 = ja[1], b0 = jb[0], b1 = jb[1];
-          a0.x -= d0; a0.y -= d1; a1.x -= d2; a1.y -= d3;
-          b0.x += d0; b0.y += d1; b1.x += d2; b1.y += d3;
-          ja[0] = a0; ja[1] = a1;
-          jb[0] = b0; jb[1] = b1;
-        }
-      }
+      ln_up = kn / ph.mu_n;
+      dln_up = dkn * dsh * ph.nid / ph.mu_n;
+    }
+    double* W = sl.W + (size_t)((K * NE + e) * CO) * sl.ws + wi;
+    W[0] = DARCY ? ph.rho_w * (lw_up * Tpw) : ph.rho_w * (lw_up * Tw - lwM * Tc);
+    W[(size_t)sl.ws] = ph.rho_n * (ln_up * Tn);
+    if (WANT_J) {
+      up |= (wa ? 1u : 0u) << (2 * e) | (na ? 2u : 0u) << (2 * e);
+      W[2 * (size_t)sl.ws] = (ph.rho_w * lw_up) * kah;
+      W[3 * (size_t)sl.ws] = DARCY ? 0.0 : (ph.rho_w * (lw_up - lwM)) * kah;
+      W[4 * (size_t)sl.ws] = DARCY ? 0.0 : (div_by(dkM, ph.mu_w, ph.rmu_w) * gsc) * Tc;
+      W[5 * (size_t)sl.ws] = (ph.rho_w * dlw_up) * (DARCY ? Tpw : Tw);
+      W[6 * (size_t)sl.ws] = (ph.rho_n * ln_up) * kah;
+      W[7 * (size_t)sl.ws] = (ph.rho_n * dln_up) * Tn;
     }
   }
-  // add this element's residual contributions to its corners' rows
+  if (WANT_J) sl.U[(size_t)K * sl.ws + wi] = (uint8_t)up;
+}
+
+template <int DIM, bool WANT_J, bool DARCY>
+__global__ void __launch_bounds__(128) k_asm_faces(const __grid_constant__ Dims d, const __grid_constant__ Phys ph,
+                                                   const __grid_constant__ AsmIn in, const __grid_constant__ Slab sl) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (sl.c1 - sl.c0) * sl.pc) return;
+  if (blockIdx.y == 0) faces_of_axis<DIM, 0, WANT_J, DARCY>(d, ph, in, sl, t);
+  else if (blockIdx.y == 1) faces_of_axis<DIM, 1, WANT_J, DARCY>(d, ph, in, sl, t);
+  else if (DIM == 3) faces_of_axis<DIM, DIM - 1, WANT_J, DARCY>(d, ph, in, sl, t);
+}
+
+// The faces around one vertex, edge by edge: edge (K, S) runs from the vertex
+// along axis K in direction S, and the 2^(d-1) elements around it each hold one
+// of its faces.  ce[c] is the workspace index of the element whose corner c
+// (bits x, y, z) the vertex is, or -1 outside the grid.
+
+// block of the stencil at offset 0 (the edge's own end) or S (its far end)
+// along K, and d1, d2 along the other axes in order
+template <int DIM, int K, int S>
+__device__ __forceinline__ int edge_blk(int far, int d1, int d2) {
+  const int dk = far ? S : 0;
+  const int dx = K == 0 ? dk : d1;
+  const int dy = K == 0 ? d1 : (K == 1 ? dk : d2);
+  const int dz = DIM == 3 ? (K == 2 ? dk : d2) : 0;
+  return DIM == 3 ? (dx + 1) + 3 * (dy + 1) + 9 * (dz + 1) : (dx + 1) + 3 * (dy + 1);
+}
+
+// the element of edge (K, S) on sides (s1, s2: 0 = below, 1 = above) of the
+// other axes: its bits as a corner index, and the edge's face position in it
+template <int DIM, int K, int S>
+__device__ __forceinline__ int edge_elem(int s1, int s2) {
+  const int bk = S > 0 ? 0 : 1, b1 = s1 ? 0 : 1, b2 = s2 ? 0 : 1;
+  const int x = K == 0 ? bk : b1, y = K == 0 ? b1 : (K == 1 ? bk : b2), z = DIM == 3 ? (K == 2 ? bk : b2) : 0;
+  return x | y << 1 | z << 2;
+}
+
+template <int DIM, int K, int S, int CO>
+__device__ __forceinline__ void edge_load(const double* __restrict__ W, int ws, int m, const int (&ce)[1 << DIM],
+                                          double (&v)[1 << (DIM - 1)]) {
+  constexpr int NE = 1 << (DIM - 1);
 #pragma unroll
-  for (int r = 0; r < NC; ++r) {
-    double2 f = F[vq[r]];
-    f.x += Fl[r][0];
-    f.y += Fl[r][1];
-    F[vq[r]] = f;
+  for (int f = 0; f < NE; ++f) {          // f: sides (s1, s2)
+    const int s1 = f & 1, s2 = (f >> 1) & 1;
+    const int c = ce[edge_elem<DIM, K, S>(s1, s2)];
+    const int e = (s1 ? 0 : 1) | (DIM == 3 ? (s2 ? 0 : 2) : 0);   // face position in that element
+    v[f] = c >= 0 ? W[(size_t)((K * NE + e) * CO + m) * ws + c] : 0.0;
   }
 }
 
-// After all colours: sources, Dirichlet p_w rows (0 = p_dir - p_w: J row -e,
-// M row 0) and the mass diagonal, per vertex.
+// adds (or subtracts) the tensor transform of the edge's faces v to the blocks
+// at its own end and to those at its far end; its factors 3 and 9 ride on the
+// accumulation's multiply-add
+// (INIT: of an accumulator that holds nothing yet, the blocks this edge is the
+// first to reach, the edges in row_diff's order, are set instead)
+template <int DIM, int K, int S, int NB, bool INIT = false>
+__device__ __forceinline__ void edge_add(const double (&v)[1 << (DIM - 1)], bool own_minus, bool far_minus,
+                                         double (&acc)[NB]) {
+  constexpr bool SET_OWN = INIT && K == 0 && S < 0, SET_FAR = INIT && K == 0;
+  double E[DIM == 3 ? 9 : 3];             // without the factors
+  if (DIM == 3) {
+#pragma unroll
+    for (int s2 = 0; s2 < 2; ++s2) {      // rows d2 = -1 and +1
+      E[6 * s2 + 0] = v[2 * s2];
+      E[6 * s2 + 1] = v[2 * s2] + v[2 * s2 + 1];
+      E[6 * s2 + 2] = v[2 * s2 + 1];
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) E[3 + t] = E[t] + E[6 + t];
+  } else {
+    E[0] = v[0]; E[1] = v[0] + v[1]; E[2] = v[1];
+  }
+#pragma unroll
+  for (int t = 0; t < (DIM == 3 ? 9 : 3); ++t) {
+    const int d1 = t % 3 - 1, d2 = DIM == 3 ? t / 3 - 1 : 0;
+    const double f = (d1 == 0 ? 3.0 : 1.0) * (DIM == 3 && d2 == 0 ? 3.0 : 1.0);
+    const int b0 = edge_blk<DIM, K, S>(0, d1, d2), b1 = edge_blk<DIM, K, S>(1, d1, d2);
+    acc[b0] = SET_OWN ? (own_minus ? -f : f) * E[t] : __fma_rn(own_minus ? -f : f, E[t], acc[b0]);
+    acc[b1] = SET_FAR ? (far_minus ? -f : f) * E[t] : __fma_rn(far_minus ? -f : f, E[t], acc[b1]);
+  }
+}
+
+// every edge of the vertex: own end -, far end + (alpha, beta, nu); sets acc
+template <int DIM, int NB, int CO>
+__device__ __forceinline__ void row_diff(const double* __restrict__ W, int ws, int m, const int (&ce)[1 << DIM],
+                                         double (&acc)[NB]) {
+  double v[1 << (DIM - 1)];
+  edge_load<DIM, 0, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 0, -1, NB, true>(v, true, false, acc);
+  edge_load<DIM, 0, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 0, 1, NB, true>(v, true, false, acc);
+  edge_load<DIM, 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 1, -1, NB, true>(v, true, false, acc);
+  edge_load<DIM, 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 1, 1, NB, true>(v, true, false, acc);
+  if (DIM == 3) {
+    edge_load<DIM, DIM - 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, DIM - 1, -1, NB, true>(v, true, false, acc);
+    edge_load<DIM, DIM - 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, DIM - 1, 1, NB, true>(v, true, false, acc);
+  }
+}
+
+// both ends + for the edges that leave upwards, - for those that come from below (gamma)
+template <int DIM, int NB, int CO>
+__device__ __forceinline__ void row_mean(const double* __restrict__ W, int ws, int m, const int (&ce)[1 << DIM],
+                                         double (&acc)[NB]) {
+  double v[1 << (DIM - 1)];
+  edge_load<DIM, 0, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 0, -1, NB>(v, true, true, acc);
+  edge_load<DIM, 0, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 0, 1, NB>(v, false, false, acc);
+  edge_load<DIM, 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 1, -1, NB>(v, true, true, acc);
+  edge_load<DIM, 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 1, 1, NB>(v, false, false, acc);
+  if (DIM == 3) {
+    edge_load<DIM, DIM - 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, DIM - 1, -1, NB>(v, true, true, acc);
+    edge_load<DIM, DIM - 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, DIM - 1, 1, NB>(v, false, false, acc);
+  }
+}
+
+// one edge's upwind terms (delta, eta; m, upwind bit BIT) and flux (mf):
+// the vertex is the edge's lower end for S > 0 (row: -) and its upper one for
+// S < 0 (row: +); a term goes to the block of the face's upwind vertex
+template <int DIM, int K, int S, int NB, int CO, bool WANT_J>
+__device__ __forceinline__ void edge_up(const Slab& sl, const int (&ce)[1 << DIM], int m, int bit, int mf,
+                                        double (&acc)[NB], double& F) {
+  constexpr int NE = 1 << (DIM - 1);
+  double fv[NE];
+  edge_load<DIM, K, S, CO>(sl.W, sl.ws, mf, ce, fv);
+#pragma unroll
+  for (int f = 0; f < NE; ++f) F = S > 0 ? F - fv[f] : F + fv[f];
+  if (WANT_J) {
+    const int b0 = edge_blk<DIM, K, S>(0, 0, 0), b1 = edge_blk<DIM, K, S>(1, 0, 0);
+    double v[NE];
+    edge_load<DIM, K, S, CO>(sl.W, sl.ws, m, ce, v);
+    double own = 0.0, far = 0.0;
+#pragma unroll
+    for (int f = 0; f < NE; ++f) {
+      const int s1 = f & 1, s2 = (f >> 1) & 1;
+      const int c = ce[edge_elem<DIM, K, S>(s1, s2)];
+      const int e = (s1 ? 0 : 1) | (DIM == 3 ? (s2 ? 0 : 2) : 0);
+      const bool lower = c >= 0 && ((sl.U[(size_t)K * sl.ws + c] >> (2 * e + bit)) & 1);
+      const bool mine = lower == (S > 0);
+      own += mine ? v[f] : 0.0;
+      far += mine ? 0.0 : v[f];
+    }
+    acc[b0] = S > 0 ? acc[b0] - own : acc[b0] + own;
+    acc[b1] = S > 0 ? acc[b1] - far : acc[b1] + far;
+  }
+}
+
+template <int DIM, int NB, int CO, bool WANT_J>
+__device__ __forceinline__ void row_up(const Slab& sl, const int (&ce)[1 << DIM], int m, int bit, int mf,
+                                       double (&acc)[NB], double& F) {
+  edge_up<DIM, 0, -1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
+  edge_up<DIM, 0, 1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
+  edge_up<DIM, 1, -1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
+  edge_up<DIM, 1, 1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
+  if (DIM == 3) {
+    edge_up<DIM, DIM - 1, -1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
+    edge_up<DIM, DIM - 1, 1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
+  }
+}
+
+// Vertex planes [v0, v1): 32 vertices per block, one warp their water rows and
+// one their NAPL rows (so that the two halves of each 32-byte block are written
+// at about the same time; the water rows' accumulators take 182 registers, and
+// blocks of two warps let an SM hold 10 warps instead of 8).  Sources, Dirichlet p_w rows (0 =
+// p_dir - p_w: J row -e, M row 0) and the mass diagonal are applied here.
 template <int DIM, bool WANT_J>
-__global__ void k_assemble_finish(Dims d, Phys ph, AsmIn in, double2* __restrict__ F, double* __restrict__ J,
-                                  double2* __restrict__ mdiag) {
-  constexpr int NC = 1 << DIM, NB = DIM == 3 ? 27 : 9;
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= d.nv) return;
-  double2 f = F[p];
-  if (in.q_in) {
-    const double2 q = in.q_in[p];
-    f.x += q.x;
-    f.y += q.y;
+__global__ void __launch_bounds__(64) k_asm_rows(const __grid_constant__ Dims d, const __grid_constant__ Phys ph,
+                                                  const __grid_constant__ AsmIn in, const __grid_constant__ Slab sl, int v0, int v1,
+                                                  double* __restrict__ F, double* __restrict__ J,
+                                                  double2* __restrict__ mdiag) {
+  constexpr int NC = 1 << DIM, NB = DIM == 3 ? 27 : 9, CO = WANT_J ? NCO : NCO_F;
+  const int napl = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nline = DIM == 2 ? 1 : sl.ax == 1 ? d.nz : d.ny;    // x-lines per vertex plane
+  const int64_t t = (int64_t)blockIdx.x * 32 + lane;
+  if (t >= (int64_t)(v1 - v0) * nline * d.nx) return;
+  const uint32_t l0 = (uint32_t)t / (uint32_t)d.nx, pl = l0 / (uint32_t)nline;   // nv < 2^31
+  const int vpos = (int)((uint32_t)t - l0 * (uint32_t)d.nx), line = (int)(l0 - pl * (uint32_t)nline), vpl = v0 + (int)pl;
+  const int i = vpos < d.E ? 2 * vpos : 2 * (vpos - d.E) + 1;
+  const int j = DIM == 2 || sl.ax == 1 ? vpl : line, k = DIM == 2 ? 0 : sl.ax == 1 ? line : vpl;
+  const int64_t p = ((int64_t)j + (int64_t)d.ny * k) * d.nx + vpos;
+  const int cx = d.nx - 1, cy = d.ny - 1, cz = DIM == 3 ? d.nz - 1 : 1, EC = (cx + 1) / 2;
+  int ce[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = DIM == 3 ? k - ((c >> 2) & 1) : 0;
+    const bool ok = ci >= 0 && ci < cx && cj >= 0 && cj < cy && ck >= 0 && ck < cz;
+    const int pos = (ci & 1) ? EC + (ci >> 1) : (ci >> 1);
+    const int plane = DIM == 2 || sl.ax == 1 ? cj : ck, cl = DIM == 2 ? 0 : sl.ax == 1 ? ck : cj;
+    ce[c] = ok ? (int)((uint32_t)plane % (uint32_t)sl.ring) * sl.pc + cl * cx + pos : -1;
   }
   const bool dirv = in.dir[p] != 0;
-  if (dirv) f.x = in.pw_dir[p] - in.u[p].x;
-  F[p] = f;
-  if (!WANT_J) return;
-  double pv = in.phiv[p];
-  if (ph.scheme & SCHEME_SHAT_STORAGE) {
-    int i, j, k;
-    pcoords(d, p, i, j, k);
-    const int cx = d.nx - 1, cy = d.ny - 1, cz = DIM == 3 ? d.nz - 1 : 1;
-    const double frac = DIM == 3 ? 0.125 : 0.25, se = in.Se[p], pdm = in.pdmin[p];
-    pv = 0.0;
-    for (int c = 0; c < NC; ++c) {
-      const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = DIM == 3 ? k - ((c >> 2) & 1) : 0;
-      if (ci < 0 || ci >= cx || cj < 0 || cj >= cy || ck < 0 || ck >= cz) continue;
-      const int64_t cell = ci + (int64_t)cx * (cj + (int64_t)cy * ck);
-      double sh, dsh;
-      shat_of(ph.lam, se, in.pd[cell], pdm, sh, dsh);
-      pv += in.phi[cell] * in.vol * frac * dsh;
+  double a1[NB];
+  double f = 0.0;
+  if (!napl) {
+    if (WANT_J) {
+      // (w, S_n): the beta sums times dpc, then gamma and delta
+      row_diff<DIM, NB, CO>(sl.W, sl.ws, 3, ce, a1);
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const int dx = b % 3 - 1, dy = (b / 3) % 3 - 1, dz = DIM == 3 ? b / 9 - 1 : 0;
+        const int ii = i + dx, jj = j + dy, kk = k + dz;
+        const bool ok = ii >= 0 && ii < d.nx && jj >= 0 && jj < d.ny && (DIM == 2 || (kk >= 0 && kk < d.nz));
+        a1[b] = ok ? a1[b] * in.dpc[pidx(d, ii, jj, kk)] : 0.0;
+      }
+      row_mean<DIM, NB, CO>(sl.W, sl.ws, 4, ce, a1);
     }
-  }
-  mdiag[p] = make_double2(dirv ? 0.0 : -ph.rho_w * pv, ph.rho_n * pv);
-  if (dirv) {
-    const int centre = DIM == 3 ? 13 : 4;
-    for (int bi = 0; bi < NB; ++bi) {
-      double2* dst = reinterpret_cast<double2*>(J + ((int64_t)bi * d.nv + p) * 4);
-      dst[0] = make_double2(bi == centre ? -1.0 : 0.0, 0.0);
+    row_up<DIM, NB, CO, WANT_J>(sl, ce, 5, 0, 0, a1, f);
+    if (WANT_J) {
+      double a0[NB];
+      row_diff<DIM, NB, CO>(sl.W, sl.ws, 2, ce, a0);
+      constexpr int C = DIM == 3 ? 13 : 4;
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const double2 e = dirv ? make_double2(b == C ? -1.0 : 0.0, 0.0) : make_double2(a0[b], a1[b]);
+        *reinterpret_cast<double2*>(J + ((int64_t)b * d.nv + p) * 4) = e;
+      }
     }
+    if (in.q_in) f += in.q_in[p].x;
+    if (dirv) f = in.pw_dir[p] - in.u[p].x;
+    F[2 * p] = f;
+    return;
   }
+  if (WANT_J) {
+    row_diff<DIM, NB, CO>(sl.W, sl.ws, 6, ce, a1);
+    double a3[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const int dx = b % 3 - 1, dy = (b / 3) % 3 - 1, dz = DIM == 3 ? b / 9 - 1 : 0;
+      const int ii = i + dx, jj = j + dy, kk = k + dz;
+      const bool ok = ii >= 0 && ii < d.nx && jj >= 0 && jj < d.ny && (DIM == 2 || (kk >= 0 && kk < d.nz));
+      a3[b] = ok ? a1[b] * in.dpc[pidx(d, ii, jj, kk)] : 0.0;
+    }
+    row_up<DIM, NB, CO, WANT_J>(sl, ce, 7, 1, 1, a3, f);
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+      *reinterpret_cast<double2*>(J + ((int64_t)b * d.nv + p) * 4 + 2) = make_double2(a1[b], a3[b]);
+    double pvol = in.phiv[p];
+    if (ph.scheme & SCHEME_SHAT_STORAGE) {
+      const double frac = DIM == 3 ? 0.125 : 0.25, se = in.Se[p], pdm = in.pdmin[p];
+      pvol = 0.0;
+      for (int c = 0; c < NC; ++c) {
+        const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = DIM == 3 ? k - ((c >> 2) & 1) : 0;
+        if (ci < 0 || ci >= cx || cj < 0 || cj >= cy || ck < 0 || ck >= cz) continue;
+        const int64_t cell = ci + (int64_t)cx * (cj + (int64_t)cy * ck);
+        double sh, dsh;
+        shat_of(ph.lam, se, in.pd[cell], pdm, sh, dsh);
+        pvol += in.phi[cell] * in.vol * frac * dsh;
+      }
+    }
+    mdiag[p] = make_double2(dirv ? 0.0 : -ph.rho_w * pvol, ph.rho_n * pvol);
+  } else {
+    row_up<DIM, NB, CO, WANT_J>(sl, ce, 7, 1, 1, a1, f);
+  }
+  if (in.q_in) f += in.q_in[p].y;
+  F[2 * p + 1] = f;
 }
 
 // ---------------------------------------------------------------- storage (S hat variant)
@@ -697,33 +923,60 @@ void launch_perm_scalar_to_p(const Dims& d, const double* nat, double* out, void
   RF_LAUNCH(k_perm_scalar_to_p, (int)((d.nv + 255) / 256), 256, 0, s, d, nat, out);
 }
 
-template <int DIM, bool WANT_J>
-static void cells_t(const Dims& d, const Phys& ph, const AsmIn& in, const AsmArrays& a, void* s) {
-  const int BS = 128;
-  const int NC = 1 << DIM;
-  const size_t smem = 0;
-  if (WANT_J) cudaMemsetAsync(a.J, 0, sizeof(double) * 4 * (size_t)d.nb * d.nv, (cudaStream_t)s);
-  cudaMemsetAsync(a.F, 0, sizeof(double) * 2 * (size_t)d.nv, (cudaStream_t)s);
-  const int cx = d.nx - 1, cy = d.ny - 1, cz = DIM == 3 ? d.nz - 1 : 1;
-  for (int c = 0; c < NC; ++c) {
-    const int px = c & 1, py = (c >> 1) & 1, pz = (c >> 2) & 1;
-    const int64_t ncol = (int64_t)((cx - px + 1) / 2) * ((cy - py + 1) / 2) * (DIM == 3 ? (cz - pz + 1) / 2 : 1);
-    if (ncol <= 0) continue;
-    RF_LAUNCH((k_assemble_cells<DIM, WANT_J>), (int)((ncol + BS - 1) / BS), BS, smem, s, d, ph, in, c, ncol,
-              (double2*)a.F, a.J);
-  }
-  RF_LAUNCH((k_assemble_finish<DIM, WANT_J>), (int)((d.nv + 255) / 256), 256, 0, s, d, ph, in, (double2*)a.F, a.J,
-            (double2*)a.mdiag);
+// Face workspace of one assembly: at most ASM_WS_BYTES (with J; F alone a
+// quarter of that, as its faces need a quarter of the numbers), at least two
+// cell planes.  At 257^3 a slab then holds 9 planes (50 MB each), 15 waves of
+// k_asm_faces.  Slabs go along z, or along y where two z planes exceed the
+// limit and y planes are smaller (wide, shallow boxes).
+constexpr size_t ASM_WS_BYTES = (size_t)512 << 20;
+
+struct SlabShape { int ax, planes, ring; int64_t plane; };
+
+static SlabShape slab_shape(const Dims& d, bool want_j) {
+  const size_t cell = (size_t)(d.dim << (d.dim - 1)) * (want_j ? NCO : NCO_F) * sizeof(double);
+  const int64_t fit = (int64_t)((want_j ? ASM_WS_BYTES : ASM_WS_BYTES / 4) / cell);   // cells
+  const int64_t zp = (int64_t)(d.nx - 1) * (d.ny - 1), yp = (int64_t)(d.nx - 1) * (d.dim == 3 ? d.nz - 1 : 1);
+  SlabShape r;
+  r.ax = d.dim == 3 && (2 * zp <= fit || zp <= yp) ? 2 : 1;
+  r.plane = r.ax == 2 ? zp : yp;
+  r.planes = (r.ax == 2 ? d.nz : d.ny) - 1;
+  const int64_t ring = fit / r.plane < 2 ? 2 : fit / r.plane;
+  r.ring = (int)(ring < r.planes ? ring : r.planes);
+  return r;
 }
 
-static void launch_assemble_cells(const Dims& d, const Phys& ph, const AsmIn& in, const AsmArrays& a, bool want_j,
-                                  void* s) {
-  if (d.dim == 3) {
-    if (want_j) cells_t<3, true>(d, ph, in, a, s);
-    else cells_t<3, false>(d, ph, in, a, s);
-  } else {
-    if (want_j) cells_t<2, true>(d, ph, in, a, s);
-    else cells_t<2, false>(d, ph, in, a, s);
+size_t assemble_workspace(const Dims& d, bool want_j) {
+  const SlabShape r = slab_shape(d, want_j);
+  const size_t cell = (size_t)(d.dim << (d.dim - 1)) * (want_j ? NCO : NCO_F) * sizeof(double);
+  return (size_t)(r.ring * r.plane) * (cell + (want_j ? d.dim : 0));
+}
+
+template <int DIM, bool WANT_J>
+static void slabs_t(const Dims& d, const Phys& ph, const AsmIn& in, const AsmArrays& a, void* s) {
+  const SlabShape sh = slab_shape(d, WANT_J);
+  const int planes = sh.planes;
+  Slab sl;
+  sl.ax = sh.ax;
+  sl.ring = sh.ring;
+  sl.pc = (int)sh.plane;
+  sl.ws = (int)(sh.plane * sh.ring);
+  sl.W = a.faces;
+  sl.U = reinterpret_cast<uint8_t*>(a.faces + (size_t)sl.ws * (DIM << (DIM - 1)) * (WANT_J ? NCO : NCO_F));
+  // the first slab fills the ring; a later one leaves the plane below it in place
+  for (int c0 = 0, v0 = 0; c0 < planes;) {
+    const int c1 = c0 == 0 ? sl.ring : (c0 + sl.ring - 1 < planes ? c0 + sl.ring - 1 : planes);
+    sl.c0 = c0;
+    sl.c1 = c1;
+    const int64_t nc = (int64_t)(c1 - c0) * sh.plane;
+    const dim3 g((unsigned)((nc + 127) / 128), DIM);
+    if (ph.scheme & SCHEME_DARCY_UPWIND) RF_LAUNCH((k_asm_faces<DIM, WANT_J, true>), g, 128, 0, s, d, ph, in, sl);
+    else RF_LAUNCH((k_asm_faces<DIM, WANT_J, false>), g, 128, 0, s, d, ph, in, sl);
+    const int v1 = c1 == planes ? planes + 1 : c1;
+    const int64_t nvert = (int64_t)(v1 - v0) * d.nx * (DIM == 2 ? 1 : sh.ax == 1 ? d.nz : d.ny);
+    RF_LAUNCH((k_asm_rows<DIM, WANT_J>), (unsigned)((nvert + 31) / 32), 64, 0, s, d, ph, in, sl, v0, v1, a.F, a.J,
+              (double2*)a.mdiag);
+    c0 = c1;
+    v0 = v1;
   }
 }
 
@@ -733,20 +986,35 @@ cudaError_t launch_assemble(const Dims& d, const PhysParams& pp, const AsmArrays
   ph.S_wr = pp.S_wr; ph.S_nr = pp.S_nr; ph.lam = pp.lambda;
   ph.den = 1.0 - pp.S_wr - pp.S_nr;
   ph.scheme = pp.scheme;
-  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; }
+  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = 1.0 / pp.h[t]; }
+  ph.rmu_w = 1.0 / pp.mu_w;
+  ph.nid = -1.0 / ph.den;
+  for (int t = 0; t < 3; ++t) {
+    ph.Af[t] = 1.0;
+    for (int m = 0; m < d.dim; ++m)
+      if (m != t) ph.Af[t] *= pp.h[m] * 0.5;
+    ph.gw[t] = pp.rho_w * pp.g[t];
+    ph.gn[t] = pp.rho_n * pp.g[t];
+  }
   const int nblk = (int)((d.nv + 255) / 256);
   RF_LAUNCH(k_vertex_state, nblk, 256, 0, s, d, ph, (const double2*)a.u, a.pdmin, a.Se, a.pn, a.pc, a.dpc,
-            a.krw, a.dkrw);
+            a.krw, a.dkrw, a.krn, a.dkrn);
   AsmIn in;
   in.u = (const double2*)a.u; in.Se = a.Se; in.pn = a.pn; in.pc = a.pc; in.dpc = a.dpc; in.krw = a.krw;
-  in.dkrw = a.dkrw; in.pdmin = a.pdmin; in.phiv = a.phiv; in.K = a.K; in.pd = a.pd; in.phi = a.phi;
+  in.dkrw = a.dkrw; in.krn = a.krn; in.dkrn = a.dkrn; in.pdmin = a.pdmin; in.phiv = a.phiv; in.K = a.K; in.pd = a.pd; in.phi = a.phi;
   in.vol = a.vol; in.dir = a.dir;
   in.pw_dir = a.pw_dir; in.q_in = (const double2*)a.q_in;
   in.law = a.law; in.kr_tab = a.kr_tab;
   const char* pv = getenv("RF_ASM_VERTEX");   // read per assembly (an alternative kept for comparison)
   const bool per_vertex = pv && atoi(pv) != 0;
   if (!per_vertex) {
-    launch_assemble_cells(d, ph, in, a, want_j, s);
+    if (d.dim == 3) {
+      if (want_j) slabs_t<3, true>(d, ph, in, a, s);
+      else slabs_t<3, false>(d, ph, in, a, s);
+    } else {
+      if (want_j) slabs_t<2, true>(d, ph, in, a, s);
+      else slabs_t<2, false>(d, ph, in, a, s);
+    }
     return cudaGetLastError();
   }
   const int BS = 128;
@@ -778,7 +1046,16 @@ void launch_storage_sw(const Dims& d, const PhysParams& pp, const double* u, con
   ph.S_wr = pp.S_wr; ph.S_nr = pp.S_nr; ph.lam = pp.lambda;
   ph.den = 1.0 - pp.S_wr - pp.S_nr;
   ph.scheme = pp.scheme;
-  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; }
+  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = 1.0 / pp.h[t]; }
+  ph.rmu_w = 1.0 / pp.mu_w;
+  ph.nid = -1.0 / ph.den;
+  for (int t = 0; t < 3; ++t) {
+    ph.Af[t] = 1.0;
+    for (int m = 0; m < d.dim; ++m)
+      if (m != t) ph.Af[t] *= pp.h[m] * 0.5;
+    ph.gw[t] = pp.rho_w * pp.g[t];
+    ph.gn[t] = pp.rho_n * pp.g[t];
+  }
   RF_LAUNCH(k_storage_sw, (int)((d.nv + 255) / 256), 256, 0, s, d, ph, (const double2*)u, pdmin, phi, pd, vol, sw);
 }
 

@@ -144,7 +144,8 @@ struct rf_grid {
   double *pdmin = nullptr, *phiv = nullptr;
   double *J = nullptr, *mdiag = nullptr;
   bool have_J = false;
-  double *Se, *pn, *pc, *dpc, *krw, *dkrw;
+  double *Se, *pn, *pc, *dpc, *krw, *dkrw, *krn, *dkrn;
+  double* faces = nullptr;      // face workspace of the assembly (column grids: of F alone)
   double *u_p = nullptr, *F_p = nullptr, *nat_a = nullptr, *nat_b = nullptr;
   // multigrid
   bool gmg_ready = false;
@@ -605,8 +606,9 @@ extern "C" rf_status rf_grid_create(const rf_grid_desc* desc, const rf_fluids* f
 
   NEED(g->J = (double*)dalloc(g, sizeof(double) * 4 * d.nb * nv, stream, false));
   NEED(g->mdiag = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
-  double** scratch[6] = {&g->Se, &g->pn, &g->pc, &g->dpc, &g->krw, &g->dkrw};
+  double** scratch[8] = {&g->Se, &g->pn, &g->pc, &g->dpc, &g->krw, &g->dkrw, &g->krn, &g->dkrn};
   for (auto p : scratch) NEED(*p = (double*)dalloc(g, sizeof(double) * nv, stream, false));
+  NEED(g->faces = (double*)dalloc(g, assemble_workspace(d, true), stream, false));
   NEED(g->u_p = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
   NEED(g->F_p = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
   // Krylov FP64 vectors (x padded: the outer operator reads it for the true residual)
@@ -643,6 +645,7 @@ extern "C" rf_status rf_grid_create(const rf_grid_desc* desc, const rf_fluids* f
 static rf_status assemble_p(rf_grid* g, bool want_j, void* s) {
   AsmArrays a;
   a.u = g->u_p; a.Se = g->Se; a.pn = g->pn; a.pc = g->pc; a.dpc = g->dpc; a.krw = g->krw; a.dkrw = g->dkrw;
+  a.krn = g->krn; a.dkrn = g->dkrn; a.faces = g->faces;
   a.pdmin = g->pdmin; a.phiv = g->phiv; a.K = g->Kcell; a.pd = g->pd; a.phi = g->phi; a.vol = g->vol;
   a.dir = g->dir; a.pw_dir = g->pw_dir;
   a.q_in = g->q_in; a.F = g->F_p; a.J = want_j ? g->J : nullptr; a.mdiag = want_j ? g->mdiag : nullptr;
@@ -1869,8 +1872,9 @@ static rf_status column_grid(rf_grid* g, int j, void* s, rf_grid** out) {
     const Dims& d = c->d;
     const int64_t nv = d.nv;
     bool ok = true;
-    double** scratch[6] = {&c->Se, &c->pn, &c->pc, &c->dpc, &c->krw, &c->dkrw};
+    double** scratch[8] = {&c->Se, &c->pn, &c->pc, &c->dpc, &c->krw, &c->dkrw, &c->krn, &c->dkrn};
     for (auto p : scratch) ok = ok && (*p = (double*)dalloc(c, sizeof(double) * nv, s, false));
+    ok = ok && (c->faces = (double*)dalloc(c, assemble_workspace(d, false), s, false));
     ok = ok && (c->u_p = (double*)dalloc(c, sizeof(double) * 2 * nv, s, false));
     ok = ok && (c->F_p = (double*)dalloc(c, sizeof(double) * 2 * nv, s, false));
     ok = ok && (c->K.x = (double2*)dvec(c, d, sizeof(double), s, false));
