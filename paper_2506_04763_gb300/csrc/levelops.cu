@@ -1559,6 +1559,194 @@ __global__ void k_dense(Dims d, Nbr nb, const double* __restrict__ J, const doub
   D[(2 * p + 1) * N + 2 * q + 1] = e3;
 }
 
+// Inverse by in-place Gauss-Jordan elimination with partial pivoting, one
+// thread-block cluster per matrix: CTA r of the cluster keeps rows r, r + cs,
+// ... in shared memory, and every step costs one cluster barrier.  Step c:
+//   - each CTA's first warp picks its largest |A[row][c]| over rows not yet
+//     used as pivots (the candidates were left by the previous update) and
+//     puts it, its row and its reciprocal into every CTA's table;
+//   - after the barrier all take the largest (the smaller row on ties) and
+//     copy the pivot row from its owner through distributed shared memory;
+//   - every other row: l = A[row][c] / pivot, A[row][t] -= l A[pivot][t], and
+//     A[row][c] = -l; one warp per row.  The pivot row itself is scaled by its
+//     owner one step later, when no one reads it any more.
+// Rows are never swapped: with pi(c) the pivot row of step c, the inverse is
+// Ainv[c][pi(t)] = B[pi(c)][t] of the final array B.  A pivot that is zero or
+// not finite, or a non-finite entry in the result (any NaN of A ends there),
+// sets status.
+// The one-CTA LU below does its N^3 / 3 multiply-adds on one SM's FP64 pipe (2
+// per clock) with four block barriers per column: 4.5 ms + 0.78 ms for the
+// inverse columns at N = 250 (5^3 vertices), 0.40 + 0.11 ms at N = 50 (5^2).
+// Spread over a cluster: 1.1 ms at N = 250, 0.10 ms at N = 50; what is left is
+// the step's chain of barrier, table, row copy and FP64 latencies (2 of 4.4 us
+// at N = 250).
+constexpr int GJ_THREADS = 512, GJ_MAX_CS = 16;
+
+struct GjShared {
+  long long key[2][GJ_MAX_CS];   // bits of |candidate|, -1: none (as integers: no FP64-pipe comparisons)
+  double inv[2][GJ_MAX_CS];
+  int row[2][GJ_MAX_CS];
+};
+
+__host__ __device__ inline size_t gj_smem(int N, int cs) {
+  const int rows = (N + cs - 1) / cs;
+  return sizeof(GjShared) + sizeof(double) * ((size_t)rows * N + N) + sizeof(long long) * rows +
+         sizeof(int) * (size_t)(N + rows + 2);
+}
+
+__device__ __forceinline__ long long gj_key(double v) {
+  const long long k = __double_as_longlong(fabs(v));
+  return k > 0x7ff0000000000000LL ? -1 : k;   // NaN: never a pivot
+}
+
+__global__ void __launch_bounds__(GJ_THREADS) k_gauss_jordan(int N, const double* __restrict__ D, InvOut out,
+                                                             int* __restrict__ status) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank(), mat = blockIdx.x / cs;
+  const int rows = (N + cs - 1) / cs, nloc = (N - rank + cs - 1) / cs;
+  extern __shared__ __align__(16) unsigned char gj_raw[];
+  GjShared& T = *reinterpret_cast<GjShared*>(gj_raw);
+  double* A = reinterpret_cast<double*>(gj_raw + sizeof(GjShared));   // [rows][N]
+  double* prow = A + (size_t)rows * N;
+  long long* cand = reinterpret_cast<long long*>(prow + N);           // [rows]
+  int* perm = reinterpret_cast<int*>(cand + rows);                    // [N]: pivot row of each step
+  int* step = perm + N;                                               // [rows]: step a local row was pivot of, or -1
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = GJ_THREADS >> 5;
+  D += (int64_t)mat * N * N;
+  for (int lr = warp; lr < nloc; lr += nw) {
+    const double* src = D + (int64_t)(lr * cs + rank) * N;
+    for (int t = lane; t < N; t += 32) {
+      const double v = src[t];
+      A[lr * N + t] = v;
+      if (t == 0) { cand[lr] = gj_key(v); step[lr] = -1; }
+    }
+  }
+  int pend = -1, pend_c = 0;      // the local row waiting for its scaling, its step and reciprocal pivot
+  double pend_inv = 0.0;
+  bool bad = false;
+  for (int c = 0; c < N; ++c) {
+    const int par = c & 1;
+    __syncthreads();
+    if (warp == 0) {
+      long long k = -1;
+      int r = N;
+      for (int lr = lane; lr < nloc; lr += 32)
+        if (cand[lr] > k) { k = cand[lr]; r = lr; }      // ascending rows: the first of equals stays
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long ok = __shfl_xor_sync(0xffffffffu, k, o);
+        const int orow = __shfl_xor_sync(0xffffffffu, r, o);
+        if (ok > k || (ok == k && orow < r)) { k = ok; r = orow; }
+      }
+      const double inv = k > 0 ? 1.0 / A[r * N + c] : 0.0;
+      if (lane < cs) {
+        GjShared& O = *cl.map_shared_rank(&T, lane);
+        O.key[par][rank] = k;
+        O.inv[par][rank] = inv;
+        O.row[par][rank] = k >= 0 ? r * cs + rank : N;
+      }
+    }
+    cl.sync();
+    long long k = -1;
+    int pr = N;
+    double inv = 0.0;
+#pragma unroll
+    for (int q = 0; q < GJ_MAX_CS; ++q) {
+      if (q >= cs) break;
+      const long long kq = T.key[par][q];
+      const int rq = T.row[par][q];
+      if (kq > k || (kq == k && rq < pr)) { k = kq; pr = rq; inv = T.inv[par][q]; }
+    }
+    if (k <= 0 || k >= 0x7ff0000000000000LL) { bad = true; break; }   // the same decision in every CTA
+    const int owner = pr % cs, plr = pr / cs;
+    const double* src = cl.map_shared_rank(A, owner) + plr * N;
+    for (int t = tid; t < N; t += GJ_THREADS) prow[t] = src[t];
+    if (tid == 0) perm[c] = pr;
+    __syncthreads();
+    for (int lr = warp; lr < nloc; lr += nw) {
+      if (rank == owner && lr == plr) {
+        if (lane == 0) { cand[lr] = -1; step[lr] = c; }
+        continue;
+      }
+      double* a = A + lr * N;
+      if (lr == pend) {
+        for (int t = lane; t < N; t += 32) a[t] = t == pend_c ? pend_inv : a[t] * pend_inv;
+        __syncwarp();
+      }
+      const double l = a[c] * inv;
+      __syncwarp();
+      const bool used = step[lr] >= 0;
+      for (int t = lane; t < N; t += 32) {
+        const double v = t == c ? -l : fma(-l, prow[t], a[t]);
+        a[t] = v;
+        if (t == c + 1) cand[lr] = used ? -1 : gj_key(v);
+      }
+    }
+    pend = rank == owner ? plr : -1;
+    pend_c = c;
+    pend_inv = inv;
+  }
+  cl.sync();   // no CTA leaves, or scales its last pivot row, while its rows are read
+  if (bad) {
+    if (tid == 0) status[mat] = 1;
+    return;
+  }
+  if (pend >= 0 && warp == 0)
+    for (int t = lane; t < N; t += 32) A[pend * N + t] = t == pend_c ? pend_inv : A[pend * N + t] * pend_inv;
+  __syncthreads();
+  double* __restrict__ Ainv = out.Ainv[mat];
+  bool finite = true;
+  for (int lr = warp; lr < nloc; lr += nw) {
+    double* dst = Ainv + (int64_t)step[lr] * N;
+    for (int t = lane; t < N; t += 32) {
+      const double v = A[lr * N + t];
+      finite = finite && ((__double2hiint(v) & 0x7ff00000) != 0x7ff00000);
+      dst[perm[t]] = v;
+    }
+  }
+  if (!finite) status[mat] = 1;
+}
+
+// Cluster size of k_gauss_jordan for N unknowns (0: it does not fit).  A step's
+// update takes N ceil(N / cs) multiply-adds of a CTA, its barrier and copies
+// grow with cs.  Measured for one inverse, cs = 1 / 4 / 8 / 16 (the call's 40 us
+// of launch and read-back included): N = 50 205 / 135 / 137 / 152 us, N = 90
+// 524 / 280 / 245 / 271, N = 126 1068 / 461 / 386 / 406, N = 144 1522 / 637 /
+// 523 / 488, N = 250 - / - / 1298 / 1131.
+static int gj_cluster(int N) {
+  static const int optin = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize, v) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return v;
+  }();
+  int cs = N <= 50 ? 4 : N < 144 ? 8 : 16;
+  while (cs < GJ_MAX_CS && gj_smem(N, cs) > (size_t)optin) cs *= 2;
+  return gj_smem(N, cs) <= (size_t)optin ? cs : 0;
+}
+
+static cudaError_t launch_gauss_jordan(int N, int nmat, int cs, const double* D, const InvOut& out, int* status, void* s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cs * nmat, 1, 1);
+  cfg.blockDim = dim3(GJ_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = gj_smem(N, cs);
+  cfg.stream = (cudaStream_t)s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, k_gauss_jordan, N, D, out, status);
+}
+
 // LU with partial pivoting in one CTA (first maximal pivot on ties).  Per
 // column: the pivot comes from candidates gathered while the previous column
 // was applied; after the row swap the pivot row (from c on) and the column's
@@ -2567,6 +2755,8 @@ cudaError_t launch_dense_inverse_batched(int N, int nmat, double* D, double* con
   if (nmat < 1 || nmat > RF_MAXSHIFT) return cudaErrorInvalidValue;
   InvOut out;
   for (int j = 0; j < RF_MAXSHIFT; ++j) out.Ainv[j] = j < nmat ? Ainv[j] : nullptr;
+  if (const int cs = gj_cluster(N)) return launch_gauss_jordan(N, nmat, cs, D, out, status, s);
+  // beyond a cluster's shared memory (N > ~650): LU in global memory
   const size_t lsm = sizeof(double) * 2 * (size_t)N;   // 64 KB at N = 4096
   cudaFuncSetAttribute(k_lu, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
   RF_LAUNCH(k_lu, nmat, 1024, lsm, s, N, D, piv, status);
