@@ -170,15 +170,18 @@ __device__ __forceinline__ void load_block(const void* A, int64_t nv, int b, int
   unpack_block<KIND>(r, sc, a);
 }
 
-// Row sum += (a_0 x_0 + a_1 x_1) for one block row: one explicit fused
-// multiply-add and an explicit add, so that every kernel applying a block
-// (per-block, batched, shared-matrix) rounds it identically, whatever the
-// compiler would otherwise contract.
+// Row sum += (a_0 x_0 + a_1 x_1) for one block row, in explicit operations, so
+// that every kernel applying a block (per-block, batched, shared-matrix) rounds
+// it identically, whatever the compiler would otherwise contract.  FP32: one
+// product, one multiply-add, one sum (a chain of one add per block).  FP64: two
+// multiply-adds, as these kernels are bound by the FP64 pipe (65^3 Jacobi: 104 us
+// a sweep with three operations per pair, 70 us with two; its 108 multiply-adds
+// per vertex take 56 us).
 __device__ __forceinline__ float blk_acc(float s, float a0, float a1, float2 x) {
   return __fadd_rn(s, __fmaf_rn(a0, x.x, __fmul_rn(a1, x.y)));
 }
 __device__ __forceinline__ double blk_acc(double s, double a0, double a1, double2 x) {
-  return __dadd_rn(s, __fma_rn(a0, x.x, __dmul_rn(a1, x.y)));
+  return __fma_rn(a0, x.x, __fma_rn(a1, x.y, s));
 }
 
 // FP16 storage holds the blocks of a row in pairs, one 16-byte load per pair
