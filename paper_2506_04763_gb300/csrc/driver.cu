@@ -145,7 +145,8 @@ struct rf_grid {
   double *J = nullptr, *mdiag = nullptr;
   bool have_J = false;
   double *Se, *pn, *pc, *dpc, *krw, *dkrw, *krn, *dkrn;
-  double* faces = nullptr;      // face workspace of the assembly (column grids: of F alone)
+  double* faces = nullptr;      // workspace of the assembly (column grids: of F alone) and of the Galerkin products
+  size_t faces_bytes = 0;
   double *u_p = nullptr, *F_p = nullptr, *nat_a = nullptr, *nat_b = nullptr;
   // multigrid
   bool gmg_ready = false;
@@ -608,7 +609,9 @@ extern "C" rf_status rf_grid_create(const rf_grid_desc* desc, const rf_fluids* f
   NEED(g->mdiag = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
   double** scratch[8] = {&g->Se, &g->pn, &g->pc, &g->dpc, &g->krw, &g->dkrw, &g->krn, &g->dkrn};
   for (auto p : scratch) NEED(*p = (double*)dalloc(g, sizeof(double) * nv, stream, false));
-  NEED(g->faces = (double*)dalloc(g, assemble_workspace(d, true), stream, false));
+  // (a Galerkin workspace beyond GAL_WS_BYTES, of grids with very large planes, waits for the set-up)
+  g->faces_bytes = std::max(assemble_workspace(d, true), std::min(galerkin_workspace(d), GAL_WS_BYTES));
+  NEED(g->faces = (double*)dalloc(g, g->faces_bytes, stream, false));
   NEED(g->u_p = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
   NEED(g->F_p = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
   // Krylov FP64 vectors (x padded: the outer operator reads it for the true residual)
@@ -842,53 +845,6 @@ static rf_status autotune_levels(rf_grid* g, void* s) {
   return RF_OK;
 }
 
-static void dfree_ptr(rf_grid* g, void* p, void* s) {
-  for (size_t i = 0; i < g->gbufs.size(); ++i)
-    if (g->gbufs[i].p == p) {
-      if (g->user_alloc) g->alloc.free(p, g->gbufs[i].bytes, s, g->alloc.ctx);
-      else cudaFree(p);
-      g->gbufs.erase(g->gbufs.begin() + i);
-      return;
-    }
-}
-
-// Galerkin operators of level C from level F, one axis at a time (x, y[, z]);
-// intermediate operators live only for the duration of the call.
-static rf_status galerkin_level(rf_grid* g, const Level& F, Level& C, bool from_fine, void* s) {
-  const int dim = F.d.dim;
-  const double* Jin = from_fine ? g->J : F.Jc;
-  const double* Min = from_fine ? nullptr : F.Mc;
-  const double* md = from_fine ? g->mdiag : nullptr;
-  int n[3] = {F.d.nx, F.d.ny, F.d.nz};
-  Dims cur = F.d;
-  std::vector<void*> temps;
-  rf_status st = RF_OK;
-  for (int axis = 0; axis < dim; ++axis) {
-    n[axis] = (n[axis] - 1) / 2 + 1;
-    const Dims nxt = make_dims(dim, n);
-    const bool last = axis == dim - 1;
-    double* Jo = C.Jc;
-    double* Mo = C.Mc;
-    if (!last) {
-      Jo = (double*)dalloc(g, sizeof(double) * 4 * nxt.nb * nxt.nv, s, true);
-      Mo = (double*)dalloc(g, sizeof(double) * 2 * nxt.nb * nxt.nv, s, true);
-      if (Jo) temps.push_back(Jo);
-      if (Mo) temps.push_back(Mo);
-      if (!Jo || !Mo) { st = fail(RF_ENOMEM, "Galerkin temporaries"); break; }
-    }
-    launch_galerkin_axis(axis, cur, axis == 0 ? F.dmask : nullptr, Jin, Min, md, nxt, last ? C.dmask : nullptr, Jo,
-                         Mo, s);
-    Jin = Jo;
-    Min = Mo;
-    md = nullptr;
-    cur = nxt;
-  }
-  cudaError_t e = cudaStreamSynchronize((cudaStream_t)s);
-  for (void* p : temps) dfree_ptr(g, p, s);
-  if (st == RF_OK && e != cudaSuccess) st = fail(RF_ECUDA, "Galerkin: %s", cudaGetErrorString(e));
-  return st;
-}
-
 #define GNEED(ptr)                                                                     \
   do {                                                                                 \
     if (!(ptr)) { dfree_all(g, g->gbufs, s); return fail(RF_ENOMEM, "device allocation failed (%s)", #ptr); } \
@@ -935,6 +891,12 @@ extern "C" rf_status rf_gmg_setup(rf_grid* g, const double* shifts, int nshift, 
     ++g->nl;
   }
   const int kind = g->kind;
+  double* gal_ws = g->faces;
+  size_t gal_bytes = g->faces_bytes;
+  if (g->nl > 1 && galerkin_workspace(g->d) > g->faces_bytes) {
+    gal_bytes = galerkin_workspace(g->d);
+    GNEED(gal_ws = (double*)dalloc(g, gal_bytes, s, true));
+  }
   for (int l = 0; l < g->nl; ++l) {
     Level& Lv = g->L[l];
     Lv.nb = make_nbr(Lv.d);
@@ -948,33 +910,32 @@ extern "C" rf_status rf_gmg_setup(rf_grid* g, const double* shifts, int nshift, 
       launch_coarse_mask(g->L[l - 1].d, g->L[l - 1].dmask, d, Lv.dmask, s);
       GNEED(Lv.Jc = (double*)dalloc(g, sizeof(double) * 4 * d.nb * d.nv, s, true));
       GNEED(Lv.Mc = (double*)dalloc(g, sizeof(double) * 2 * d.nb * d.nv, s, true));
-      rf_status gst = galerkin_level(g, g->L[l - 1], Lv, l == 1, s);
-      if (gst) { dfree_all(g, g->gbufs, s); return gst; }
+      const Level& Lf = g->L[l - 1];
+      launch_galerkin(Lf.d, Lf.dmask, l == 1 ? g->J : Lf.Jc, l == 1 ? nullptr : Lf.Mc, l == 1 ? g->mdiag : nullptr, d,
+                      Lv.dmask, Lv.Jc, Lv.Mc, gal_ws, gal_bytes, s);
     }
     const int lk = Lv.kind;
     const size_t te = t_size(kind), se = s_size(lk);
     if (l < g->nl - 1 || g->nl == 1) {
       // smoothed levels: storage + inverse diagonal blocks per shift
-      if (l == 0) {
-        if (kind == STORE_F64) {
-          Lv.A[0] = g->J;
-        } else {
-          GNEED(Lv.A[0] = dalloc(g, se * 4 * stored_blocks(kind, d.nb) * d.nv, s, true));
-          if (kind == STORE_F16) GNEED(Lv.scale[0] = (float*)dalloc(g, sizeof(float) * 4 * d.nv, s, true));
-          launch_pack_level(d, true, g->J, nullptr, g->mdiag, 0.0, kind, Lv.A[0], Lv.scale[0], nullptr, s);
-        }
-        for (int j = 0; j < nshift; ++j) {
-          GNEED(Lv.Dinv[j] = dalloc(g, te * 4 * d.nv, s, true));
-          launch_pack_level(d, true, g->J, nullptr, g->mdiag, shifts[j], kind, nullptr, nullptr, Lv.Dinv[j], s);
-        }
-      } else {
-        for (int j = 0; j < nshift; ++j) {
-          GNEED(Lv.A[j] = dalloc(g, se * 4 * stored_blocks(lk, d.nb) * d.nv, s, true));
-          if (lk == STORE_F16) GNEED(Lv.scale[j] = (float*)dalloc(g, sizeof(float) * 4 * d.nv, s, true));
-          GNEED(Lv.Dinv[j] = dalloc(g, te * 4 * d.nv, s, true));
-          launch_pack_level(d, false, Lv.Jc, Lv.Mc, nullptr, shifts[j], lk, Lv.A[j], Lv.scale[j], Lv.Dinv[j], s);
-        }
+      PackOut po{};
+      po.n = nshift;
+      for (int j = 0; j < nshift; ++j) {
+        po.shift[j] = shifts[j];
+        GNEED(Lv.Dinv[j] = dalloc(g, te * 4 * d.nv, s, true));
+        po.Dinv[j] = Lv.Dinv[j];
       }
+      if (l == 0 && kind == STORE_F64) {
+        Lv.A[0] = g->J;          // the finest FP64 level smooths with J itself
+        po.diag_only = true;
+      } else {
+        for (int j = 0; j < (l == 0 ? 1 : nshift); ++j) {
+          GNEED(Lv.A[j] = dalloc(g, se * 4 * stored_blocks(lk, d.nb) * d.nv, s, true));
+          po.A[j] = Lv.A[j];
+        }
+        if (lk == STORE_F16) GNEED(Lv.scale[0] = (float*)dalloc(g, sizeof(float) * 4 * d.nv, s, true));
+      }
+      launch_pack_level(d, l == 0, l == 0 ? g->J : Lv.Jc, Lv.Mc, g->mdiag, lk, po, Lv.scale[0], s);
     }
     GNEED(Lv.x = dvec(g, d, te, s, true, &Lv.pad));
     GNEED(Lv.b = dvec(g, d, te, s, true));

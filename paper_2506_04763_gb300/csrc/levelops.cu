@@ -1370,90 +1370,246 @@ cudaError_t launch_vcycle_tail(const TailParams& P, int kind, int nb, int csize,
 // so P_m^T A P_m = D_c P^T (D_f A D_f) P D_c is computed as three 1D
 // coarsenings (x, then y, then z): the output grid halves one axis, every
 // block offset along that axis becomes a coarse offset, the other offsets stay.
-// Output entry (I, D) along the axis = sum over fine rows 2I+a (weight w_a) and
-// fine columns 2(I+D)+c (weight w_c), |2D+c-a| <= 1, w_0 = 1, w_+-1 = 1/2.
+// With L, C, R the blocks of fine rows 2I - 1, 2I, 2I + 1 (missing rows are
+// zero) at offsets -1, 0, 1 along the axis, the output blocks of row I are
+//   D = -1: (L[-1] + L[0]/2 + C[-1]) / 2
+//   D =  0: C[0] + (C[-1] + C[1] + L[1] + R[-1] + (L[0] + R[0])/2) / 2
+//   D = +1: (R[1] + R[0]/2 + C[1]) / 2.
 // The fine masks D_f are applied while reading the first stage, the coarse
 // masks D_c (and the identity of coarse Dirichlet rows) when writing the last.
-__global__ void __launch_bounds__(256) k_galerkin_axis(int axis, Dims din, const uint8_t* __restrict__ dmf,
-                                                       const double* __restrict__ Jin, const double* __restrict__ Min,
-                                                       const double2* __restrict__ mdiag, Dims dout,
-                                                       const uint8_t* __restrict__ dmc, double* __restrict__ Jout,
-                                                       double* __restrict__ Mout) {
-  const int nb = dout.nb;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= dout.nv * nb) return;
-  const int bo = (int)(t / dout.nv);
-  const int64_t po = t - (int64_t)bo * dout.nv;
-  int oc[3];
-  pcoords(dout, po, oc[0], oc[1], oc[2]);
-  int off[3] = {bo % 3 - 1, (bo / 3) % 3 - 1, dout.dim == 3 ? bo / 9 - 1 : 0};
-  const int nin[3] = {din.nx, din.ny, din.nz}, nout[3] = {dout.nx, dout.ny, dout.nz};
-  const int D = off[axis];
-  double j0 = 0, j1 = 0, j2 = 0, j3 = 0, m0 = 0, m1 = 0;
-  const int Ic = oc[axis];
-  // the column vertex must exist on the output grid
-  bool col_ok = Ic + D >= 0 && Ic + D < nout[axis];
-  for (int q = 0; q < 3; ++q)
-    if (q != axis && (oc[q] + off[q] < 0 || oc[q] + off[q] >= nout[q])) col_ok = false;
-  if (col_ok) {
-    for (int a = -1; a <= 1; ++a) {
-      const int f = 2 * Ic + a;
-      if (f < 0 || f >= nin[axis]) continue;
-      int rc[3] = {oc[0], oc[1], oc[2]};
-      rc[axis] = f;
-      const int64_t pi = pidx(din, rc[0], rc[1], rc[2]);
-      const double wa = a ? 0.5 : 1.0;
-      const bool mrow = dmf && dmf[pi];
-      for (int c = -1; c <= 1; ++c) {
-        const int e = 2 * D + c - a;
-        if (e < -1 || e > 1) continue;
-        const int gcol = 2 * (Ic + D) + c;
-        if (gcol < 0 || gcol >= nin[axis]) continue;
-        const double w = wa * (c ? 0.5 : 1.0);
-        int eo[3] = {off[0], off[1], off[2]};
-        eo[axis] = e;
-        const int bi = blk_of(din.dim, eo[0], eo[1], eo[2]);
-        bool mcol = false;
-        if (dmf) {
-          int cc[3] = {rc[0] + eo[0], rc[1] + eo[1], rc[2] + eo[2]};
-          mcol = dmf[pidx(din, cc[0], cc[1], cc[2])] != 0;
-        }
-        const double* A = Jin + ((int64_t)bi * din.nv + pi) * 4;
-        const double a0 = mrow || mcol ? 0.0 : A[0], a1 = mrow ? 0.0 : A[1], a2 = mcol ? 0.0 : A[2], a3 = A[3];
-        j0 += w * a0; j1 += w * a1; j2 += w * a2; j3 += w * a3;
-        double s0, s1;
-        if (Min) {
-          const double* M = Min + ((int64_t)bi * din.nv + pi) * 2;
-          s0 = M[0]; s1 = M[1];
-        } else {
-          const bool centre = eo[0] == 0 && eo[1] == 0 && eo[2] == 0;
-          const double2 md = centre ? mdiag[pi] : make_double2(0.0, 0.0);
-          s0 = md.x; s1 = md.y;
-        }
-        m0 += w * (mrow ? 0.0 : s0);
-        m1 += w * s1;
-      }
-    }
-    if (dmc) {
-      const bool crow = dmc[po] != 0;
-      const bool ccol = dmc[pidx(dout, oc[0] + off[0], oc[1] + off[1], oc[2] + off[2])] != 0;
-      if (crow) { j0 = 0.0; j1 = 0.0; m0 = 0.0; }
-      if (ccol) { j0 = 0.0; j2 = 0.0; }
-      if (crow && bo == (dout.dim == 3 ? 13 : 4)) j0 = -1.0;   // Dirichlet row: A = +identity
-    }
+//
+// A thread makes the three blocks D of one row and one pair of other offsets:
+// 9 block loads and 12 FP64 operations per entry (the set-up is FP64-pipe-bound
+// on large grids).  M of the finest level is vertex-diagonal, so until the
+// stages have spread it along an axis its blocks off that axis are zero and
+// neither read nor written.  The stages run over windows of planes along the
+// last axis, the intermediate operators of a window in a workspace that stays
+// with the grid: the x stage's planes, and the y stage's planes in a ring, as
+// the last plane of a window is also the first of the next (2D: the x stage's
+// planes are the ring).  129^3 -> 65^3: one thread per output block over whole
+// intermediate grids, its products and M's zeros unshared, took 3.63 ms (x 2.44,
+// y 0.78, z 0.40) and 2 GB of temporaries; now 1.98 ms (1.02, 0.56, 0.40).
+struct GalView {            // an operator, whole or a window of its planes
+  const double* J;          // [block][plane slot][in-plane][4]
+  const double* M;          // [block][plane slot][in-plane][2]; null: mdiag
+  int64_t bs;               // vertices per block
+  int f0, ring;             // plane q is slot q - f0, or q % ring where ring > 0
+  __device__ __forceinline__ int64_t at(int pp, int plane, int q) const {
+    return (int64_t)(ring > 0 ? (int)((uint32_t)plane % (uint32_t)ring) : plane - f0) * pp + q;
   }
-  double* o = Jout + ((int64_t)bo * dout.nv + po) * 4;
-  o[0] = j0; o[1] = j1; o[2] = j2; o[3] = j3;
-  double* om = Mout + ((int64_t)bo * dout.nv + po) * 2;
-  om[0] = m0; om[1] = m1;
+};
+struct GalStage {
+  int nxi, nyi, nzi, nxo, nyo;   // in-plane extents before and after, planes before (2D: ny = 1, planes along y)
+  int o0, o1;                    // output planes
+  bool mfull;                    // the source's M is a full stencil (not the finest level's diagonal)
+  const double2* mdiag;
+  const uint8_t *dmf, *dmc;
+  GalView in, out;
+};
+
+template <int DIM>
+__device__ __forceinline__ int gal_blk(int dx, int dy, int dz) {
+  return DIM == 3 ? (dx + 1) + 3 * (dy + 1) + 9 * (dz + 1) : (dx + 1) + 3 * (dz + 1);
 }
 
-void launch_galerkin_axis(int axis, const Dims& din, const uint8_t* dmf, const double* Jin, const double* Min,
-                          const double* mdiag, const Dims& dout, const uint8_t* dmc, double* Jout, double* Mout,
-                          void* s) {
-  const int64_t n = dout.nv * dout.nb;
-  RF_LAUNCH(k_galerkin_axis, (int)((n + 255) / 256), 256, 0, s, axis, din, dmf, Jin, Min, (const double2*)mdiag,
-            dout, dmc, Jout, Mout);
+__device__ __forceinline__ double2 gal_half(double2 a, double2 b) {   // a + b / 2
+  return make_double2(fma(0.5, b.x, a.x), fma(0.5, b.y, a.y));
+}
+__device__ __forceinline__ double2 gal_add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 gal_scale(double2 a) { return make_double2(0.5 * a.x, 0.5 * a.y); }
+
+// AX: 0 = x, 1 = y (3D), 2 = the last axis
+template <int DIM, int AX>
+__global__ void __launch_bounds__(128) k_galerkin(const __grid_constant__ GalStage S) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int ppo = S.nxo * S.nyo, ppi = S.nxi * S.nyi;
+  if (t >= (int64_t)(S.o1 - S.o0) * ppo) return;
+  const uint32_t line = (uint32_t)t / (uint32_t)S.nxo, pl = line / (uint32_t)S.nyo;
+  const int xt = (int)((uint32_t)t - line * (uint32_t)S.nxo), yo = (int)(line - pl * (uint32_t)S.nyo);
+  const int zo = S.o0 + (int)pl;
+  const int Eo = (S.nxo + 1) / 2, Ei = (S.nxi + 1) / 2;
+  // x: threads in natural order (the fine rows they read are contiguous runs);
+  // y, last: in parity-split order, unchanged by the stage
+  const int xo = AX == 0 ? xt : (xt < Eo ? 2 * xt : 2 * (xt - Eo) + 1);
+  const int xpo = AX == 0 ? ((xt & 1) ? Eo + (xt >> 1) : (xt >> 1)) : xt;
+  // the two other offsets of this thread's blocks
+  const int g0 = (int)blockIdx.y % 3 - 1, g1 = DIM == 3 ? (int)blockIdx.y / 3 - 1 : 0;
+  const int dx = AX == 0 ? 0 : g0, dy = AX == 0 ? (DIM == 3 ? g0 : 0) : AX == 1 ? 0 : (DIM == 3 ? g1 : 0);
+  const int dz = AX == 0 ? (DIM == 3 ? g1 : g0) : AX == 1 ? g1 : 0;
+  const int c = AX == 0 ? xo : AX == 1 ? yo : zo;                  // I
+  const int nin = AX == 0 ? S.nxi : AX == 1 ? S.nyi : S.nzi;
+  const int bst = AX == 0 ? 1 : AX == 1 ? 3 : (DIM == 3 ? 9 : 3);  // block step along the axis
+  const int b0 = gal_blk<DIM>(dx, dy, dz);                         // offset 0 along the axis
+  int64_t pr[3];
+  bool has[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int f = 2 * c + a - 1;
+    has[a] = f >= 0 && f < nin;
+    if (AX == 0) pr[a] = S.in.at(ppi, zo, yo * S.nxi + ((f & 1) ? Ei + (f >> 1) : (f >> 1)));
+    else if (AX == 1) pr[a] = S.in.at(ppi, zo, f * S.nxi + xt);
+    else pr[a] = has[a] ? S.in.at(ppi, f, yo * S.nxi + xt) : 0;
+  }
+  // first stage: row masks of the three rows, column masks of the five columns
+  uint32_t mrow = 0, mcol = 0;
+  if (AX == 0 && S.dmf) {
+    const int yc = yo + dy, zc = zo + dz;
+    const bool cin = yc >= 0 && yc < S.nyi && zc >= 0 && zc < S.nzi;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      const int f = 2 * c + q - 2;
+      if (f < 0 || f >= S.nxi) continue;
+      const int xp = (f & 1) ? Ei + (f >> 1) : (f >> 1);
+      if (cin && S.dmf[((int64_t)zc * S.nyi + yc) * S.nxi + xp]) mcol |= 1u << q;
+      if (q >= 1 && q <= 3 && S.dmf[((int64_t)zo * S.nyi + yo) * S.nxi + xp]) mrow |= 1u << (q - 1);
+    }
+  }
+  bool crow = false, ccol[3] = {false, false, false};
+  if (AX == 2 && S.dmc) {
+    const int nzo = (S.nzi - 1) / 2 + 1;
+    crow = S.dmc[((int64_t)zo * S.nyo + yo) * S.nxo + xt] != 0;
+    const int xc = xo + dx, yc = yo + dy;
+    const bool cin = xc >= 0 && xc < S.nxo && yc >= 0 && yc < S.nyo;
+    const int xp = (xc & 1) ? Eo + (xc >> 1) : (xc >> 1);
+#pragma unroll
+    for (int D = -1; D <= 1; ++D)
+      if (cin && zo + D >= 0 && zo + D < nzo) ccol[D + 1] = S.dmc[((int64_t)(zo + D) * S.nyo + yc) * S.nxo + xp] != 0;
+  }
+  const int64_t po = S.out.at(ppo, zo, yo * S.nxo + xpo);
+  const int h0 = gridDim.z == 2 ? (int)blockIdx.z : 0, h1 = gridDim.z == 2 ? h0 + 1 : 2;
+  // M along the axes the stages have not reached yet: only the diagonal
+  const bool has_m = S.mfull || (AX == 0 ? (dy == 0 && dz == 0) : AX == 1 ? dz == 0 : true);
+  for (int h = h0; h < h1; ++h) {          // h = 0: the water row's entries, 1: the NAPL row's
+    double2 A[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        // row a - 1 reaches offset e - 1: L[-1], L[0], L[1], C[..], R[..]
+        A[a][e] = make_double2(0.0, 0.0);
+        if (has[a]) A[a][e] = reinterpret_cast<const double2*>(S.in.J)[((int64_t)(b0 + (e - 1) * bst) * S.in.bs + pr[a]) * 2 + h];
+        if (AX == 0) {
+          const bool mr = (mrow >> a) & 1, mc = (mcol >> (a + e)) & 1;
+          if ((h == 0 && mr) || mc) A[a][e].x = 0.0;
+          if (h == 0 && mr) A[a][e].y = 0.0;
+        }
+      }
+    double2 o[3];
+    o[0] = gal_scale(gal_add(gal_half(A[0][0], A[0][1]), A[1][0]));
+    o[1] = gal_half(A[1][1], gal_half(gal_add(gal_add(A[1][0], A[1][2]), gal_add(A[0][2], A[2][0])), gal_add(A[0][1], A[2][1])));
+    o[2] = gal_scale(gal_add(gal_half(A[2][2], A[2][1]), A[1][2]));
+    double m[3] = {0.0, 0.0, 0.0};
+    if (has_m) {
+      double B[3][3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          B[a][e] = 0.0;
+          if (!has[a] || (!S.mfull && e != 1)) continue;
+          if (S.in.M) B[a][e] = S.in.M[((int64_t)(b0 + (e - 1) * bst) * S.in.bs + pr[a]) * 2 + h];
+          else B[a][e] = h == 0 ? S.mdiag[pr[a]].x : S.mdiag[pr[a]].y;
+          if (AX == 0 && h == 0 && ((mrow >> a) & 1)) B[a][e] = 0.0;
+        }
+      m[0] = 0.5 * (fma(0.5, B[0][1], B[0][0]) + B[1][0]);
+      m[1] = fma(0.5, fma(0.5, B[0][1] + B[2][1], (B[1][0] + B[1][2]) + (B[0][2] + B[2][0])), B[1][1]);
+      m[2] = 0.5 * (fma(0.5, B[2][1], B[2][2]) + B[1][2]);
+    }
+#pragma unroll
+    for (int D = 0; D < 3; ++D) {
+      const int bo = b0 + (D - 1) * bst;
+      if (AX == 2 && S.dmc) {
+        if (h == 0 && crow) { o[D] = make_double2(0.0, 0.0); m[D] = 0.0; }
+        if (ccol[D]) o[D].x = 0.0;
+        if (h == 0 && crow && bo == (DIM == 3 ? 13 : 4)) o[D].x = -1.0;   // Dirichlet row: A = +identity
+      }
+      reinterpret_cast<double2*>(const_cast<double*>(S.out.J))[((int64_t)bo * S.out.bs + po) * 2 + h] = o[D];
+      if (has_m) const_cast<double*>(S.out.M)[((int64_t)bo * S.out.bs + po) * 2 + h] = m[D];
+    }
+  }
+}
+
+// Doubles per plane of the x stage and of the ring, and the planes along the
+// last axis that a window may hold in `bytes` (at least 4: two new fine planes,
+// the kept one, and the last).
+static int gal_window(const Dims& f, size_t bytes, int64_t& t1, int64_t& t2) {
+  const int nxc = (f.nx - 1) / 2 + 1, nyc = (f.ny - 1) / 2 + 1;
+  t1 = f.dim == 3 ? (int64_t)nxc * f.ny * f.nb * 6 : 0;
+  t2 = (f.dim == 3 ? (int64_t)nxc * nyc : (int64_t)nxc) * f.nb * 6;
+  const int nz = f.dim == 3 ? f.nz : f.ny;
+  int64_t n = (int64_t)(bytes / sizeof(double)) / (t1 + t2);
+  if (n < 4) n = 4;
+  return (int)(n < nz ? n : nz);
+}
+
+size_t galerkin_workspace(const Dims& f) {
+  int64_t t1, t2;
+  const int planes = gal_window(f, GAL_WS_BYTES, t1, t2);
+  return sizeof(double) * (size_t)(t1 + t2) * planes;
+}
+
+template <int DIM, int AX>
+static void gal_launch(const GalStage& S, void* s) {
+  const int64_t n = (int64_t)(S.o1 - S.o0) * S.nxo * S.nyo;
+  if (n <= 0) return;
+  // small windows take the two halves of a block in separate threads
+  const dim3 g((unsigned)((n + 127) / 128), DIM == 3 ? 9 : 3, n <= 32768 ? 2 : 1);
+  RF_LAUNCH((k_galerkin<DIM, AX>), g, 128, 0, s, S);
+}
+
+// Galerkin operators (Jc, Mc) of coarse level c from level f: J, M of level f
+template <int DIM>
+static void galerkin_t(const Dims& f, const uint8_t* dmf, const double* J, const double* M, const double* mdiag,
+                       const Dims& c, const uint8_t* dmc, double* Jc, double* Mc, double* ws, size_t ws_bytes, void* s) {
+  int64_t t1, t2;
+  const int planes = gal_window(f, ws_bytes, t1, t2);
+  const int nz = DIM == 3 ? f.nz : f.ny, nzc = DIM == 3 ? c.nz : c.ny;
+  const int nyf = DIM == 3 ? f.ny : 1, nyc = DIM == 3 ? c.ny : 1;
+  // workspace: x planes (J then M), ring planes (J then M)
+  const int64_t v1 = (int64_t)c.nx * nyf, v2 = (int64_t)c.nx * nyc;   // vertices per plane
+  double* w2 = ws + t1 * planes;
+  GalStage S{};
+  S.mfull = M != nullptr;
+  S.mdiag = (const double2*)mdiag;
+  S.nzi = nz;
+  // windows: fine planes [f0, f1) join the ring, then coarse planes K with 2K + 1 < f1 (or at the end, all)
+  int K0 = 0;
+  for (int f0 = 0; f0 < nz;) {
+    int f1 = f0 == 0 ? planes : f0 + planes - 1;
+    if (f1 < nz && (f1 & 1)) --f1;      // an even count so far: the plane kept is 2K - 1
+    if (f1 > nz) f1 = nz;
+    const GalView src{J, M, f.nv, 0, 0};
+    const GalView ring{w2, w2 + (int64_t)4 * f.nb * v2 * planes, v2 * planes, 0, planes};
+    const GalView x1{ws, ws + (int64_t)4 * f.nb * v1 * (f1 - f0), v1 * (f1 - f0), f0, 0};
+    S.nxi = f.nx; S.nyi = nyf; S.nxo = c.nx; S.nyo = nyf;
+    S.o0 = f0; S.o1 = f1;
+    S.dmf = dmf; S.dmc = nullptr;
+    S.in = src;
+    S.out = DIM == 3 ? x1 : ring;
+    gal_launch<DIM, 0>(S, s);
+    S.dmf = nullptr;
+    if (DIM == 3) {
+      S.nxi = c.nx; S.nyo = nyc;
+      S.in = x1;
+      S.out = ring;
+      gal_launch<DIM, 1>(S, s);
+    }
+    S.nxi = c.nx; S.nyi = nyc; S.nxo = c.nx; S.nyo = nyc;
+    S.dmc = dmc;
+    S.in = ring;
+    S.out = GalView{Jc, Mc, c.nv, 0, 0};
+    const int K1 = f1 == nz ? nzc : f1 / 2;
+    S.o0 = K0; S.o1 = K1;
+    gal_launch<DIM, 2>(S, s);
+    K0 = K1;
+    f0 = f1;
+  }
+}
+
+void launch_galerkin(const Dims& f, const uint8_t* dmf, const double* J, const double* M, const double* mdiag,
+                     const Dims& c, const uint8_t* dmc, double* Jc, double* Mc, double* ws, size_t ws_bytes, void* s) {
+  if (f.dim == 3) galerkin_t<3>(f, dmf, J, M, mdiag, c, dmc, Jc, Mc, ws, ws_bytes, s);
+  else galerkin_t<2>(f, dmf, J, M, mdiag, c, dmc, Jc, Mc, ws, ws_bytes, s);
 }
 
 __global__ void k_coarse_mask(Dims df, const uint8_t* __restrict__ dmf, Dims dc, uint8_t* __restrict__ dmc) {
@@ -1465,70 +1621,130 @@ __global__ void k_coarse_mask(Dims df, const uint8_t* __restrict__ dmf, Dims dc,
 }
 
 // ----------------------------------------------------------------- packing
-// Per vertex: entries of A (coarse: shift*Mc - Jc; fine: J itself) into the
-// storage kind, FP16 with one FP32 scale per entry position over the block
-// row, and the inverse of the 2x2 diagonal block of A = shift*M - J.
-template <int KIND>
-__global__ void k_pack(Dims d, bool fine, const double* __restrict__ J, const double* __restrict__ M,
-                       const double2* __restrict__ md, double shift, void* __restrict__ Aout,
-                       float* __restrict__ scale, typename Ty<KIND>::T* __restrict__ Dinv) {
-  typedef typename Ty<KIND>::T T;
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// Entries of A (coarse: shift*Mc - Jc for every shift; fine: J itself) in the
+// storage kind, FP64 or FP32: a thread takes CH blocks of one vertex, J and M
+// read once for all shifts.  Large levels take 9 (their loads in flight), small
+// ones 1 (one thread per vertex walking 27 blocks took 24 us on the smallest
+// levels, once per shift; now 8 us for all).
+__device__ __forceinline__ void store_block(double a, double b, double c, double e, double* o) {
+  reinterpret_cast<double2*>(o)[0] = make_double2(a, b);
+  reinterpret_cast<double2*>(o)[1] = make_double2(c, e);
+}
+__device__ __forceinline__ void store_block(double a, double b, double c, double e, float* o) {
+  *reinterpret_cast<float4*>(o) = make_float4((float)a, (float)b, (float)c, (float)e);
+}
+
+template <typename T, int CH>
+__global__ void __launch_bounds__(256) k_pack(Dims d, bool fine, const double* __restrict__ J, const double* __restrict__ M,
+                                              const __grid_constant__ PackOut out) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= d.nv) return;
-  const int nb = d.nb, C = d.dim == 3 ? 13 : 4;
-  if (Aout) {
-    double mx[4] = {0, 0, 0, 0};
-    for (int b = 0; b < nb; ++b) {
-      const double* a = J + ((int64_t)b * d.nv + p) * 4;
-      double e[4] = {a[0], a[1], a[2], a[3]};
-      if (!fine) {
-        const double* m = M + ((int64_t)b * d.nv + p) * 2;
-        e[0] = -e[0]; e[1] = shift * m[0] - e[1]; e[2] = -e[2]; e[3] = shift * m[1] - e[3];
-      }
-      if (KIND == STORE_F16) {
-        for (int q = 0; q < 4; ++q) mx[q] = fmax(mx[q], fabs(e[q]));
-      } else {
-        typename Ty<KIND>::S* o = reinterpret_cast<typename Ty<KIND>::S*>(Aout) + ((int64_t)b * d.nv + p) * 4;
-        for (int q = 0; q < 4; ++q) o[q] = (typename Ty<KIND>::S)e[q];
-      }
-    }
-    if (KIND == STORE_F16) {
-      // A position whose largest magnitude is below the smallest normal float
-      // holds only entries that FP32 arithmetic flushes anyway: scale 1, entries 0.
-      float sc[4];
-      for (int q = 0; q < 4; ++q) sc[q] = mx[q] >= 1.17549435e-38 ? (float)mx[q] : 1.0f;
-      reinterpret_cast<float4*>(scale)[p] = make_float4(sc[0], sc[1], sc[2], sc[3]);
-      for (int b = 0; b < nb; ++b) {
-        const double* a = J + ((int64_t)b * d.nv + p) * 4;
-        double e[4] = {a[0], a[1], a[2], a[3]};
-        if (!fine) {
-          const double* m = M + ((int64_t)b * d.nv + p) * 2;
-          e[0] = -e[0]; e[1] = shift * m[0] - e[1]; e[2] = -e[2]; e[3] = shift * m[1] - e[3];
-        }
-        const int sl = f16_slot_of_block(nb, b);   // paired layout, see stencil_sum_f16
-        __half* o = reinterpret_cast<__half*>(Aout) + (((int64_t)(sl >> 1) * d.nv + p) * 2 + (sl & 1)) * 4;
-        for (int q = 0; q < 4; ++q) o[q] = __double2half(e[q] / (double)sc[q]);
-      }
-      if (nb & 1) {   // the empty slot
-        __half* o = reinterpret_cast<__half*>(Aout) + (((int64_t)(nb >> 1) * d.nv + p) * 2 + 1) * 4;
-        for (int q = 0; q < 4; ++q) o[q] = __float2half(0.f);
-      }
+  const int b0 = blockIdx.y * CH;
+  double2 u[CH], w[CH], m[CH];
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    const double2* a = reinterpret_cast<const double2*>(J) + ((int64_t)(b0 + c) * d.nv + p) * 2;
+    u[c] = __ldcs(a);
+    w[c] = __ldcs(a + 1);
+    if (!fine) m[c] = reinterpret_cast<const double2*>(M)[(int64_t)(b0 + c) * d.nv + p];
+  }
+  if (fine) {
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+      store_block(u[c].x, u[c].y, w[c].x, w[c].y, reinterpret_cast<T*>(out.A[0]) + ((int64_t)(b0 + c) * d.nv + p) * 4);
+    return;
+  }
+  for (int j = 0; j < out.n; ++j) {
+    const double s = out.shift[j];
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+      store_block(-u[c].x, s * m[c].x - u[c].y, -w[c].x, s * m[c].y - w[c].y,
+                  reinterpret_cast<T*>(out.A[j]) + ((int64_t)(b0 + c) * d.nv + p) * 4);
+  }
+}
+
+// The inverse of the 2x2 diagonal block of A = shift*M - J per shift, from its
+// FP64 entries.
+template <typename T>
+__global__ void __launch_bounds__(256) k_pack_dinv(Dims d, bool fine, const double* __restrict__ J, const double* __restrict__ M,
+                                                   const double2* __restrict__ md, const __grid_constant__ PackOut out) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (p >= d.nv) return;
+  const int C = d.dim == 3 ? 13 : 4;
+  const double2* a = reinterpret_cast<const double2*>(J) + ((int64_t)C * d.nv + p) * 2;
+  const double2 u = a[0], w = a[1];
+  const double2 m = fine ? md[p] : reinterpret_cast<const double2*>(M)[(int64_t)C * d.nv + p];
+  for (int j = 0; j < out.n; ++j) {
+    const double a00 = -u.x, a01 = out.shift[j] * m.x - u.y, a10 = -w.x, a11 = out.shift[j] * m.y - w.y;
+    const double det = a00 * a11 - a01 * a10, r = 1.0 / det;
+    const uint32_t e = ((uint32_t)__double2hiint(det) >> 20) & 0x7ffu;
+    double q[4] = {a11, -a01, -a10, a00};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) q[t] = e - 256u < 1536u ? div_by(q[t], det, r) : q[t] / det;
+    store_block(q[0], q[1], q[2], q[3], reinterpret_cast<T*>(out.Dinv[j]) + p * 4);
+  }
+}
+
+// The finest level in FP16: per vertex and entry position one FP32 scale (the
+// largest magnitude over the block row), entries J / scale rounded to nearest,
+// blocks in the paired layout of stencil_sum_f16.  The quotients take one
+// Newton step on the product with the rounded reciprocal (Markstein's
+// correction: the correctly rounded quotient for normal operands, here |J| <=
+// scale; below 2^-900 of the FP64 range both round to the same half, zero): 3
+// FP64 operations (108 divisions per vertex took 2.9 ms at 129^3; the set-up
+// there went from 11.6 to 6.2 ms with this, k_galerkin and one pack for Dinv).
+__global__ void __launch_bounds__(128) k_pack_f16(Dims d, const double* __restrict__ J, uint4* __restrict__ A,
+                                                  float4* __restrict__ scale) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (p >= d.nv) return;
+  const int nb = d.nb;
+  const double2* q = reinterpret_cast<const double2*>(J) + p * 2;
+  const int64_t bs = d.nv * 2;
+  long long mx[4] = {0, 0, 0, 0};       // bits of the largest magnitudes (as integers: off the FP64 pipe)
+#pragma unroll 9
+  for (int b = 0; b < nb; ++b) {
+    const double2 u = q[b * bs], w = q[b * bs + 1];
+    const double e[4] = {u.x, u.y, w.x, w.y};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const long long k = __double_as_longlong(e[t]) & 0x7fffffffffffffffLL;
+      if (k > mx[t] && k <= 0x7ff0000000000000LL) mx[t] = k;    // a NaN sets no scale
     }
   }
-  if (Dinv) {
-    // diagonal block of A in FP64
-    const double* a = J + ((int64_t)C * d.nv + p) * 4;
-    double A00, A01, A10, A11;
-    if (fine) {
-      const double2 m = md[p];
-      A00 = -a[0]; A01 = shift * m.x - a[1]; A10 = -a[2]; A11 = shift * m.y - a[3];
-    } else {
-      const double* m = M + ((int64_t)C * d.nv + p) * 2;
-      A00 = -a[0]; A01 = shift * m[0] - a[1]; A10 = -a[2]; A11 = shift * m[1] - a[3];
+  // A position whose largest magnitude is below the smallest normal float
+  // holds only entries that FP32 arithmetic flushes anyway: scale 1, entries 0.
+  float sc[4];
+  double r[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const double v = __longlong_as_double(mx[t]);
+    sc[t] = v >= 1.17549435e-38 ? (float)v : 1.0f;
+    r[t] = 1.0 / (double)sc[t];
+  }
+  scale[p] = make_float4(sc[0], sc[1], sc[2], sc[3]);
+  const int slots = (nb + 1) & ~1;
+  for (int s2 = 0; s2 < slots; s2 += 2) {
+    uint4 o;
+    uint32_t hw[4];
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const int b = nb == 27 ? f16_block_of_slot(27, s2 + hh) : f16_block_of_slot(9, s2 + hh);
+      double e[4] = {0.0, 0.0, 0.0, 0.0};
+      if (b >= 0) {                       // (the empty slot stays zero)
+        const double2 u = q[b * bs], w = q[b * bs + 1];
+        e[0] = u.x; e[1] = u.y; e[2] = w.x; e[3] = w.y;
+      }
+      __half v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const double s64 = (double)sc[t], y0 = e[t] * r[t];
+        v[t] = __double2half(sc[t] < INFINITY ? fma(fma(-y0, s64, e[t]), r[t], y0) : e[t] / s64);
+      }
+      hw[2 * hh] = (uint32_t)__half_as_ushort(v[0]) | (uint32_t)__half_as_ushort(v[1]) << 16;
+      hw[2 * hh + 1] = (uint32_t)__half_as_ushort(v[2]) | (uint32_t)__half_as_ushort(v[3]) << 16;
     }
-    const double det = A00 * A11 - A01 * A10;
-    T* o = Dinv + p * 4;
-    o[0] = (T)(A11 / det); o[1] = (T)(-A01 / det); o[2] = (T)(-A10 / det); o[3] = (T)(A00 / det);
+    o.x = hw[0]; o.y = hw[1]; o.z = hw[2]; o.w = hw[3];
+    A[(int64_t)(s2 >> 1) * d.nv + p] = o;
   }
 }
 
@@ -2733,18 +2949,20 @@ void launch_coarse_mask(const Dims& df, const uint8_t* dmf, const Dims& dc, uint
   RF_LAUNCH(k_coarse_mask, (int)((dc.nv + 255) / 256), 256, 0, s, df, dmf, dc, dmc);
 }
 
-void launch_pack_level(const Dims& d, bool fine, const double* J, const double* M, const double* mdiag,
-                       double shift, int kind, void* A_out, float* scale_out, void* Dinv_out, void* s) {
-  const int g = (int)((d.nv + 127) / 128);
-  if (kind == STORE_F64)
-    RF_LAUNCH(k_pack<STORE_F64>, g, 128, 0, s, d, fine, J, M, (const double2*)mdiag, shift, A_out, scale_out,
-              (double*)Dinv_out);
-  else if (kind == STORE_F32)
-    RF_LAUNCH(k_pack<STORE_F32>, g, 128, 0, s, d, fine, J, M, (const double2*)mdiag, shift, A_out, scale_out,
-              (float*)Dinv_out);
-  else
-    RF_LAUNCH(k_pack<STORE_F16>, g, 128, 0, s, d, fine, J, M, (const double2*)mdiag, shift, A_out, scale_out,
-              (float*)Dinv_out);
+void launch_pack_level(const Dims& d, bool fine, const double* J, const double* M, const double* mdiag, int kind,
+                       PackOut out, float* scale, void* s) {
+  const unsigned g = (unsigned)((d.nv + 255) / 256);
+  const bool wide = d.nv >= 65536;
+  const dim3 gb(g, wide ? d.nb / 9 : d.nb);
+  if (!out.diag_only) {
+    if (kind == STORE_F16) RF_LAUNCH(k_pack_f16, (unsigned)((d.nv + 127) / 128), 128, 0, s, d, J, (uint4*)out.A[0], (float4*)scale);
+    else if (kind == STORE_F64 && wide) RF_LAUNCH((k_pack<double, 9>), gb, 256, 0, s, d, fine, J, M, out);
+    else if (kind == STORE_F64) RF_LAUNCH((k_pack<double, 1>), gb, 256, 0, s, d, fine, J, M, out);
+    else if (wide) RF_LAUNCH((k_pack<float, 9>), gb, 256, 0, s, d, fine, J, M, out);
+    else RF_LAUNCH((k_pack<float, 1>), gb, 256, 0, s, d, fine, J, M, out);
+  }
+  if (kind == STORE_F64) RF_LAUNCH(k_pack_dinv<double>, g, 256, 0, s, d, fine, J, M, (const double2*)mdiag, out);
+  else RF_LAUNCH(k_pack_dinv<float>, g, 256, 0, s, d, fine, J, M, (const double2*)mdiag, out);
 }
 
 void launch_dense_coarsest(const Dims& d, const Nbr& nb, const double* Jc, const double* Mc,

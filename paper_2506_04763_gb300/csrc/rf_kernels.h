@@ -128,13 +128,27 @@ cudaError_t launch_barrier_check(unsigned* bar, int rounds, int extra, double* s
                                  unsigned* passed, int* blocks_out, void* s);
 
 // set-up kernels (levelops.cu)
-void launch_galerkin_axis(int axis, const Dims& din, const uint8_t* dmf, const double* Jin, const double* Min,
-                          const double* mdiag, const Dims& dout, const uint8_t* dmc, double* Jout, double* Mout,
-                          void* s);
+// Galerkin operators Jc, Mc of coarse level c from level f's J and M (M null:
+// the finest level's mdiag), with a workspace of ws_bytes (galerkin_workspace of
+// the finest level serves every level: windows are sized to it, and a coarser
+// level's smallest window is smaller)
+constexpr size_t GAL_WS_BYTES = (size_t)512 << 20;   // its size where planes allow it
+size_t galerkin_workspace(const Dims& f);
+void launch_galerkin(const Dims& f, const uint8_t* dmf, const double* J, const double* M, const double* mdiag,
+                     const Dims& c, const uint8_t* dmc, double* Jc, double* Mc, double* ws, size_t ws_bytes, void* s);
 void launch_coarse_mask(const Dims& df, const uint8_t* dmf, const Dims& dc, uint8_t* dmc, void* s);
-// pack A = shift*M - J (coarse: from Jc/Mc; fine: keep J, only Dinv) into storage `kind`; write Dinv
-void launch_pack_level(const Dims& d, bool fine, const double* J, const double* M, const double* mdiag,
-                       double shift, int kind, void* A_out, float* scale_out, void* Dinv_out, void* s);
+// Pack a level into storage `kind`.  Coarse: A[j] = shift[j]*M - J for j < n;
+// fine: J itself into A[0] (diag_only: no entries).  Dinv[j]: the inverses of
+// the diagonal blocks of shift[j]*M - J.
+struct PackOut {
+  void* A[RF_MAXSHIFT];
+  void* Dinv[RF_MAXSHIFT];
+  double shift[RF_MAXSHIFT];
+  int n;
+  bool diag_only;
+};
+void launch_pack_level(const Dims& d, bool fine, const double* J, const double* M, const double* mdiag, int kind,
+                       PackOut out, float* scale, void* s);
 void launch_dense_coarsest(const Dims& d, const Nbr& nb, const double* Jc, const double* Mc,
                            const double* mdiag, bool fine, double shift, double* D, void* s);
 cudaError_t launch_dense_inverse(int N, double* D, double* Ainv, int* piv, double* work, int* status,
