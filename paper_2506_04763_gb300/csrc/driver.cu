@@ -93,6 +93,7 @@ struct Level {
   // stencil loads 9 blocks per memory round trip.
   int block = 128;
   bool batched = true;
+  bool small = false;
   // matrix storage of this level (STORE_*): the hierarchy's precision, except
   // that FP16 storage applies to the finest level only and the coarser levels
   // keep FP32 (their sweeps are latency-bound, and FP16 unpacking made them
@@ -100,20 +101,27 @@ struct Level {
   int kind = STORE_F64;
 };
 
-// Default kernel shape per level, from the autotuner's timings at 257^3 (one
-// sweep + one residual per candidate, GB300):
-//   FP32 storage: batched loads win everywhere — GS 2.62 -> 2.48 ms on the
-//     finest level, about 2x on levels of 65^3 and below (their time is one
-//     thread's chain of round trips), equal at 129^3; Jacobi 2.51 -> 2.27 ms
-//     on the finest level and 0.32 -> 0.29 ms at 129^3.
-//   FP64 storage: equal on the two finest levels, batched 1.2-1.6x faster on
-//     the levels below.  (On the finest level of the 65^3 FP64 LIMEX step,
-//     batched Jacobi measured no faster either.)
-//   FP16 storage (the finest level only, blocks stored in pairs): one pair
-//     per round trip, 1.80 ms per sweep + residual against 1.93 ms with two.
-static void default_shape(Level& Lv, int l, int kind) {
+// Default kernel shape per level (GB300; the autotuner may change block and
+// batched):
+//   small: at most 40000 vertices (33^3): the k_*_small kernels.  FP32 GS pair
+//     launches at 17^3 6.9 -> 4.7 us and at 33^3 8.5 -> 4.8 us, FP64 (per colour
+//     before) 33^3 2 x 17 -> 9.7 us, FP64 Jacobi at 17^3 12 -> 8 us.  At 65^3 a
+//     launch has blocks for every SM, and its bytes or FP64 operations count.
+//   FP32 storage: batched loads on every level (257^3: GS 2.62 -> 2.48 ms per
+//     sweep + residual, Jacobi 2.51 -> 2.27 ms; about 2x on levels of 65^3 and
+//     below, whose time is one thread's chain of round trips).
+//   FP64 storage: batched up to 400000 vertices with GS (a colour is 1/8 of the
+//     level) and 100000 with Jacobi; above, full occupancy hides the round trips
+//     (equal on the two finest levels of 257^3) and the FP64 pipe bounds both.
+//   FP16 storage (the finest level only, blocks stored in pairs): batched when
+//     small; else one pair per round trip (257^3: 1.80 ms per sweep + residual
+//     against 1.93 ms with two).
+static void default_shape(Level& Lv, int kind, int smoother) {
+  const int64_t nv = Lv.d.nv;
   Lv.block = 128;
-  Lv.batched = kind == STORE_F32 || (kind == STORE_F64 && l >= 2);
+  Lv.small = nv <= 40000;
+  Lv.batched = kind == STORE_F32 || (kind == STORE_F64 && nv <= (smoother == RF_SMOOTH_GS8 ? 400000 : 100000)) ||
+               (kind == STORE_F16 && Lv.small);
 }
 
 struct Alloc {
@@ -731,6 +739,7 @@ static LevelOp level_op(rf_grid* g, int l, int sh) {
   op.dmask = Lv.dmask;
   op.block = Lv.block;
   op.batched = Lv.batched;
+  op.small = Lv.small;
   return op;
 }
 
@@ -845,6 +854,94 @@ static rf_status autotune_levels(rf_grid* g, void* s) {
   return RF_OK;
 }
 
+// The parameters of a one-launch tail from level `first` for shift index j.
+static void fill_tail(rf_grid* g, int first, int j) {
+  TailParams& P = g->tail[j];
+  P = TailParams();
+  P.first = first;
+  P.coarsest = g->nl - 1;
+  P.smoother = g->gopt.smoother;
+  P.nu1 = g->gopt.nu1;
+  P.nu2 = g->gopt.nu2;
+  P.omega = g->gopt.omega;
+  fill_tail_masks(P, g->d.dim);
+  P.Ainv = g->Ainv[j];
+  P.N = (int)(2 * g->L[g->nl - 1].d.nv);
+  P.bar = g->tail_bar;
+  P.status = g->K.scal + RF_SCAL_TAIL;
+  P.limit_ns = 2000000000LL;   // 2 s: a phase takes microseconds
+  for (int l = first; l < g->nl; ++l) {
+    P.L[l].op = level_op(g, l, j);
+    P.L[l].x = g->L[l].x;
+    P.L[l].b = g->L[l].b;
+    P.L[l].r = g->L[l].r;
+    P.L[l].t = g->L[l].t;
+  }
+}
+
+// The first level of at most RF_TAIL_NV vertices and all below it run as one
+// launch: a thread-block cluster with its vectors in shared memory
+// (k_vcycle_cl), with RF_TAIL_SMEM=0 one that works in global memory, or with
+// RF_TAIL_MODE=coop a cooperative launch of every co-resident block with bounded
+// grid barriers; RF_TAIL_NV=0 launches every phase.  All compute the
+// launch-per-phase V-cycle bit for bit.  Defaults (k_vcycle_cl only; a level
+// whose vectors do not fit is left to its own launches): from 17^3, or 129 x 65,
+// down.  FP64 Jacobi, a single launch per sweep, only from 9^3 or 65 x 33: the 16
+// SMs' FP64 pipes take as long for a larger level as its launch does (17^3: 8 us).
+static long long tail_vertices(const rf_grid* g) {
+  const bool gs = g->gopt.smoother == RF_SMOOTH_GS8;
+  if (g->d.dim == 2) return gs || g->kind != STORE_F64 ? 9000 : 2500;
+  return gs || g->kind != STORE_F64 ? 6000 : 800;
+}
+
+static rf_status plan_tail(rf_grid* g, void* s) {
+  g->tail_first = -1;
+  g->tail_blocks = 0;
+  g->tail_cs = 0;
+  g->tail_bar = nullptr;   // (a hierarchy buffer: freed with the previous set-up)
+  const char* env = getenv("RF_TAIL_NV");
+  const char* mode = getenv("RF_TAIL_MODE");
+  const char* sm_env = getenv("RF_TAIL_SMEM");
+  const bool coop = mode && strcmp(mode, "coop") == 0;
+  const bool smem = !coop && !(sm_env && atoi(sm_env) == 0);
+  const long long thr = env ? atoll(env) : tail_vertices(g);
+  int first = -1;
+  if (thr > 0)
+    for (int l = 1; l < g->nl - 1 && first < 0; ++l)
+      if (g->L[l].d.nv <= thr) first = l;
+  if (first < 0) return RF_OK;
+  const int lk = g->L[first].kind;
+  if (smem) {
+    // from the first level that fits (the named one only, where the environment names it)
+    for (int l = first; l < (env ? first + 1 : g->nl - 1) && g->tail_first < 0; ++l) {
+      fill_tail(g, l, 0);
+      if (!tail_cl_plan(g->tail[0], lk, g->d.nb)) continue;
+      g->tail_first = l;
+      for (int j = 1; j < g->nshift; ++j) {
+        fill_tail(g, l, j);
+        tail_cl_plan(g->tail[j], lk, g->d.nb);
+      }
+    }
+    if (g->tail_first > 0 || !env) return RF_OK;
+  }
+  if (coop) {
+    g->tail_blocks = coop_tail_blocks(lk, g->d.nb);
+    g->tail_bar = g->tail_blocks > 0 ? (unsigned*)dalloc(g, 2 * sizeof(unsigned), s, true) : nullptr;
+    if (!g->tail_bar) {
+      g->tail_blocks = 0;
+      return RF_OK;
+    }
+    CU(cudaMemsetAsync(g->tail_bar, 0, 2 * sizeof(unsigned), (cudaStream_t)s));
+  } else {
+    g->tail_cs = tail_cluster_size(lk, g->d.nb);
+    cudaGetLastError();
+    if (g->tail_cs == 0) return RF_OK;
+  }
+  g->tail_first = first;
+  for (int j = 0; j < g->nshift; ++j) fill_tail(g, first, j);
+  return RF_OK;
+}
+
 #define GNEED(ptr)                                                                     \
   do {                                                                                 \
     if (!(ptr)) { dfree_all(g, g->gbufs, s); return fail(RF_ENOMEM, "device allocation failed (%s)", #ptr); } \
@@ -901,7 +998,7 @@ extern "C" rf_status rf_gmg_setup(rf_grid* g, const double* shifts, int nshift, 
     Level& Lv = g->L[l];
     Lv.nb = make_nbr(Lv.d);
     Lv.kind = (kind == STORE_F16 && l > 0) ? STORE_F32 : kind;
-    default_shape(Lv, l, Lv.kind);
+    default_shape(Lv, Lv.kind, o->smoother);
     const Dims& d = Lv.d;
     if (l == 0) {
       Lv.dmask = g->dir;
@@ -985,78 +1082,11 @@ extern "C" rf_status rf_gmg_setup(rf_grid* g, const double* shifts, int nshift, 
     }
   }
   if (o->autotune) {
-    rf_status ts = autotune_levels(g, s);
-    if (ts) { dfree_all(g, g->gbufs, s); return ts; }
+    rf_status as = autotune_levels(g, s);
+    if (as) { dfree_all(g, g->gbufs, s); return as; }
   }
-  // The small levels (<= RF_TAIL_NV vertices, default 6000: 17^3 and below)
-  // run as one launch: one thread-block cluster with hardware barriers, or
-  // with RF_TAIL_MODE=coop a cooperative launch of every co-resident block with
-  // bounded grid barriers; RF_TAIL_NV=0 launches every phase.  Both compute
-  // the launch-per-phase V-cycle bit for bit.  Measured on GB300 at 257^3:
-  // the cluster from 17^3 saves ~0.5 ms per solve (95.4 against 96.0 ms);
-  // from 33^3, or as a cooperative launch, the barrier-separated phases are
-  // no faster than the launches they replace, and a cluster whose first level
-  // is too large for 16 SMs (65^3) costs ~40% of an FP64 LIMEX step.
-  g->tail_first = -1;
-  g->tail_blocks = 0;
-  g->tail_bar = nullptr;   // (a hierarchy buffer: freed with the previous set-up)
-  {
-    const char* env = getenv("RF_TAIL_NV");
-    const char* mode = getenv("RF_TAIL_MODE");
-    const bool cluster = !(mode && strcmp(mode, "coop") == 0);
-    // the default applies to FP32 coarse levels: with FP64 storage the
-    // whole V-cycle in one kernel spills registers, and the 65^3 FP64 LIMEX
-    // step, its columns one after another, took 113.5 against 99.3 ms
-    const long long thr = env ? atoll(env) : (g->kind == STORE_F64 ? 0 : 6000);
-    if (thr > 0)
-      for (int l = 1; l < g->nl - 1; ++l)
-        if (g->L[l].d.nv <= thr) { g->tail_first = l; break; }
-    if (g->tail_first > 0 && cluster) {
-      g->tail_cs = tail_cluster_size(g->L[g->tail_first].kind, g->d.nb);
-      cudaGetLastError();
-      if (g->tail_cs == 0) g->tail_first = -1;
-    } else if (g->tail_first > 0) {
-      g->tail_blocks = coop_tail_blocks(g->L[g->tail_first].kind, g->d.nb);
-      g->tail_bar = g->tail_blocks > 0 ? (unsigned*)dalloc(g, 2 * sizeof(unsigned), s, true) : nullptr;
-      if (!g->tail_bar) {
-        g->tail_first = -1;
-        g->tail_blocks = 0;
-      } else {
-        CU(cudaMemsetAsync(g->tail_bar, 0, 2 * sizeof(unsigned), (cudaStream_t)s));
-      }
-    }
-    if (g->tail_first > 0)
-      for (int j = 0; j < nshift; ++j) {
-        TailParams& P = g->tail[j];
-        P = TailParams();
-        P.first = g->tail_first;
-        P.coarsest = g->nl - 1;
-        P.smoother = o->smoother;
-        P.nu1 = o->nu1;
-        P.nu2 = o->nu2;
-        P.omega = o->omega;
-        fill_tail_masks(P, g->d.dim);
-        P.Ainv = g->Ainv[j];
-        P.N = (int)(2 * g->L[g->nl - 1].d.nv);
-        P.bar = g->tail_bar;
-        P.status = g->K.scal + RF_SCAL_TAIL;
-        P.limit_ns = 2000000000LL;   // 2 s: a phase takes microseconds
-        for (int l = g->tail_first; l < g->nl; ++l) {
-          P.L[l].op = level_op(g, l, j);
-          P.L[l].x = g->L[l].x;
-          P.L[l].b = g->L[l].b;
-          P.L[l].r = g->L[l].r;
-          P.L[l].t = g->L[l].t;
-        }
-        // the cluster form with the FP32 levels' matrices in shared memory
-        // (GS smoother; RF_TAIL_SMEM=0 keeps them in global memory): when
-        // every CTA's rows fit
-        const char* sm_env = getenv("RF_TAIL_SMEM");
-        if (g->tail_blocks == 0 && g->L[g->tail_first].kind == STORE_F32 && o->smoother == RF_SMOOTH_GS8 &&
-            !(sm_env && atoi(sm_env) == 0))
-          tail_sm_plan(P, g->d.nb, g->tail_cs);
-      }
-  }
+  rf_status ts = plan_tail(g, s);
+  if (ts) { dfree_all(g, g->gbufs, s); return ts; }
   CU(cudaStreamSynchronize((cudaStream_t)s));
   CU(cudaGetLastError());
   g->gmg_ready = true;
@@ -1149,7 +1179,7 @@ static void vcycle_level(rf_grid* g, int l, int sh, const void* b, void* x, void
     }
     ProfScope ps(g, s, RF_PROF_COARSE_LEVELS, by, 1);
     if (g->tail_blocks > 0) launch_vcycle_coop(g->tail[sh], k, g->d.nb, g->tail_blocks, s);
-    else if (g->tail[sh].sm_bytes > 0) launch_vcycle_tail_sm(g->tail[sh], g->d.nb, s);
+    else if (g->tail[sh].cl_bytes > 0) launch_vcycle_cl(g->tail[sh], k, g->d.nb, s);
     else launch_vcycle_tail(g->tail[sh], k, g->d.nb, g->tail_cs, s);
     return;
   }
@@ -1903,7 +1933,6 @@ static rf_status column_grid(rf_grid* g, int j, void* s, rf_grid** out) {
     c->nshift = g->nshift;
     for (int k = 0; k < RF_MAXSHIFT; ++k) { c->shifts[k] = g->shifts[k]; c->Ainv[k] = g->Ainv[k]; }
     c->nl = g->nl;
-    c->tail_first = -1;
     const size_t te = t_size(c->kind);
     bool ok = true;
     for (int l = 0; l < RF_MAXL; ++l) {
@@ -1934,6 +1963,24 @@ static rf_status column_grid(rf_grid* g, int j, void* s, rf_grid** out) {
     }
     c->gen = g->hier_gen;
   }
+  // the parent's one-launch tail on this column's vectors (the cooperative form
+  // keeps barrier words per grid: its columns launch every phase)
+  c->tail_first = g->tail_blocks > 0 ? -1 : g->tail_first;
+  c->tail_cs = g->tail_cs;
+  c->tail_blocks = 0;
+  c->tail_bar = nullptr;
+  if (c->tail_first > 0)
+    for (int k = 0; k < c->nshift; ++k) {
+      c->tail[k] = g->tail[k];
+      c->tail[k].bar = nullptr;
+      c->tail[k].status = c->K.scal + RF_SCAL_TAIL;
+      for (int l = c->tail_first; l < c->nl; ++l) {
+        c->tail[k].L[l].x = c->L[l].x;
+        c->tail[k].L[l].b = c->L[l].b;
+        c->tail[k].L[l].r = c->L[l].r;
+        c->tail[k].L[l].t = c->L[l].t;
+      }
+    }
   *out = c;
   return RF_OK;
 }
@@ -2501,6 +2548,7 @@ extern "C" rf_status rf_limex_step_batched(rf_grid* const* grids, double* const*
     if (c) return fail(c, "problem %d: %s", i, t_err.c_str());
   }
   bool batched = true;
+  bool small = false;
   for (int i = 0; i < nprob; ++i) batched = batched && limex_batched(&o[i]);
   if (!batched) return limex_batched_threads(grids, u, H, nprob, o, infos, max_concurrent, stream);
   int workers = max_concurrent > 0 ? max_concurrent : (nprob < 16 ? nprob : 16);

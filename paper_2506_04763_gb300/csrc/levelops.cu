@@ -12,6 +12,8 @@
 //   - the coarsest level's dense LU (partial pivoting) and explicit inverse.
 // All of these are HBM-bandwidth kernels except the set-up ones.
 #include <cooperative_groups.h>
+#include <algorithm>
+#include <type_traits>
 
 #include "rf_common.cuh"
 #include "rf_kernels.h"
@@ -306,7 +308,9 @@ __device__ __forceinline__ void stencil_sum(const LevelOp& L, int64_t p, int par
 // not bandwidth, sets the time.
 // Stencil blocks (FP16: block pairs) whose loads a batched kernel issues per
 // memory round trip; an unbatched FP16 kernel loads one pair per round trip.
-__host__ __device__ constexpr int chunk_of(int kind) { return kind == STORE_F16 ? 2 : 9; }
+// Batched FP16 is for small levels, where a thread's round trips set the time:
+// seven pairs (GS at 17^3: 12.7 us a pair launch unbatched, 6.8 us so).
+__host__ __device__ constexpr int chunk_of(int kind) { return kind == STORE_F16 ? 7 : 9; }
 
 template <int KIND, int NB, int CH, bool SAME = false>
 __device__ __forceinline__ void stencil_sum_batched(const LevelOp& L, int64_t p, int par,
@@ -551,14 +555,236 @@ __global__ void __launch_bounds__(GS_PAIR_MAX_THREADS) k_gs_pair(LevelOp L, cons
   }
 }
 
+// ----------------------------------------------------------------- small FP32 levels
+// On levels that cannot fill the GPU a launch costs its chain of latencies, not
+// its bytes: the launch itself, the round trips to L2, the last block.  These
+// forms of the FP32 kernels load a row's whole stencil and D^-1 before
+// griddepcontrol.wait (matrices do not change during a solve, so this overlaps
+// the predecessor's tail), then gather b and all neighbours in one round trip.
+// 27 float4 and 27 float2 take up to 200 registers, which the few blocks of such
+// a level afford.  Same sums in the same order as the kernels above.
+template <int NB>
+struct RowF32 {
+  float4 a[NB], d;
+};
+template <int NB, bool CENTRE>
+__device__ __forceinline__ void row_load(const LevelOp& L, int64_t p, uint32_t mask, RowF32<NB>& R) {
+  const float4* A = reinterpret_cast<const float4*>(L.A) + p;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if (!CENTRE && b == (NB == 27 ? 13 : 4)) continue;
+    if (!((mask >> b) & 1u)) R.a[b] = __ldg(A + (int64_t)b * L.d.nv);
+  }
+  R.d = __ldg(reinterpret_cast<const float4*>(L.Dinv) + p);
+}
+template <int NB, bool CENTRE, bool SAME>
+__device__ __forceinline__ void row_sum(const LevelOp& L, int64_t p, int par, const float2* __restrict__ x, uint32_t mask,
+                                        const RowF32<NB>& R, float& s0, float& s1) {
+  float2 xv[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if (!CENTRE && b == (NB == 27 ? 13 : 4)) continue;
+    if (!((mask >> b) & 1u)) xv[b] = ld_xn<SAME, NB>(x + p + (par ? L.nb.off[1][b] : L.nb.off[0][b]), b);
+  }
+  float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if ((!CENTRE && b == (NB == 27 ? 13 : 4)) || ((mask >> b) & 1u)) continue;
+    a0 = blk_acc(a0, R.a[b].x, R.a[b].y, xv[b]);
+    a1 = blk_acc(a1, R.a[b].z, R.a[b].w, xv[b]);
+  }
+  s0 = a0;
+  s1 = a1;
+}
+// (A x)_p with A = shift*M - J on the finest level, as apply_row
+template <int NB, bool FINE>
+__device__ __forceinline__ void row_apply(const LevelOp& L, int64_t p, const float2* __restrict__ x, const RowF32<NB>& R,
+                                          float& s0, float& s1) {
+  const int par = (int)((uint32_t)p % (uint32_t)L.d.nx) >= L.d.E;   // nv < 2^31
+  row_sum<NB, true, false>(L, p, par, x, 0u, R, s0, s1);
+  if (FINE) {
+    const double2 m = reinterpret_cast<const double2*>(L.mdiag)[p];
+    const float xs = x[p].y, sh = (float)L.shift;
+    s0 = (sh * (float)m.x) * xs - s0;
+    s1 = (sh * (float)m.y) * xs - s1;
+  }
+}
+
+template <int NB, bool FINE>
+__global__ void __launch_bounds__(64) k_residual_small(const __grid_constant__ LevelOp L, const float2* __restrict__ b,
+                                                       const float2* __restrict__ x, float2* __restrict__ r) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  RowF32<NB> R;
+  if (p < L.d.nv) row_load<NB, true>(L, p, 0u, R);
+  rf_pdl_begin();
+  if (p >= L.d.nv) return;
+  const float2 bv = b[p];
+  float s0, s1;
+  row_apply<NB, FINE>(L, p, x, R, s0, s1);
+  r[p] = make_float2(bv.x - s0, bv.y - s1);
+}
+
+template <int NB, bool FINE>
+__global__ void __launch_bounds__(64) k_jacobi_small(const __grid_constant__ LevelOp L, const float2* __restrict__ b,
+                                                     const float2* __restrict__ xin, float2* __restrict__ xout, double omega) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  RowF32<NB> R;
+  if (p < L.d.nv) row_load<NB, true>(L, p, 0u, R);
+  rf_pdl_begin();
+  if (p >= L.d.nv) return;
+  const float2 bv = b[p], x0 = xin[p];
+  float s0, s1;
+  row_apply<NB, FINE>(L, p, xin, R, s0, s1);
+  const float r0 = bv.x - s0, r1 = bv.y - s1;
+  const float y0 = R.d.x * r0 + R.d.y * r1, y1 = R.d.z * r0 + R.d.w * r1;
+  xout[p] = make_float2(x0.x + (float)omega * y0, x0.y + (float)omega * y1);
+}
+
+template <int NB, bool FINE, int FPX>
+__global__ void __launch_bounds__(GS_PAIR_MAX_THREADS) k_gs_pair_small(const __grid_constant__ LevelOp L,
+                                                                       const float2* __restrict__ b, float2* __restrict__ x,
+                                                                       int py, int pz, int lines_y, int nlines, int lpb,
+                                                                       uint32_t skip_first, uint32_t skip_second) {
+  const int l0 = blockIdx.x * lpb, nl = min(lpb, nlines - l0), v = threadIdx.x;
+  const int cnt0 = FPX ? L.d.nx / 2 : (L.d.nx + 1) / 2, cnt1 = FPX ? (L.d.nx + 1) / 2 : L.d.nx / 2;
+  const bool on0 = v < nl * cnt0, on1 = v < nl * cnt1;
+  const int64_t p0 = on0 ? pair_vertex(L.d, l0, v, cnt0, FPX, py, pz, lines_y) : 0;
+  const int64_t p1 = on1 ? pair_vertex(L.d, l0, v, cnt1, 1 - FPX, py, pz, lines_y) : 0;
+  RowF32<NB> R;
+  if (on0) row_load<NB, false>(L, p0, skip_first, R);
+  rf_pdl_begin();
+  auto update = [&](int64_t p, float2 bv, float s0, float s1) {
+    const float r0 = FINE ? bv.x + s0 : bv.x - s0, r1 = FINE ? bv.y + s1 : bv.y - s1;   // as gs_vertex
+    x[p] = make_float2(R.d.x * r0 + R.d.y * r1, R.d.z * r0 + R.d.w * r1);
+  };
+  float s0, s1;
+  const float2 b0 = on0 ? b[p0] : make_float2(0.f, 0.f), b1 = on1 ? b[p1] : make_float2(0.f, 0.f);
+  if (on0) {
+    row_sum<NB, false, false>(L, p0, FPX, x, skip_first, R, s0, s1);
+    update(p0, b0, s0, s1);
+  }
+  if (on1) row_load<NB, false>(L, p1, skip_second, R);
+  __syncthreads();
+  if (on1) {
+    row_sum<NB, false, true>(L, p1, 1 - FPX, x, skip_second, R, s0, s1);
+    update(p1, b1, s0, s1);
+  }
+}
+
+// ----------------------------------------------------------------- small FP64 levels
+// Two neighbouring lanes per vertex, lane h its row h: a small FP64 level has
+// fewer warps than the GPU has FP64 schedulers (one warp instruction takes 64
+// cycles on each), so half the chain per thread is half the time.  As in the
+// FP32 forms the matrix rows are loaded before griddepcontrol.wait.  Same sums in
+// the same order; D^-1 and the updates as dinv_apply's callers.
+template <int NB>
+struct RowF64 {
+  double2 a[NB], d;
+};
+template <int NB, bool CENTRE>
+__device__ __forceinline__ void row_load(const LevelOp& L, int64_t p, int h, uint32_t mask, RowF64<NB>& R) {
+  const double2* A = reinterpret_cast<const double2*>(L.A) + p * 2 + h;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if (!CENTRE && b == (NB == 27 ? 13 : 4)) continue;
+    if (!((mask >> b) & 1u)) R.a[b] = __ldg(A + (int64_t)b * L.d.nv * 2);
+  }
+  R.d = __ldg(reinterpret_cast<const double2*>(L.Dinv) + p * 2 + h);
+}
+template <int NB, bool CENTRE, bool SAME>
+__device__ __forceinline__ double row_sum(const LevelOp& L, int64_t p, int par, const double2* __restrict__ x, uint32_t mask,
+                                          const RowF64<NB>& R) {
+  double s = 0.0;
+#pragma unroll
+  for (int b0 = 0; b0 < NB; b0 += 9) {
+    double2 xv[9];
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+      const int b = b0 + c;
+      if ((!CENTRE && b == (NB == 27 ? 13 : 4)) || ((mask >> b) & 1u)) continue;
+      xv[c] = ld_xn<SAME, NB>(x + p + (par ? L.nb.off[1][b] : L.nb.off[0][b]), b);
+    }
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+      const int b = b0 + c;
+      if ((!CENTRE && b == (NB == 27 ? 13 : 4)) || ((mask >> b) & 1u)) continue;
+      s = blk_acc(s, R.a[b].x, R.a[b].y, xv[c]);
+    }
+  }
+  return s;
+}
+// row h of A x at p with A = shift*M - J on the finest level, as apply_row
+template <int NB, bool FINE>
+__device__ __forceinline__ double row_apply(const LevelOp& L, int64_t p, int h, const double2* __restrict__ x, const RowF64<NB>& R) {
+  const int par = (int)((uint32_t)p % (uint32_t)L.d.nx) >= L.d.E;   // nv < 2^31
+  const double s = row_sum<NB, true, false>(L, p, par, x, 0u, R);
+  if (!FINE) return s;
+  const double m = L.mdiag[2 * p + h];
+  return (L.shift * m) * x[p].y - s;
+}
+__device__ __forceinline__ double pair_other(double v) { return __shfl_xor_sync(3u << (threadIdx.x & 30), v, 1); }
+
+template <int NB, bool FINE>
+__global__ void __launch_bounds__(64) k_residual_small64(const __grid_constant__ LevelOp L, const double2* __restrict__ b,
+                                                         const double2* __restrict__ x, double2* __restrict__ r) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, p = t >> 1;
+  const int h = (int)(t & 1);
+  RowF64<NB> R;
+  if (p < L.d.nv) row_load<NB, true>(L, p, h, 0u, R);
+  rf_pdl_begin();
+  if (p >= L.d.nv) return;
+  const double bv = reinterpret_cast<const double*>(b)[t];
+  reinterpret_cast<double*>(r)[t] = bv - row_apply<NB, FINE>(L, p, h, x, R);
+}
+
+template <int NB, bool FINE>
+__global__ void __launch_bounds__(64) k_jacobi_small64(const __grid_constant__ LevelOp L, const double2* __restrict__ b,
+                                                       const double2* __restrict__ xin, double2* __restrict__ xout, double omega) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, p = t >> 1;
+  const int h = (int)(t & 1);
+  RowF64<NB> R;
+  if (p < L.d.nv) row_load<NB, true>(L, p, h, 0u, R);
+  rf_pdl_begin();
+  if (p >= L.d.nv) return;
+  const double bv = reinterpret_cast<const double*>(b)[t], x0 = reinterpret_cast<const double*>(xin)[t];
+  const double mine = bv - row_apply<NB, FINE>(L, p, h, xin, R), other = pair_other(mine);
+  const double y = h ? R.d.x * other + R.d.y * mine : R.d.x * mine + R.d.y * other;
+  reinterpret_cast<double*>(xout)[t] = x0 + omega * y;
+}
+
+template <int NB, bool FINE, int FPX>
+__global__ void __launch_bounds__(NB == 27 ? 128 : 288) k_gs_pair_small64(const __grid_constant__ LevelOp L, const double2* __restrict__ b,
+                                                        double2* __restrict__ x, int py, int pz, int lines_y,
+                                                        uint32_t skip_first, uint32_t skip_second) {
+  // one line per block (longer runs in several rounds)
+  const int cnt0 = FPX ? L.d.nx / 2 : (L.d.nx + 1) / 2, cnt1 = FPX ? (L.d.nx + 1) / 2 : L.d.nx / 2;
+  const int h = threadIdx.x & 1;
+  auto colour = [&](auto same, int cnt, int px, uint32_t skip, bool wait) {
+    for (int v = threadIdx.x >> 1; v < cnt || wait; v += blockDim.x >> 1) {
+      const bool on = v < cnt;
+      const int64_t p = on ? pair_vertex(L.d, blockIdx.x, v, cnt, px, py, pz, lines_y) : 0;
+      RowF64<NB> R;
+      if (on) row_load<NB, false>(L, p, h, skip, R);
+      if (wait) rf_pdl_begin();
+      wait = false;
+      if (!on) break;
+      const double bv = reinterpret_cast<const double*>(b)[2 * p + h];
+      const double s = row_sum<NB, false, decltype(same)::value>(L, p, px, x, skip, R);
+      const double mine = FINE ? bv + s : bv - s, other = pair_other(mine);   // as gs_vertex
+      reinterpret_cast<double*>(x)[2 * p + h] = h ? R.d.x * other + R.d.y * mine : R.d.x * mine + R.d.y * other;
+    }
+  };
+  colour(std::false_type{}, cnt0, FPX, skip_first, true);
+  __syncthreads();
+  colour(std::true_type{}, cnt1, 1 - FPX, skip_second, false);
+}
+
 // ----------------------------------------------------------------- transfers
 template <typename T>
-__device__ __forceinline__ void restrict_point(const Dims& df, const Dims& dc, const uint8_t* __restrict__ dmf,
-                                               const uint8_t* __restrict__ dmc, const typename V2<T>::t* __restrict__ rf,
-                                               typename V2<T>::t* __restrict__ bc, int64_t pc) {
+__device__ __forceinline__ typename V2<T>::t restrict_value(const Dims& df, const Dims& dc, const uint8_t* __restrict__ dmf,
+                                                            const uint8_t* __restrict__ dmc,
+                                                            const typename V2<T>::t* rf, int64_t pc, int I, int J, int K) {
   typedef typename V2<T>::t V;
-  int I, J, K;
-  pcoords(dc, pc, I, J, K);
   const bool mc = dmc[pc] != 0;
   // all 3^d fine values and masks are loaded first (one memory round trip),
   // then summed in the fixed (dz, dy, dx) order
@@ -592,7 +818,16 @@ __device__ __forceinline__ void restrict_point(const Dims& df, const Dims& dc, c
   V o;
   o.x = s0;
   o.y = s1;
-  bc[pc] = o;
+  return o;
+}
+
+template <typename T>
+__device__ __forceinline__ void restrict_point(const Dims& df, const Dims& dc, const uint8_t* __restrict__ dmf,
+                                               const uint8_t* __restrict__ dmc, const typename V2<T>::t* __restrict__ rf,
+                                               typename V2<T>::t* __restrict__ bc, int64_t pc) {
+  int I, J, K;
+  pcoords(dc, pc, I, J, K);
+  bc[pc] = restrict_value<T>(df, dc, dmf, dmc, rf, pc, I, J, K);
 }
 
 template <typename T>
@@ -606,13 +841,12 @@ __global__ void __launch_bounds__(256) k_restrict(Dims df, Dims dc, const uint8_
   restrict_point<T>(df, dc, dmf, dmc, rf, bc, pc);
 }
 
-template <typename T>
-__device__ __forceinline__ void prolong_point(const Dims& df, const Dims& dc, const uint8_t* __restrict__ dmf,
-                                              const uint8_t* __restrict__ dmc, const typename V2<T>::t* __restrict__ xc,
-                                              typename V2<T>::t* __restrict__ xf, int64_t pf) {
+// the corrected fine value x_f + (P x_c)
+template <typename T, typename XC>
+__device__ __forceinline__ typename V2<T>::t prolong_value(const Dims& df, const Dims& dc, const uint8_t* __restrict__ dmf,
+                                                           const uint8_t* __restrict__ dmc, XC xc,
+                                                           const typename V2<T>::t* xf, int64_t pf, int fi, int fj, int fk) {
   typedef typename V2<T>::t V;
-  int fi, fj, fk;
-  pcoords(df, pf, fi, fj, fk);
   const bool mf = dmf[pf] != 0;
   // the (up to) 2^d coarse parents, loaded first, summed in (K, J, I) order
   V c[8];
@@ -625,7 +859,7 @@ __device__ __forceinline__ void prolong_point(const Dims& df, const Dims& dc, co
             (((q >> 2) & 1) == 0 || (fk & 1)) && K < dc.nz && J < dc.ny && I < dc.nx;
     if (in[q]) {
       const int64_t pc = pidx(dc, I, J, K);
-      c[q] = xc[pc];
+      c[q] = xc((int)pc);
       m[q] = dmc[pc];
     } else {
       c[q].x = 0;
@@ -646,7 +880,16 @@ __device__ __forceinline__ void prolong_point(const Dims& df, const Dims& dc, co
   V o = xf[pf];
   o.x += s0;
   o.y += s1;
-  xf[pf] = o;
+  return o;
+}
+
+template <typename T>
+__device__ __forceinline__ void prolong_point(const Dims& df, const Dims& dc, const uint8_t* __restrict__ dmf,
+                                              const uint8_t* __restrict__ dmc, const typename V2<T>::t* __restrict__ xc,
+                                              typename V2<T>::t* __restrict__ xf, int64_t pf) {
+  int fi, fj, fk;
+  pcoords(df, pf, fi, fj, fk);
+  xf[pf] = prolong_value<T>(df, dc, dmf, dmc, [&](int pc) { return xc[pc]; }, xf, pf, fi, fj, fk);
 }
 
 template <typename T>
@@ -906,44 +1149,10 @@ __device__ __forceinline__ bool grid_sync_bounded(unsigned* bar, unsigned expect
   return s_ok != 0;
 }
 
-// Shared-memory rows of the tail (k_vcycle_tail_sm, FP32 levels).  A row's
-// stencil sum takes its blocks from shared memory (sA: block b of local row
-// lr at sA[b * rows + lr]) and gathers all its x values first, then sums the
-// blocks in stencil order with blk_acc: the values of stencil_sum_batched.
-// x is read with ordinary (coherent) loads: other CTAs of the cluster wrote it
-// in earlier phases.
-template <int NB>
-__device__ __forceinline__ void sm_row_sum(const LevelOp& L, const float4* __restrict__ sA, int rows, int lr,
-                                           int64_t p, int par, const float2* x, bool skip_centre,
-                                           uint32_t skipmask, float& s0, float& s1) {
-  constexpr int C = NB == 27 ? 13 : 4;
-  float2 xv[NB];
-#pragma unroll
-  for (int b = 0; b < NB; ++b)
-    if (!((skip_centre && b == C) || ((skipmask >> b) & 1u))) xv[b] = x[p + (par ? L.nb.off[1][b] : L.nb.off[0][b])];
-  float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    if ((skip_centre && b == C) || ((skipmask >> b) & 1u)) continue;
-    const float4 a = sA[b * rows + lr];
-    a0 = blk_acc(a0, a.x, a.y, xv[b]);
-    a1 = blk_acc(a1, a.z, a.w, xv[b]);
-  }
-  s0 = a0;
-  s1 = a1;
-}
-
-// The line owned as item i by CTA `rank` of a cluster of cs CTAs.
-__device__ __forceinline__ int sm_line(int rank, int cs, int i) { return rank + cs * i; }
-
 // The V-cycle below level P.first; sync() separates phases and returns false
-// when the launch must end (coop: a barrier gave up).  SM: the shared-memory
-// form (FP32 levels, GS smoother; sm holds this CTA's rows, rank is its rank
-// in the cluster), whose GS and residual phases update the vertices of the
-// CTA's own x-lines.
-template <int KIND, int NB, bool SM = false, typename Sync>
-__device__ __forceinline__ void vcycle_tail_body(const TailParams& P, int64_t gt, int64_t nthr, Sync&& sync,
-                                                 const float4* sm = nullptr, int rank = 0) {
+// when the launch must end (coop: a barrier gave up).
+template <int KIND, int NB, typename Sync>
+__device__ __forceinline__ void vcycle_tail_body(const TailParams& P, int64_t gt, int64_t nthr, Sync&& sync) {
   typedef typename Ty<KIND>::T T;
   typedef typename V2<T>::t V;
   // batched stencil loads (a thread's round trips set a phase's time); FP64
@@ -951,47 +1160,6 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams& P, int64_t gt
   constexpr int CH = KIND == STORE_F64 ? 3 : chunk_of(KIND);
   const int ncol = 1 << P.L[P.first].op.d.dim;
   V* curs[RF_MAXL];
-  auto gs_sweep_sm = [&](int l, const LevelOp& op, const V* b, V* x, bool forward, bool zero_start) {
-    const int nx = op.d.nx, ny = op.d.ny, nlines = op.d.ny * (op.d.dim == 3 ? op.d.nz : 1);
-    const int rows = P.sm_rows[l];
-    const float4* sA = sm + P.sm_base[l];
-    const float* sD = reinterpret_cast<const float*>(sA + NB * rows);
-    // colour pairs (c, c ^ 1), as in k_gs_pair: the CTA owns whole x-lines,
-    // so the pair's second colour waits only for a block barrier and reads
-    // its same-line neighbours after it (plain loads); one cluster barrier
-    // per pair
-    for (int cc = 0; cc < ncol; cc += 2) {
-      const int c1 = forward ? cc : ncol - 1 - cc;
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        const int col = h ? (c1 ^ 1) : c1;
-        const int px = col & 1, py = (col >> 1) & 1, pz = (col >> 2) & 1;
-        const int cnt = px ? nx / 2 : (nx + 1) / 2;
-        const uint32_t skip = (zero_start && forward) ? P.zmask[col] : 0u;
-        const int items = P.sm_lines[l] * cnt;
-        for (int t = threadIdx.x; t < items; t += blockDim.x) {
-          const int i = t / cnt, pos = t - i * cnt;
-          const int Ln = sm_line(rank, P.sm_cs, i);
-          if (Ln >= nlines) continue;
-          const int k = Ln / ny, j = Ln - k * ny;
-          if ((j & 1) != py || (k & 1) != pz) continue;
-          const int u = (px ? op.d.E : 0) + pos;
-          const int64_t p = (int64_t)Ln * nx + u;
-          const int lr = i * nx + u;
-          const float2 bv = ((const float2*)b)[p];
-          float s0, s1;
-          sm_row_sum<NB>(op, sA, rows, lr, p, px, (const float2*)x, true, skip, s0, s1);
-          const float r0 = bv.x - s0, r1 = bv.y - s1;   // coarse level: A_pq as stored
-          float y0, y1;
-          dinv_apply<float>(sD, lr, r0, r1, y0, y1);
-          ((float2*)x)[p] = make_float2(y0, y1);
-        }
-        if (h == 0) __syncthreads();
-      }
-      if (!sync()) return false;
-    }
-    return true;
-  };
   auto gs_sweep = [&](const LevelOp& op, const V* b, V* x, bool forward, bool zero_start) {
     for (int cc = 0; cc < ncol; ++cc) {
       const int col = forward ? cc : ncol - 1 - cc;
@@ -1018,13 +1186,8 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams& P, int64_t gt
     V* tmp = (V*)Lv.t;
     V* cur = x;
     if (P.smoother == 1) {
-      for (int sw = 0; sw < P.nu1; ++sw) {
-        if constexpr (SM) {
-          if (!gs_sweep_sm(l, Lv.op, b, x, true, sw == 0)) return;
-        } else {
-          if (!gs_sweep(Lv.op, b, x, true, sw == 0)) return;
-        }
-      }
+      for (int sw = 0; sw < P.nu1; ++sw)
+        if (!gs_sweep(Lv.op, b, x, true, sw == 0)) return;
     } else {
       V* first = ((P.nu1 + P.nu2) & 1) ? x : tmp;
       if (!jacobi_sweep(Lv.op, b, nullptr, first, true)) return;
@@ -1036,23 +1199,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams& P, int64_t gt
       }
     }
     curs[l] = cur;
-    if constexpr (SM) {
-      const int nx = Lv.op.d.nx, nlines = Lv.op.d.ny * (Lv.op.d.dim == 3 ? Lv.op.d.nz : 1);
-      const int rows = P.sm_rows[l];
-      const float4* sA = sm + P.sm_base[l];
-      for (int t = threadIdx.x; t < rows; t += blockDim.x) {
-        const int i = t / nx, u = t - i * nx;
-        const int Ln = sm_line(rank, P.sm_cs, i);
-        if (Ln >= nlines) continue;
-        const int64_t p = (int64_t)Ln * nx + u;
-        const float2 bv = ((const float2*)b)[p];
-        float s0, s1;
-        sm_row_sum<NB>(Lv.op, sA, rows, t, p, u >= Lv.op.d.E, (const float2*)cur, false, 0u, s0, s1);
-        ((float2*)Lv.r)[p] = make_float2(bv.x - s0, bv.y - s1);
-      }
-    } else {
-      for (int64_t p = gt; p < Lv.op.d.nv; p += nthr) residual_point<KIND, false, NB, CH>(Lv.op, b, cur, (V*)Lv.r, p);
-    }
+    for (int64_t p = gt; p < Lv.op.d.nv; p += nthr) residual_point<KIND, false, NB, CH>(Lv.op, b, cur, (V*)Lv.r, p);
     if (!sync()) return;
     for (int64_t p = gt; p < Lc.op.d.nv; p += nthr)
       restrict_point<T>(Lv.op.d, Lc.op.d, Lv.op.dmask, Lc.op.dmask, (const V*)Lv.r, (V*)Lc.b, p);
@@ -1087,13 +1234,8 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams& P, int64_t gt
       prolong_point<T>(Lv.op.d, Lc.op.d, Lv.op.dmask, Lc.op.dmask, (const V*)Lc.x, cur, p);
     if (!sync()) return;
     if (P.smoother == 1) {
-      for (int sw = 0; sw < P.nu2; ++sw) {
-        if constexpr (SM) {
-          if (!gs_sweep_sm(l, Lv.op, b, x, false, false)) return;
-        } else {
-          if (!gs_sweep(Lv.op, b, x, false, false)) return;
-        }
-      }
+      for (int sw = 0; sw < P.nu2; ++sw)
+        if (!gs_sweep(Lv.op, b, x, false, false)) return;
     } else {
       for (int sw = 0; sw < P.nu2; ++sw) {
         V* dst = (cur == x) ? tmp : x;
@@ -1115,49 +1257,373 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_vcycle_tail(const __grid_const
   });
 }
 
-// The tail with the levels' matrices in shared memory: each CTA of the
-// cluster first copies the stencil blocks and D^-1 of its own x-lines
-// (cp.async, 16 bytes per copy; the matrices are not written during the
-// launch), then runs the V-cycle.  Its GS colour phases read no matrix data
-// from L2 or HBM, only the x values around each vertex.
+// The cluster tail with its vectors in shared memory.  Every CTA of the cluster
+// keeps a copy of x (Jacobi: of both iterates) of every tail level, zero halo
+// included, and owns the x-lines rank + cs * i of each level: it computes their
+// values and stores each into the copies of the CTAs that own a neighbouring line
+// (distributed shared memory), so a phase reads x and b from its own shared
+// memory and costs one cluster barrier.
+// The blocks and D^-1 of the own lines are copied to shared memory too (cp.async,
+// before the predecessor's results are waited for), the smallest levels first
+// as far as they fit; other levels stream them from L2.  GS sweeps colour
+// pairs as k_gs_pair does (all kinds: here the pair saves a barrier): the pair's
+// second colour reaches the first only on its own line, so a block barrier
+// lies between them.  r crosses through global memory (one phase per level).
+// Sums, order and operations per vertex are those of the launch-per-phase
+// kernels, bit for bit.  Bound by latency: at 17^3 and below a pair phase is two
+// chains of 26 blocks from shared memory (0.3 us each), 5 remote stores and the
+// barrier (0.4 us).  With x read through L2 the V-cycle from 17^3 down took 180 us
+// (FP32 GS), now 100; FP64 GS, then 32 launches a level, 33^3 solve's coarse part
+// 690 -> 270 us a V-cycle, 2D from 129 x 65 down 430 -> 230 us.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-template <int NB>
-__global__ void __launch_bounds__(TAIL_THREADS) k_vcycle_tail_sm(const __grid_constant__ TailParams P) {
-  extern __shared__ float4 tail_sm[];
+// What a CTA of k_vcycle_cl needs of one level, read from the parameters once
+// per level and sweep: indexed reads of them in the row loops (a neighbour
+// table, say) cost more than the sums.
+struct ClLevel {
+  int nx, ny, pl, E, xl0, xr0, xl1, xr1;   // pl = nx ny; x offsets of dx = -1, +1 for even and odd vertices
+  int rows, lines, nlines;
+  float inv_nx;
+  uint32_t peers;                          // CTAs that own a line next to one of this CTA's, this one included
+  int64_t nv;
+  const void* A;
+  const void* Dinv;
+  const float4* sA;
+};
+
+// a / d for 0 <= a < 2^20 with inv = 1.0f / d: the quotient's distance to the
+// next whole number, at least 1 / (2 d), is beyond the rounding of the product
+__device__ __forceinline__ int cl_div(int a, float inv) { return (int)(((float)a + 0.5f) * inv); }
+
+// Residual b - (stencil sum) of local row lr = vertex p, x and b in shared memory,
+// the blocks there or (L.sA null) in global memory, CH at a time: their loads
+// first (MASKED: blocks of skipmask left out; a sweep that skips none keeps
+// its loads free of branches), then the sums in stencil order.  FP64: a pair of
+// neighbouring lanes shares a vertex, lane h sums its row h (an SM's FP64 pipe
+// takes 64 cycles per warp instruction on each of its four schedulers, and a
+// cluster's few rows leave most of them idle); both get both residuals.
+template <int KIND, int NB, bool CENTRE, bool MASKED>
+__device__ __forceinline__ void cl_residual(const ClLevel& L, int lr, int p, int par, int h,
+                                            const typename V2<typename Ty<KIND>::T>::t* x,
+                                            const typename V2<typename Ty<KIND>::T>::t bv, uint32_t skipmask,
+                                            typename Ty<KIND>::T& r0, typename Ty<KIND>::T& r1) {
+  typedef typename Ty<KIND>::T T;
+  constexpr int C = NB == 27 ? 13 : 4;
+  const int xl = par ? L.xl1 : L.xl0, xr = par ? L.xr1 : L.xr0;
+  auto xat = [&](int b) {
+    const int dx = b % 3 - 1, dy = (b / 3) % 3 - 1, dz = b / 9 - (NB == 27 ? 1 : 0);
+    return x[p + (dx < 0 ? xl : dx > 0 ? xr : 0) + dy * L.nx + dz * L.pl];
+  };
+  auto skipped = [&](int b) { return (!CENTRE && b == C) || (MASKED && ((skipmask >> b) & 1u)); };
+  if constexpr (KIND == STORE_F64) {
+    const double2* sm = reinterpret_cast<const double2*>(L.sA) + h * L.rows + lr;
+    const double2* gm = reinterpret_cast<const double2*>(L.A) + (int64_t)p * 2 + h;
+    double a0 = 0.0;
+    auto sum = [&](auto shared) {
+      constexpr int CH = decltype(shared)::value ? 3 : 9;
+#pragma unroll
+      for (int b0 = 0; b0 < NB; b0 += CH) {
+        double2 a[CH], xv[CH];
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (!skipped(b0 + c)) a[c] = decltype(shared)::value ? sm[2 * (b0 + c) * L.rows] : __ldg(gm + (int64_t)(b0 + c) * L.nv * 2);
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (!skipped(b0 + c)) xv[c] = xat(b0 + c);
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (!skipped(b0 + c)) a0 = blk_acc(a0, a[c].x, a[c].y, xv[c]);
+      }
+    };
+    if (L.sA) sum(std::true_type{});
+    else sum(std::false_type{});
+    const double mine = (h ? bv.y : bv.x) - a0;
+    const double other = __shfl_xor_sync(3u << (threadIdx.x & 30), mine, 1);
+    r0 = h ? other : mine;
+    r1 = h ? mine : other;
+  } else {
+    T a0 = 0, a1 = 0;
+    auto sum = [&](auto shared) {
+      constexpr int CH = 9;
+#pragma unroll
+      for (int b0 = 0; b0 < NB; b0 += CH) {
+        float4 a[CH];
+        float2 xv[CH];
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (!skipped(b0 + c))
+            a[c] = decltype(shared)::value ? L.sA[(b0 + c) * L.rows + lr]
+                                           : __ldg(reinterpret_cast<const float4*>(L.A) + (int64_t)(b0 + c) * L.nv + p);
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (!skipped(b0 + c)) xv[c] = xat(b0 + c);
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (!skipped(b0 + c)) {
+            a0 = blk_acc(a0, a[c].x, a[c].y, xv[c]);
+            a1 = blk_acc(a1, a[c].z, a[c].w, xv[c]);
+          }
+      }
+    };
+    if (L.sA) sum(std::true_type{});
+    else sum(std::false_type{});
+    r0 = bv.x - a0;
+    r1 = bv.y - a1;
+  }
+}
+
+template <int KIND, int NB>
+__global__ void __launch_bounds__(TAIL_THREADS, 1) k_vcycle_cl(const __grid_constant__ TailParams P) {
+  typedef typename Ty<KIND>::T T;
+  typedef typename V2<T>::t V;
+  constexpr int PARTS = KIND == STORE_F64 ? 2 : 1;   // 16-byte parts of a block
+  constexpr int RS = PARTS;                          // threads per vertex
+  extern __shared__ __align__(16) unsigned char cl_raw[];
   cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank();
-  for (int l = P.first; l < P.coarsest; ++l) {
+  const int rank = (int)cl.block_rank(), cs = P.cl_cs, tid = threadIdx.x, nt = blockDim.x;
+  auto xbuf = [&](int l) { return reinterpret_cast<V*>(cl_raw + P.cl_x[l]); };   // interior (after the halo)
+  auto tbuf = [&](int l) { return reinterpret_cast<V*>(cl_raw + P.cl_t[l]); };
+  auto bbuf = [&](int l) { return reinterpret_cast<V*>(cl_raw + P.cl_b[l]); };   // own rows (coarsest: all)
+  // the own lines of level l by (y, z) parity: their counts, then their numbers
+  auto list = [&](int l, int cls) { return reinterpret_cast<int*>(cl_raw + P.cl_list[l]) + 4 + cls * (P.cl_rows[l] / P.L[l].op.d.nx); };
+  auto count = [&](int l, int cls) { return reinterpret_cast<int*>(cl_raw + P.cl_list[l])[cls]; };
+  auto level = [&](int l) {
     const LevelOp& op = P.L[l].op;
-    const int nx = op.d.nx, nlines = op.d.ny * (op.d.dim == 3 ? op.d.nz : 1);
-    const int rows = P.sm_rows[l], items = (NB + 1) * rows;
-    float4* dst = tail_sm + P.sm_base[l];
-    const float4* A = reinterpret_cast<const float4*>(op.A);
-    const float4* D = reinterpret_cast<const float4*>(op.Dinv);
-    for (int t = threadIdx.x; t < items; t += blockDim.x) {
-      const int b = t / rows, lr = t - b * rows;
-      const int i = lr / nx, u = lr - i * nx;
-      const int Ln = sm_line(rank, P.sm_cs, i);
-      if (Ln >= nlines) continue;
-      const int64_t p = (int64_t)Ln * nx + u;
-      cp_async16(dst + t, b < NB ? A + (int64_t)b * op.d.nv + p : D + p);
+    ClLevel L;
+    L.nx = op.d.nx; L.ny = op.d.ny; L.E = op.d.E; L.pl = NB == 27 ? op.d.nx * op.d.ny : 0;
+    L.xl0 = L.E - 1; L.xr0 = L.E; L.xl1 = -L.E; L.xr1 = 1 - L.E;
+    L.rows = P.cl_rows[l];
+    L.inv_nx = 1.0f / (float)L.nx;
+    L.lines = cl_div(L.rows, L.inv_nx);
+    L.nlines = op.d.ny * (NB == 27 ? op.d.nz : 1);
+    L.nv = op.d.nv;
+    L.A = op.A;
+    L.Dinv = op.Dinv;
+    L.sA = P.cl_a[l] >= 0 ? reinterpret_cast<const float4*>(cl_raw + P.cl_a[l]) : nullptr;
+    // line Ln = rank + cs * i, so its neighbours' owners are the same for every own line
+    L.peers = 0;
+#pragma unroll
+    for (int c = -1; c <= 1; ++c) {
+      const int o = rank + (NB == 27 ? c * L.ny : 0);
+      L.peers |= 1u << ((o - 1) & (cs - 1)) | 1u << (o & (cs - 1)) | 1u << ((o + 1) & (cs - 1));
+    }
+    return L;
+  };
+  auto put = [&](uint32_t peers, auto* dst, auto v) {   // into the copies of these CTAs
+    for (uint32_t m = peers; m; m &= m - 1) *cl.map_shared_rank(dst, __ffs(m) - 1) = v;
+  };
+  const uint32_t everyone = cs == 32 ? ~0u : (1u << cs) - 1;
+  // zeros in every vector (reads of neighbours outside the grid, and of colours
+  // not yet visited, must meet finite values), the matrices, the line lists
+  for (int t = tid; t < P.cl_vec_bytes / 16; t += nt) reinterpret_cast<float4*>(cl_raw)[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
+  for (int l = P.first; l < P.coarsest; ++l) {
+    const ClLevel L = level(l);
+    if (L.sA) {
+      float4* dst = const_cast<float4*>(L.sA);
+      const float4* A = reinterpret_cast<const float4*>(L.A);
+      const float4* D = reinterpret_cast<const float4*>(L.Dinv);
+      for (int lr = tid; lr < L.rows; lr += nt) {
+        const int i = cl_div(lr, L.inv_nx), Ln = rank + cs * i, p = Ln * L.nx + (lr - i * L.nx);
+        if (Ln >= L.nlines) continue;
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+          for (int h = 0; h < PARTS; ++h) cp_async16(dst + (b * PARTS + h) * L.rows + lr, A + ((int64_t)b * L.nv + p) * PARTS + h);
+#pragma unroll
+        for (int h = 0; h < PARTS; ++h) cp_async16(dst + (NB * PARTS + h) * L.rows + lr, D + (int64_t)p * PARTS + h);
+      }
+    }
+    if (tid < 4) {
+      int n = 0;
+      for (int i = 0; i < L.lines; ++i) {
+        const int Ln = rank + cs * i;
+        if (Ln >= L.nlines) break;
+        const int k = Ln / L.ny, j = Ln - k * L.ny;
+        if (((j & 1) | (k & 1) << 1) == tid) list(l, tid)[n++] = i;
+      }
+      reinterpret_cast<int*>(cl_raw + P.cl_list[l])[tid] = n;
+    }
+  }
+  __syncthreads();
+  rf_pdl_begin();
+  {
+    const ClLevel L = level(P.first);
+    const V* b = (const V*)P.L[P.first].b;
+    V* sb = bbuf(P.first);
+    for (int lr = tid; lr < L.rows; lr += nt) {
+      const int i = cl_div(lr, L.inv_nx), Ln = rank + cs * i;
+      if (Ln < L.nlines) sb[lr] = b[Ln * L.nx + (lr - i * L.nx)];
     }
   }
   cp_async_wait_all();
-  __syncthreads();
-  const int64_t nthr = (int64_t)cl.num_blocks() * blockDim.x;
-  const int64_t gt = (int64_t)rank * blockDim.x + threadIdx.x;
-  vcycle_tail_body<STORE_F32, NB, true>(
-      P, gt, nthr,
-      [&]() {
-        cl.sync();
-        return true;
-      },
-      tail_sm, rank);
+  cl.sync();               // every CTA's vectors are zero before a peer writes into them
+
+  // D^-1 r of a row (FP64: the component of row h), then out = x + w D^-1 r (w = 0:
+  // out = D^-1 r) into the peers' copies
+  auto update = [&](const ClLevel& L, int lr, int p, int h, T r0, T r1, V* out, bool add, V xv, T w) {
+    if constexpr (KIND == STORE_F64) {
+      const double2 D = L.sA ? reinterpret_cast<const double2*>(L.sA)[(2 * NB + h) * L.rows + lr]
+                             : __ldg(reinterpret_cast<const double2*>(L.Dinv) + (int64_t)p * 2 + h);
+      const T y = D.x * r0 + D.y * r1;
+      put(L.peers, reinterpret_cast<T*>(out + p) + h, add ? (h ? xv.y : xv.x) + w * y : y);
+    } else {
+      const float4 D = L.sA ? L.sA[NB * L.rows + lr] : __ldg(reinterpret_cast<const float4*>(L.Dinv) + p);
+      const T y0 = D.x * r0 + D.y * r1, y1 = D.z * r0 + D.w * r1;
+      V o;
+      o.x = add ? xv.x + w * y0 : y0;
+      o.y = add ? xv.y + w * y1 : y1;
+      put(L.peers, out + p, o);
+    }
+  };
+  auto gs_sweep = [&](int l, V* x, bool forward, bool zero_start) {
+    const ClLevel L = level(l);
+    const V* sb = bbuf(l);
+    const int ncol = NB == 27 ? 8 : 4;
+    const float inv_e = 1.0f / (float)L.E, inv_o = 1.0f / (float)(L.nx - L.E);
+    V none;
+    none.x = 0;
+    none.y = 0;
+#pragma unroll 1
+    for (int cc = 0; cc < ncol; cc += 2) {
+      const int c1 = forward ? cc : ncol - 1 - cc, cls = c1 >> 1, nln = count(l, cls);
+      const int* ln = list(l, cls);
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        const int col = half ? (c1 ^ 1) : c1, px = col & 1;
+        const int cnt = px ? L.nx - L.E : L.E;
+        const float inv = px ? inv_o : inv_e;
+        const uint32_t skip = (zero_start && forward) ? P.zmask[col] : 0u;
+        for (int t = tid; t < nln * cnt * RS; t += nt) {
+          const int it = t / RS, h = t % RS, li = cl_div(it, inv), i = ln[li], u = (px ? L.E : 0) + it - li * cnt;
+          const int p = (rank + cs * i) * L.nx + u, lr = i * L.nx + u;
+          T r0, r1;
+          if (skip) cl_residual<KIND, NB, false, true>(L, lr, p, px, h, x, sb[lr], skip, r0, r1);   // coarse level: A_pq as stored
+          else cl_residual<KIND, NB, false, false>(L, lr, p, px, h, x, sb[lr], 0u, r0, r1);
+          update(L, lr, p, h, r0, r1, x, false, none, (T)0);
+        }
+        if (half == 0) __syncthreads();
+      }
+      cl.sync();
+    }
+  };
+  auto jacobi_sweep = [&](int l, const V* xin, V* xout, bool zero_x) {
+    const ClLevel L = level(l);
+    const V* sb = bbuf(l);
+    for (int t = tid; t < L.rows * RS; t += nt) {
+      const int lr = t / RS, h = t % RS, i = cl_div(lr, L.inv_nx), Ln = rank + cs * i, u = lr - i * L.nx, p = Ln * L.nx + u;
+      if (Ln >= L.nlines) continue;
+      T r0 = sb[lr].x, r1 = sb[lr].y;
+      V x0;
+      x0.x = 0;
+      x0.y = 0;
+      if (!zero_x) {
+        cl_residual<KIND, NB, true, false>(L, lr, p, u >= L.E, h, xin, sb[lr], 0u, r0, r1);
+        x0 = xin[p];
+      }
+      update(L, lr, p, h, r0, r1, xout, true, x0, (T)P.omega);
+    }
+    cl.sync();
+  };
+
+  const bool gs = P.smoother == 1;
+  const bool first_x = ((P.nu1 + P.nu2) & 1) != 0;   // Jacobi: which buffer the first sweep fills
+  // one place for each direction's sweeps (the kernel holds them once)
+  auto sweeps = [&](int l, V* cur, int n, bool forward, bool zero_start) {
+#pragma unroll 1
+    for (int sw = 0; sw < n; ++sw) {
+      if (gs) {
+        gs_sweep(l, cur, forward, zero_start && sw == 0);
+      } else {
+        const bool zero = zero_start && sw == 0;
+        V* dst = zero ? cur : cur == xbuf(l) ? tbuf(l) : xbuf(l);
+        jacobi_sweep(l, cur, dst, zero);
+        cur = dst;
+      }
+    }
+    return cur;
+  };
+#pragma unroll 1
+  for (int l = P.first; l < P.coarsest; ++l) {
+    V* cur = sweeps(l, gs || first_x ? xbuf(l) : tbuf(l), P.nu1, true, true);
+    const ClLevel L = level(l);
+    const LevelOp& op = P.L[l].op;
+    const V* sb = bbuf(l);
+    V* r = (V*)P.L[l].r;
+    for (int t = tid; t < L.rows * RS; t += nt) {
+      const int lr = t / RS, h = t % RS, i = cl_div(lr, L.inv_nx), Ln = rank + cs * i, u = lr - i * L.nx, p = Ln * L.nx + u;
+      if (Ln >= L.nlines) continue;
+      V o;
+      cl_residual<KIND, NB, true, false>(L, lr, p, u >= L.E, h, cur, sb[lr], 0u, o.x, o.y);
+      if (h == 0) r[p] = o;
+    }
+    cl.sync();
+    const LevelOp& oc = P.L[l + 1].op;
+    const bool last = l + 1 == P.coarsest;
+    V* bc = bbuf(l + 1);
+    const int nxc = oc.d.nx, n = last ? (int)oc.d.nv : P.cl_rows[l + 1];
+    const float inv = 1.0f / (float)nxc;
+    for (int t = last ? rank * nt + tid : tid; t < n; t += last ? cs * nt : nt) {
+      // the coarsest level's b goes to everyone, another level's own rows stay
+      const int q = cl_div(t, inv), Ln = last ? q : rank + cs * q, u = t - q * nxc;
+      const int K = NB == 27 ? Ln / oc.d.ny : 0, J = Ln - K * oc.d.ny, I = u < oc.d.E ? 2 * u : 2 * (u - oc.d.E) + 1;
+      if (NB == 27 ? K >= oc.d.nz : J >= oc.d.ny) continue;
+      const V o = restrict_value<T>(op.d, oc.d, op.dmask, oc.dmask, r, Ln * nxc + u, I, J, K);
+      if (last) put(everyone, bc + t, o);
+      else bc[t] = o;
+    }
+    if (last) cl.sync();
+    else __syncthreads();
+  }
+  {
+    // x = A^-1 b on the coarsest level: one warp per row, the xor-shuffle sum of coarse_solve_body
+    const T* bc = reinterpret_cast<const T*>(bbuf(P.coarsest));
+    T* xc = reinterpret_cast<T*>(xbuf(P.coarsest));
+    const int lane = tid & 31;
+    for (int r = rank * (nt >> 5) + (tid >> 5); r < P.N; r += cs * (nt >> 5)) {
+      const double* row = P.Ainv + (int64_t)r * P.N;
+      double s = 0.0;
+      for (int c = lane; c < P.N; c += 32) s += row[c] * (double)bc[c];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane < cs) *cl.map_shared_rank(xc + r, lane) = (T)s;
+    }
+    cl.sync();
+  }
+  // where a level's iterate lies after n sweeps
+  auto after = [&](int l, int n) { return gs || first_x == ((n & 1) != 0) ? xbuf(l) : tbuf(l); };
+#pragma unroll 1
+  for (int l = P.coarsest - 1; l >= P.first; --l) {
+    const ClLevel L = level(l);
+    const LevelOp& op = P.L[l].op;
+    const LevelOp& oc = P.L[l + 1].op;
+    V* cur = after(l, P.nu1);
+    const bool last = l + 1 == P.coarsest;
+    const V* xc = last ? xbuf(l + 1) : after(l + 1, P.nu1 + P.nu2);
+    const float inv_nxc = 1.0f / (float)oc.d.nx;
+    for (int lr = tid; lr < L.rows; lr += nt) {
+      const int i = cl_div(lr, L.inv_nx), Ln = rank + cs * i, u = lr - i * L.nx;
+      if (Ln >= L.nlines) continue;
+      const int k = NB == 27 ? Ln / L.ny : 0, j = Ln - k * L.ny;
+      put(L.peers, cur + Ln * L.nx + u,
+          prolong_value<T>(op.d, oc.d, op.dmask, oc.dmask, [&](int pc) {
+            // a level's values from the CTA that owns their line (the coarsest: from the own copy)
+            return last ? xc[pc] : *cl.map_shared_rank(xc + pc, cl_div(pc, inv_nxc) & (cs - 1));
+          }, cur, Ln * L.nx + u, u < L.E ? 2 * u : 2 * (u - L.E) + 1, j, k));
+    }
+    cl.sync();
+    cur = sweeps(l, cur, P.nu2, false, false);
+    if (l == P.first) {
+      V* xg = (V*)P.L[l].x;
+      for (int lr = tid; lr < L.rows; lr += nt) {
+        const int i = cl_div(lr, L.inv_nx), Ln = rank + cs * i, p = Ln * L.nx + (lr - i * L.nx);
+        if (Ln < L.nlines) xg[p] = cur[p];
+      }
+    }
+  }
 }
 
 template <int KIND, int NB>
@@ -1289,69 +1755,99 @@ void fill_tail_masks(TailParams& P, int dim) {
   for (int c = 0; c < 8; ++c) P.zmask[c] = c < (1 << dim) ? zero_start_mask(dim, c) : 0u;
 }
 
-template <int NB>
-static cudaLaunchConfig_t tail_sm_config(int csize, int bytes, void* s, cudaLaunchAttribute* attr) {
-  cudaLaunchConfig_t cfg = tail_config<STORE_F32, NB>(csize, s, attr);
+// Runs f(kernel) on the instantiation of k_vcycle_cl for a storage kind and stencil.
+template <typename F>
+static auto with_cl(int kind, int nb, F f) {
+  if (nb == 27) return kind == STORE_F64 ? f(k_vcycle_cl<STORE_F64, 27>) : f(k_vcycle_cl<STORE_F32, 27>);
+  return kind == STORE_F64 ? f(k_vcycle_cl<STORE_F64, 9>) : f(k_vcycle_cl<STORE_F32, 9>);
+}
+
+static cudaLaunchConfig_t tail_cl_config(int csize, int bytes, void* s, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(csize, 1, 1);
+  cfg.blockDim = dim3(TAIL_THREADS, 1, 1);
   cfg.dynamicSmemBytes = (size_t)bytes;
+  cfg.stream = (cudaStream_t)s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = csize;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
   return cfg;
 }
 
-// The kernel's dynamic shared-memory cap is set to the device's opt-in
-// maximum, not to this plan's size: grids of different sizes share the
-// kernel, and each launch passes its own size.
-template <int NB>
-static bool tail_sm_fits(int csize, int bytes, int optin) {
-  if (cudaFuncSetAttribute(k_vcycle_tail_sm<NB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute(k_vcycle_tail_sm<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+// Lays out k_vcycle_cl's shared memory for a cluster of csize CTAs: every level's
+// vectors first, then the matrices of as many levels as fit, the smallest first.
+static bool tail_cl_layout(TailParams& P, int kind, int nb, int csize, int optin) {
+  const int te = kind == STORE_F64 ? 8 : 4;
+  long long at = 0;
+  auto take = [&](long long bytes) {
+    const long long o = at;
+    at += (bytes + 15) / 16 * 16;
+    return o;
+  };
+  for (int l = P.first; l < P.coarsest; ++l) {
+    const Dims& d = P.L[l].op.d;
+    const int nl = d.ny * (d.dim == 3 ? d.nz : 1);
+    const long long halo = ((d.dim == 3 ? (long long)d.nx * d.ny : 0) + d.nx + d.E + 1) / 2 * 2;   // pairs, 16-byte multiple
+    if (d.nv >= (1 << 20)) return false;   // (cl_div's range)
+    P.cl_rows[l] = (nl + csize - 1) / csize * d.nx;
+    P.cl_x[l] = (int)(take((d.nv + 2 * halo) * 2 * te) + halo * 2 * te);
+    P.cl_t[l] = P.smoother == 1 ? P.cl_x[l] : (int)(take((d.nv + 2 * halo) * 2 * te) + halo * 2 * te);
+    P.cl_b[l] = (int)take((long long)P.cl_rows[l] * 2 * te);
+    P.cl_list[l] = (int)take((4 + 4LL * (P.cl_rows[l] / d.nx)) * sizeof(int));
+    if (at > optin) return false;
   }
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = tail_sm_config<NB>(csize, bytes, nullptr, attr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_vcycle_tail_sm<NB>, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  P.cl_b[P.coarsest] = (int)take((long long)P.N * te);
+  P.cl_x[P.coarsest] = P.cl_t[P.coarsest] = (int)take((long long)P.N * te);
+  P.cl_vec_bytes = (int)at;
+  for (int l = P.coarsest - 1; l >= P.first; --l) {
+    const long long bytes = (long long)(nb + 1) * P.cl_rows[l] * 4 * te;
+    P.cl_a[l] = at + bytes <= optin ? (int)take(bytes) : -1;
   }
-  return n >= 1;
+  P.cl_bytes = (int)at;
+  P.cl_cs = csize;
+  return at <= optin;
 }
 
-bool tail_sm_plan(TailParams& P, int nb, int csize) {
-  P.sm_bytes = 0;
-  P.sm_cs = 0;
-  if (csize <= 0) return false;
+// The kernel's dynamic shared-memory cap is set to the device's opt-in maximum,
+// not to this plan's size: grids of different sizes share the kernel, and each
+// launch passes its own size.
+bool tail_cl_plan(TailParams& P, int kind, int nb) {
+  P.cl_bytes = 0;
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  long long base = 0;
-  for (int l = P.first; l < P.coarsest; ++l) {
-    const Dims& d = P.L[l].op.d;
-    const int nlines = d.ny * (d.dim == 3 ? d.nz : 1);
-    P.sm_lines[l] = (nlines + csize - 1) / csize;
-    P.sm_rows[l] = P.sm_lines[l] * d.nx;
-    P.sm_base[l] = (int)base;
-    base += (long long)(nb + 1) * P.sm_rows[l];
+  for (int csize = 16; csize >= 8; csize /= 2) {
+    if (!tail_cl_layout(P, kind, nb, csize, optin)) continue;
+    const bool ok = with_cl(kind, nb, [&](auto kernel) {
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
+        return false;
+      cudaLaunchAttribute attr[2];
+      cudaLaunchConfig_t cfg = tail_cl_config(csize, P.cl_bytes, nullptr, attr);
+      cfg.numAttrs = 1;
+      int n = 0;
+      return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+    });
+    if (ok) return true;
+    cudaGetLastError();
   }
-  const long long bytes = 16 * base;
-  if (bytes <= 0 || bytes > optin) return false;
-  if (!(nb == 27 ? tail_sm_fits<27>(csize, (int)bytes, optin) : tail_sm_fits<9>(csize, (int)bytes, optin))) return false;
-  P.sm_bytes = (int)bytes;
-  P.sm_cs = csize;
-  return true;
+  P.cl_bytes = 0;
+  return false;
 }
 
-cudaError_t launch_vcycle_tail_sm(const TailParams& P, int nb, void* s) {
-  cudaLaunchAttribute attr[1];
+cudaError_t launch_vcycle_cl(const TailParams& P, int kind, int nb, void* s) {
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = tail_cl_config(P.cl_cs, P.cl_bytes, s, attr);
   count_launch();
-  if (nb == 27) {
-    cudaLaunchConfig_t cfg = tail_sm_config<27>(P.sm_cs, P.sm_bytes, s, attr);
-    return cudaLaunchKernelEx(&cfg, k_vcycle_tail_sm<27>, P);
-  }
-  cudaLaunchConfig_t cfg = tail_sm_config<9>(P.sm_cs, P.sm_bytes, s, attr);
-  return cudaLaunchKernelEx(&cfg, k_vcycle_tail_sm<9>, P);
+  return with_cl(kind, nb, [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, P); });
 }
 
 cudaError_t launch_vcycle_tail(const TailParams& P, int kind, int nb, int csize, void* s) {
@@ -2501,20 +2997,35 @@ __global__ void __launch_bounds__(GS_PAIR_MAX_THREADS) k_gs_pair_shared(const __
 }
 
 // ----------------------------------------------------------------- launchers
+// FP64 levels that are not small launch without programmatic dependence: their
+// kernels are FP64-pipe-bound and few waves long, and blocks of the next launch
+// that settle early on the SMs that finish first leave it unevenly spread
+// (FP64 GS solves with and without: 97^3 21.3 and 16.0 ms, 129^3 32.1 and 29.5
+// ms).  FP32 kernels gain from it (97^3 GS 8.5 and 8.1 ms).
+static bool level_pdl(const LevelOp& L) { return L.kind != STORE_F64 || L.small; }
+
 template <int KIND, bool FINE>
 static void residual_t(const LevelOp& L, const void* b, const void* x, void* r, void* s) {
   typedef typename V2<typename Ty<KIND>::T>::t V;
   const int bs = L.block > 0 ? L.block : 256;
   const int g = (int)((L.d.nv + bs - 1) / bs);
-  if (L.batched) {
+  if (KIND == STORE_F32 && L.small) {
+    const int gs = (int)((L.d.nv + 63) / 64);
+    if (L.d.nb == 27) RF_LAUNCH_PDL((k_residual_small<27, FINE>), gs, 64, 0, s, L, (const float2*)b, (const float2*)x, (float2*)r);
+    else RF_LAUNCH_PDL((k_residual_small<9, FINE>), gs, 64, 0, s, L, (const float2*)b, (const float2*)x, (float2*)r);
+  } else if (KIND == STORE_F64 && L.small) {
+    const int gs = (int)((2 * L.d.nv + 63) / 64);
+    if (L.d.nb == 27) RF_LAUNCH_PDL((k_residual_small64<27, FINE>), gs, 64, 0, s, L, (const double2*)b, (const double2*)x, (double2*)r);
+    else RF_LAUNCH_PDL((k_residual_small64<9, FINE>), gs, 64, 0, s, L, (const double2*)b, (const double2*)x, (double2*)r);
+  } else if (L.batched) {
     if (L.d.nb == 27)
-      RF_LAUNCH_PDL((k_residual<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
     else
-      RF_LAUNCH_PDL((k_residual<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
   } else if (L.d.nb == 27)
-    RF_LAUNCH_PDL((k_residual<KIND, FINE, 27, 0>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual<KIND, FINE, 27, 0>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
   else
-    RF_LAUNCH_PDL((k_residual<KIND, FINE, 9, 0>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual<KIND, FINE, 9, 0>), g, bs, 0, s, L, (const V*)b, (const V*)x, (V*)r);
 }
 
 template <int KIND, bool FINE>
@@ -2523,15 +3034,27 @@ static void jacobi_t(const LevelOp& L, const void* b, const void* xin, void* xou
   typedef typename V2<typename Ty<KIND>::T>::t V;
   const int bs = L.block > 0 ? L.block : 256;
   const int g = (int)((L.d.nv + bs - 1) / bs);
-  if (L.batched) {
+  if (KIND == STORE_F32 && L.small && !zero_x) {
+    const int gs = (int)((L.d.nv + 63) / 64);
     if (L.d.nb == 27)
-      RF_LAUNCH_PDL((k_jacobi<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
+      RF_LAUNCH_PDL((k_jacobi_small<27, FINE>), gs, 64, 0, s, L, (const float2*)b, (const float2*)xin, (float2*)xout, omega);
     else
-      RF_LAUNCH_PDL((k_jacobi<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
+      RF_LAUNCH_PDL((k_jacobi_small<9, FINE>), gs, 64, 0, s, L, (const float2*)b, (const float2*)xin, (float2*)xout, omega);
+  } else if (KIND == STORE_F64 && L.small && !zero_x) {
+    const int gs = (int)((2 * L.d.nv + 63) / 64);
+    if (L.d.nb == 27)
+      RF_LAUNCH_PDL((k_jacobi_small64<27, FINE>), gs, 64, 0, s, L, (const double2*)b, (const double2*)xin, (double2*)xout, omega);
+    else
+      RF_LAUNCH_PDL((k_jacobi_small64<9, FINE>), gs, 64, 0, s, L, (const double2*)b, (const double2*)xin, (double2*)xout, omega);
+  } else if (L.batched) {
+    if (L.d.nb == 27)
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
+    else
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
   } else if (L.d.nb == 27)
-    RF_LAUNCH_PDL((k_jacobi<KIND, FINE, 27, 0>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi<KIND, FINE, 27, 0>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
   else
-    RF_LAUNCH_PDL((k_jacobi<KIND, FINE, 9, 0>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi<KIND, FINE, 9, 0>), g, bs, 0, s, L, (const V*)b, (const V*)xin, (V*)xout, omega, (int)zero_x);
 }
 
 // First forward sweep from x = 0: the neighbours of colour c that have a
@@ -2640,16 +3163,40 @@ static void for_colour_pairs(const Dims& d, bool forward, bool zero_start, bool 
 template <int KIND, bool FINE>
 static void gs_t(const LevelOp& L, const void* b, void* x, bool forward, bool zero_start, bool flip, void* s) {
   typedef typename V2<typename Ty<KIND>::T>::t V;
-  // FP64 levels keep one launch per colour: with pairs the all-FP64 solve
-  // measured 3% slower (its fine smoother 6%), and the batched FP64 pair
-  // kernel needs 129 registers, one 288-thread block per SM
+  // FP64 levels take one launch per colour unless they are small: with pairs
+  // the all-FP64 257^3 solve measured 3% slower (its fine smoother 6%), as the
+  // batched FP64 pair kernel needs 129 registers, one 288-thread block per SM
   int lpb = 1, threads = 32;
-  if (KIND != STORE_F64 && gs_pairs() && pair_shape(L.d.nx, lpb, threads)) {
+  if ((KIND != STORE_F64 || L.small) && gs_pairs() && pair_shape(L.d.nx, lpb, threads)) {
+    if (L.small) {       // spread over the SMs
+      lpb = 1;
+      threads = ((L.d.nx + 1) / 2 + 31) / 32 * 32;
+    }
     for_colour_pairs(L.d, forward, zero_start, flip,
                      [&](int fpx, int py, int pz, int lines_y, int nlines, uint32_t s1, uint32_t s2, int rev) {
       const int g = (nlines + lpb - 1) / lpb;
+      if (KIND == STORE_F32 && L.small) {
+#define RF_PAIR_SMALL(NBv, F)                                                                                      \
+  RF_LAUNCH_PDL((k_gs_pair_small<NBv, FINE, F>), g, threads, 0, s, L, (const float2*)b, (float2*)x, py, pz, lines_y, \
+                nlines, lpb, s1, s2)
+        if (L.d.nb == 27) { if (fpx) RF_PAIR_SMALL(27, 1); else RF_PAIR_SMALL(27, 0); }
+        else if (fpx) RF_PAIR_SMALL(9, 1);
+        else RF_PAIR_SMALL(9, 0);
+#undef RF_PAIR_SMALL
+        return;
+      }
+      if (KIND == STORE_F64 && L.small) {
+#define RF_PAIR_SMALL(NBv, F)                                                                                         \
+  RF_LAUNCH_PDL((k_gs_pair_small64<NBv, FINE, F>), nlines, std::min(NBv == 27 ? 128 : 288, (L.d.nx + 32) / 32 * 32), 0, s, L, (const double2*)b, (double2*)x, py, pz, lines_y, \
+                s1, s2)
+        if (L.d.nb == 27) { if (fpx) RF_PAIR_SMALL(27, 1); else RF_PAIR_SMALL(27, 0); }
+        else if (fpx) RF_PAIR_SMALL(9, 1);
+        else RF_PAIR_SMALL(9, 0);
+#undef RF_PAIR_SMALL
+        return;
+      }
 #define RF_PAIR(NBv, CHv, F)                                                                                     \
-  RF_LAUNCH_PDL((k_gs_pair<KIND, FINE, NBv, CHv, F>), g, threads, 0, s, L, (const V*)b, (V*)x, py, pz, lines_y, \
+  RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_pair<KIND, FINE, NBv, CHv, F>), g, threads, 0, s, L, (const V*)b, (V*)x, py, pz, lines_y, \
                 nlines, lpb, s1, s2, rev)
 #define RF_PAIR_PX(NBv, CHv) \
   if (fpx) RF_PAIR(NBv, CHv, 1); else RF_PAIR(NBv, CHv, 0)
@@ -2671,13 +3218,13 @@ static void gs_t(const LevelOp& L, const void* b, void* x, bool forward, bool ze
     const int g = (int)((count + bs - 1) / bs);
     if (L.batched) {
       if (L.d.nb == 27)
-        RF_LAUNCH_PDL((k_gs_colour<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
+        RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
       else
-        RF_LAUNCH_PDL((k_gs_colour<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
+        RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
     } else if (L.d.nb == 27) {
-      RF_LAUNCH_PDL((k_gs_colour<KIND, FINE, 27, 0>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour<KIND, FINE, 27, 0>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
     } else {
-      RF_LAUNCH_PDL((k_gs_colour<KIND, FINE, 9, 0>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour<KIND, FINE, 9, 0>), g, bs, 0, s, L, (const V*)b, (V*)x, px, py, pz, cnt_x, lines_y, count, skip, rev);
     }
   });
 }
@@ -2764,12 +3311,12 @@ static void residual_bt(const LevelOp& L, const SysBatch& B, void* s) {
   const int bs = L.block > 0 ? L.block : 256;
   const dim3 g((unsigned)((L.d.nv + bs - 1) / bs), (unsigned)B.n);
   if (L.batched) {
-    if (L.d.nb == 27) RF_LAUNCH_PDL((k_residual_b<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, B);
-    else RF_LAUNCH_PDL((k_residual_b<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, B);
+    if (L.d.nb == 27) RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual_b<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, B);
+    else RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual_b<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, B);
   } else if (L.d.nb == 27) {
-    RF_LAUNCH_PDL((k_residual_b<KIND, FINE, 27, 0>), g, bs, 0, s, L, B);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual_b<KIND, FINE, 27, 0>), g, bs, 0, s, L, B);
   } else {
-    RF_LAUNCH_PDL((k_residual_b<KIND, FINE, 9, 0>), g, bs, 0, s, L, B);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_residual_b<KIND, FINE, 9, 0>), g, bs, 0, s, L, B);
   }
 }
 
@@ -2779,12 +3326,12 @@ static void jacobi_bt(const LevelOp& L, const SysBatch& B, double omega, bool ze
   const dim3 g((unsigned)((L.d.nv + bs - 1) / bs), (unsigned)B.n);
   const int zx = zero_x ? 1 : 0;
   if (L.batched) {
-    if (L.d.nb == 27) RF_LAUNCH_PDL((k_jacobi_b<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, B, omega, zx);
-    else RF_LAUNCH_PDL((k_jacobi_b<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, B, omega, zx);
+    if (L.d.nb == 27) RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi_b<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, B, omega, zx);
+    else RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi_b<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, B, omega, zx);
   } else if (L.d.nb == 27) {
-    RF_LAUNCH_PDL((k_jacobi_b<KIND, FINE, 27, 0>), g, bs, 0, s, L, B, omega, zx);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi_b<KIND, FINE, 27, 0>), g, bs, 0, s, L, B, omega, zx);
   } else {
-    RF_LAUNCH_PDL((k_jacobi_b<KIND, FINE, 9, 0>), g, bs, 0, s, L, B, omega, zx);
+    RF_LAUNCH_PDL_IF(level_pdl(L), (k_jacobi_b<KIND, FINE, 9, 0>), g, bs, 0, s, L, B, omega, zx);
   }
 }
 
@@ -2796,7 +3343,7 @@ static void gs_bt(const LevelOp& L, const SysBatch& B, bool forward, bool zero_s
                      [&](int fpx, int py, int pz, int lines_y, int nlines, uint32_t s1, uint32_t s2, int rev) {
       const dim3 g((unsigned)((nlines + lpb - 1) / lpb), (unsigned)B.n);
 #define RF_PAIR(NBv, CHv, F) \
-  RF_LAUNCH_PDL((k_gs_pair_b<KIND, FINE, NBv, CHv, F>), g, threads, 0, s, L, B, py, pz, lines_y, nlines, lpb, s1, s2, rev)
+  RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_pair_b<KIND, FINE, NBv, CHv, F>), g, threads, 0, s, L, B, py, pz, lines_y, nlines, lpb, s1, s2, rev)
 #define RF_PAIR_PX(NBv, CHv) \
   if (fpx) RF_PAIR(NBv, CHv, 1); else RF_PAIR(NBv, CHv, 0)
       if (L.batched) {
@@ -2817,13 +3364,13 @@ static void gs_bt(const LevelOp& L, const SysBatch& B, bool forward, bool zero_s
     const dim3 g((unsigned)((count + bs - 1) / bs), (unsigned)B.n);
     if (L.batched) {
       if (L.d.nb == 27)
-        RF_LAUNCH_PDL((k_gs_colour_b<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
+        RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour_b<KIND, FINE, 27, chunk_of(KIND)>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
       else
-        RF_LAUNCH_PDL((k_gs_colour_b<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
+        RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour_b<KIND, FINE, 9, chunk_of(KIND)>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
     } else if (L.d.nb == 27) {
-      RF_LAUNCH_PDL((k_gs_colour_b<KIND, FINE, 27, 0>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour_b<KIND, FINE, 27, 0>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
     } else {
-      RF_LAUNCH_PDL((k_gs_colour_b<KIND, FINE, 9, 0>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
+      RF_LAUNCH_PDL_IF(level_pdl(L), (k_gs_colour_b<KIND, FINE, 9, 0>), g, bs, 0, s, L, B, px, py, pz, cnt_x, lines_y, count, skip, rev);
     }
   });
 }

@@ -120,13 +120,13 @@ __device__ __forceinline__ void rf_pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// launch with the programmatic-stream-serialisation attribute (the kernel
-// must begin with rf_pdl_begin())
+// launch with the programmatic-stream-serialisation attribute where `pdl` says
+// (the kernel must begin with rf_pdl_begin())
 template <typename... KArgs, typename... Args>
-inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+inline void launch_pdl(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                        Args&&... args) {
   count_launch();
-  if (!pdl_enabled()) {
+  if (!pdl || !pdl_enabled()) {
     kernel<<<grid, block, smem, stream>>>(std::forward<Args>(args)...);
     return;
   }
@@ -151,5 +151,7 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     kernel<<<(grid), (block), (smem), (cudaStream_t)(stream)>>>(__VA_ARGS__); \
   } while (0)
 
+#define RF_LAUNCH_PDL_IF(pdl, kernel, grid, block, smem, stream, ...) \
+  ::rf::launch_pdl(pdl, kernel, dim3(grid), dim3(block), (size_t)(smem), (cudaStream_t)(stream), __VA_ARGS__)
 #define RF_LAUNCH_PDL(kernel, grid, block, smem, stream, ...) \
-  ::rf::launch_pdl(kernel, dim3(grid), dim3(block), (size_t)(smem), (cudaStream_t)(stream), __VA_ARGS__)
+  ::rf::launch_pdl(true, kernel, dim3(grid), dim3(block), (size_t)(smem), (cudaStream_t)(stream), __VA_ARGS__)

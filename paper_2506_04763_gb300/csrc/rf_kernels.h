@@ -68,6 +68,7 @@ struct LevelOp {
   const uint8_t* dmask;  // [nv]
   int block = 256;       // threads per block of the smoothing / residual kernels (autotuned)
   bool batched = false;  // smoothing / residual kernels issue 9 blocks' loads per round trip
+  bool small = false;    // a level whose launches cost latency: colour pairs spread over the SMs, FP32 rows loaded whole
   uint32_t nomask = 0;   // always 0: a stencil skip mask the compiler cannot fold (see apply_row)
 };
 
@@ -103,22 +104,22 @@ struct TailParams {
   unsigned* bar;
   double* status;
   long long limit_ns;
-  // shared-memory form (k_vcycle_tail_sm, sm_bytes > 0): CTA r of the
-  // cluster's sm_cs keeps the stencil blocks and D^-1 of its x-lines
-  // L = r + sm_cs * i (i < sm_lines[l]) of every level below the coarsest,
-  // level l's blocks from float4 sm_base[l] on, block b of local row lr at
-  // sm_base[l] + b * sm_rows[l] + lr, D^-1 after the last block
-  int sm_bytes, sm_cs;
-  int sm_lines[RF_MAXL], sm_rows[RF_MAXL], sm_base[RF_MAXL];
+  // k_vcycle_cl (cl_bytes > 0), a cluster of cl_cs CTAs: byte offsets in each
+  // CTA's shared memory of every level's x and second iterate (after their
+  // halos), b, line lists and matrix rows (-1: left in global memory); rows per CTA; the
+  // vectors' total, from the start
+  int cl_bytes, cl_cs, cl_vec_bytes;
+  int cl_rows[RF_MAXL], cl_x[RF_MAXL], cl_t[RF_MAXL], cl_b[RF_MAXL], cl_a[RF_MAXL],
+      cl_list[RF_MAXL];
   TailLevel L[RF_MAXL];
 };
 int tail_cluster_size(int kind, int nb);
 void fill_tail_masks(TailParams& P, int dim);
 cudaError_t launch_vcycle_tail(const TailParams& P, int kind, int nb, int csize, void* s);
-// the shared-memory form (FP32 levels, GS smoother): fills P.sm_* for cluster
-// size csize and returns true if it fits and can be co-scheduled
-bool tail_sm_plan(TailParams& P, int nb, int csize);
-cudaError_t launch_vcycle_tail_sm(const TailParams& P, int nb, void* s);
+// the form with its vectors in shared memory (FP64 and FP32 levels): fills
+// P.cl_* and returns true if it fits and can be co-scheduled
+bool tail_cl_plan(TailParams& P, int kind, int nb);
+cudaError_t launch_vcycle_cl(const TailParams& P, int kind, int nb, void* s);
 // the same V-cycle as one cooperative launch of `blocks` blocks (coop_tail_blocks: all that fit at once)
 int coop_tail_blocks(int kind, int nb);
 cudaError_t launch_vcycle_coop(const TailParams& P, int kind, int nb, int blocks, void* s);
