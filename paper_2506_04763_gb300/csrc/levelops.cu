@@ -13,6 +13,9 @@
 // All of these are HBM-bandwidth kernels except the set-up ones.
 #include <cooperative_groups.h>
 #include <algorithm>
+#include <array>
+#include <map>
+#include <mutex>
 #include <type_traits>
 
 #include "rf_common.cuh"
@@ -1826,7 +1829,13 @@ bool tail_cl_plan(TailParams& P, int kind, int nb) {
   }
   for (int csize = 16; csize >= 8; csize /= 2) {
     if (!tail_cl_layout(P, kind, nb, csize, optin)) continue;
-    const bool ok = with_cl(kind, nb, [&](auto kernel) {
+    // whether such a cluster can be co-scheduled: asked once per process
+    static std::mutex mu;
+    static std::map<std::array<int, 5>, bool> asked;
+    std::lock_guard<std::mutex> lk(mu);
+    const std::array<int, 5> key{dev, kind, nb, csize, P.cl_bytes};
+    const auto it = asked.find(key);
+    const bool ok = it != asked.end() ? it->second : with_cl(kind, nb, [&](auto kernel) {
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
           cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
         return false;
@@ -1836,6 +1845,7 @@ bool tail_cl_plan(TailParams& P, int kind, int nb) {
       int n = 0;
       return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
     });
+    asked[key] = ok;
     if (ok) return true;
     cudaGetLastError();
   }
