@@ -44,8 +44,9 @@ namespace rf {
 struct Phys {
   double rho_w, rho_n, mu_w, mu_n, S_wr, S_nr, lam, den;
   double h[3], g[3];
-  double rh[3], rmu_w, nid;   // 1 / h, 1 / mu_w (rounded), -1 / den
+  double rh[3], rmu_w, rmu_n, rden, nid;   // 1 / h, 1 / mu_w, 1 / mu_n, 1 / den (rounded), -1 / den
   double Af[3], gw[3], gn[3]; // SCV face sizes, rho_w g, rho_n g per axis
+  double gt[3][3];            // w / h by axis and number of 1/4 factors in w
   int scheme;   // SCHEME_* bits (0: the discretisation of Sec. 3)
 };
 
@@ -217,7 +218,7 @@ __global__ void k_vertex_state(Dims d, Phys ph, const double2* __restrict__ u, c
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= d.nv) return;
   double2 uv = u[p];
-  double se = __ddiv_rn(__dsub_rn(__dsub_rn(1.0, uv.y), ph.S_wr), ph.den);
+  double se = div_by(__dsub_rn(__dsub_rn(1.0, uv.y), ph.S_wr), ph.den, ph.rden);
   double J, dJ, k, dk;
   leverett(ph.lam, se, J, dJ);
   krw_of(ph.lam, se, k, dk);
@@ -225,17 +226,17 @@ __global__ void k_vertex_state(Dims d, Phys ph, const double2* __restrict__ u, c
   double c = __dmul_rn(pdm, J);
   Se[p] = se;
   pc[p] = c;
-  dpc[p] = -(pdm * dJ) / ph.den;
+  dpc[p] = div_by(-(pdm * dJ), ph.den, ph.rden);
   pn[p] = __dadd_rn(uv.x, c);
   // the upwinded water mobility lambda_w = k_rw / mu_w and its S_n-derivative,
   // divided here once per vertex instead of once per face visit
-  krw[p] = k / ph.mu_w;
-  dkrw[p] = (-dk / ph.den) / ph.mu_w;
+  krw[p] = div_by(k, ph.mu_w, ph.rmu_w);
+  dkrw[p] = div_by(div_by(-dk, ph.den, ph.rden), ph.mu_w, ph.rmu_w);
   // lambda_n = k_rn / mu_n where S hat = S_e (the elements of the vertex's
   // lowest entry pressure), and its S_n-derivative
   krn_of(ph.lam, se, k, dk);
-  krn[p] = k / ph.mu_n;
-  dkrn[p] = dk * 1.0 * ph.nid / ph.mu_n;
+  krn[p] = div_by(k, ph.mu_n, ph.rmu_n);
+  dkrn[p] = div_by(dk * ph.nid, ph.mu_n, ph.rmu_n);
 }
 
 // ---------------------------------------------------------------- K1 / K1r
@@ -445,46 +446,43 @@ __global__ void __launch_bounds__(128) k_assemble(Dims d, Phys ph, AsmIn in, dou
 // K1 is FP64-pipe-bound on GB300 (0.53 T FMA/s against 6.8 TB/s), so it is
 // organised to evaluate nothing twice.  Two passes over slabs of cell planes:
 //   k_asm_faces  one thread per element and axis evaluates the element's SCV
-//     faces along that axis and leaves, per face, the fluxes F_w, F_n and six
-//     numbers from which every entry of J they reach follows;
-//   k_asm_rows   gathers them per vertex: the water threads write the entries
+//     faces along that axis and leaves, per face, the fluxes F_w, F_n and their
+//     derivatives by the 2^d corners' unknowns;
+//   k_asm_rows   adds them up per vertex: the water threads write the entries
 //     (w, p_w), (w, S_n) and F_w, the NAPL threads (n, p_w), (n, S_n), F_n and
 //     M.  Every row is written once, complete (no zero fill, no read-modify-
-//     write, no colours, no atomics), in a fixed order of sums.
-// Face f of row r along axis k, with D the 3-bit offset of corner q from r and
-// W = prod over the other axes of (D_t ? 1/4 : 3/4):
-//   dF_w/dp_w(q) = -+ alpha W,  dF_w/dS_n(q) = -+ beta W dpc(q) +- gamma W/2
-//   (+ delta at the upwind vertex),  the same with nu and eta for F_n,
-//   alpha = rho_w lam_w,up K A_f / h,  beta = rho_w (lam_w,up - lam_w,M) K A_f / h,
-//   gamma = rho_w lam_w,M' T_c,  delta = rho_w lam_w,up' T_w,  nu = rho_n
-//   lam_n,up K A_f / h,  eta = rho_n lam_n,up' T_n.
-// The four faces around one edge of r differ only in W, which factors over the
-// two other axes: their 3 x 3 entries are the tensor transform (a, b) -> (a,
-// 3 (a + b), b) along each, 5 sums (the 1/16 is stored with the coefficient,
-// exactly, and the 3s go into multiply-adds); and since dpc(q)
-// depends on the vertex q alone, the beta of all faces are summed before one
-// product per block.  The face arithmetic that a decision rests on (gradients, T,
-// S_e at x_M, S hat) is the vertex kernel's, operation by operation, and k_rw,
-// k_rn and their derivatives are too (1 - S_e^2 cancels where k_rn ~ 0).
+//     write, no atomics).
+// A preconditioned solve amplifies a last-bit difference of its matrix or right-
+// hand side by 10^2 or more per iteration, so the values are those of the
+// element-by-element assembly to the last bit: each derivative in the vertex
+// kernel's operations, and a row's contributions added in the order of the
+// elements' colours (parities of their lower corner), within an element along
+// x, y, z.  The row pass takes its vertex's neighbours mirrored along the
+// axes where the vertex's coordinate is odd: the colour order is then the same
+// sequence of offsets for every vertex, and the 27 accumulators stay in
+// registers.
+// Of a face's derivatives by p_w only d are distinct (the weights of its
+// corners: 3/4 or 1/4 per other axis), +- by side; those are stored once.
 // Measured on GB300 (F, J and M; then F alone), against one thread per element
 // adding its faces' 768 entries into J colour by colour (4,154 FP64 instructions
 // per vertex; on small grids 8 dependent chains of about 190 us): 257^3 150.9 ->
-// 63.1 ms (52.1 -> 25.8 ms), 65^3 2.79 -> 1.10 ms (1.00 -> 0.48), 17^3 1.57 ->
-// 0.067 ms (0.60 -> 0.042), 33^2 0.224 -> 0.041 ms.  ncu at 97^3: FP64 pipe 83%
-// busy in k_asm_faces, 73% in k_asm_rows, DRAM below 15% of its peak.
-constexpr int NCO = 8;   // numbers per face with J: F_w, F_n, alpha, beta, gamma, delta, nu, eta
-constexpr int NCO_F = 2; // without
+// 91.0 ms (52.1 -> 25.2 ms), 65^3 2.79 -> 1.54 ms (1.00 -> 0.47), 17^3 1.57 -> 0.071
+// ms (0.60 -> 0.042), 33^2 0.224 -> 0.039 ms.  About 1790 FP64 instructions per
+// element in the first pass and 840 per vertex in the second, whose pipe is 83%
+// and 80% busy (ncu at 97^3); DRAM below 15% of its peak.  (Summing a row's faces
+// before their products with dp_c/dS_n, not to the last bit, took 63.1 ms.)
+// numbers per face: F_w, F_n, and with J the distinct dF_w/dp_w and dF_n/dp_w
+// and the 2^d dF_w/dS_n and dF_n/dS_n
+__host__ __device__ constexpr int nco(int dim, bool want_j) { return want_j ? 2 + 2 * dim + (2 << dim) : 2; }
 
 // A slab: cell planes [c0, c1) along axis ax (z in 3D, y in 2D; y in 3D too
 // where z planes are too large for the workspace) in face workspace W, plane c
 // in ring slot c % ring (the plane below the slab stays for the slab's first
 // vertex plane).  Number m of face f (axis * 2^(d-1) + position) of in-plane
-// cell q lies at W[(f * NCO + m) * ws + slot * pc + q], its axis' upwind bits
-// (2 per position: water, NAPL from the lower vertex) at U[axis * ws + ...].
-// Cells are parity-split along x as vertices are.
+// cell q lies at W[(f * nco + m) * ws + slot * pc + q].  Cells are parity-split
+// along x as vertices are.
 struct Slab {
   double* W;
-  uint8_t* U;
   int ws, pc, ring, c0, c1, ax;
 };
 
@@ -501,9 +499,15 @@ __device__ __forceinline__ bool not_below(double x) {
   return hi >= 0 || (((uint32_t)hi << 1) | (uint32_t)__double2loint(x)) == 0u;
 }
 
+// -x where neg: the sign bit alone (an addition and a subtraction behind a
+// select would both issue on the FP64 pipe)
+__device__ __forceinline__ double flip_sign(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
+}
+
 template <int DIM, int K, bool WANT_J, bool DARCY>
 __device__ __forceinline__ void faces_of_axis(const Dims& d, const Phys& ph, const AsmIn& in, const Slab& sl, int t) {
-  constexpr int NC = 1 << DIM, NE = 1 << (DIM - 1), CO = WANT_J ? NCO : NCO_F;
+  constexpr int NC = 1 << DIM, NE = 1 << (DIM - 1), CO = nco(DIM, WANT_J);
   constexpr int O1 = K == 0 ? 1 : 0, O2 = K == 2 ? 1 : 2;   // the other axes, in order
   const int cx = d.nx - 1, cy = d.ny - 1, EC = (cx + 1) / 2;
   const int pl = (int)((uint32_t)t / (uint32_t)sl.pc), q0 = t - pl * sl.pc;
@@ -532,10 +536,14 @@ __device__ __forceinline__ void faces_of_axis(const Dims& d, const Phys& ph, con
     if (DARCY) dw[e] = __dsub_rn(in.u[vq[b]].x, in.u[vq[a]].x);
   }
   const double gw = ph.gw[K], gn = ph.gn[K];
-  const double kah = div_by(KA, h, rh) * (DIM == 3 ? 0.0625 : 0.25);
-  const double gsc = ph.rho_w * ph.nid * (DIM == 3 ? 0.03125 : 0.125);
   const int wi = (int)((uint32_t)plane % (uint32_t)sl.ring) * sl.pc + q0;
-  uint32_t up = 0;
+  double dT[DIM], dpcq[NC];        // K A_f w / h by the number of 1/4 factors
+  if (WANT_J) {
+#pragma unroll
+    for (int m = 0; m < DIM; ++m) dT[m] = KA * ph.gt[K][m];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) dpcq[q] = in.dpc[vq[q]];
+  }
 #pragma unroll
   for (int e = 0; e < NE; ++e) {
     const int a = (e & 1) << O1 | (DIM == 3 ? (e >> 1) << O2 : 0), b = a | 1 << K;
@@ -602,16 +610,47 @@ __device__ __forceinline__ void faces_of_axis(const Dims& d, const Phys& ph, con
     W[0] = DARCY ? ph.rho_w * (lw_up * Tpw) : ph.rho_w * (lw_up * Tw - lwM * Tc);
     W[(size_t)sl.ws] = ph.rho_n * (ln_up * Tn);
     if (WANT_J) {
-      up |= (wa ? 1u : 0u) << (2 * e) | (na ? 2u : 0u) << (2 * e);
-      W[2 * (size_t)sl.ws] = (ph.rho_w * lw_up) * kah;
-      W[3 * (size_t)sl.ws] = DARCY ? 0.0 : (ph.rho_w * (lw_up - lwM)) * kah;
-      W[4 * (size_t)sl.ws] = DARCY ? 0.0 : (div_by(dkM, ph.mu_w, ph.rmu_w) * gsc) * Tc;
-      W[5 * (size_t)sl.ws] = (ph.rho_w * dlw_up) * (DARCY ? Tpw : Tw);
-      W[6 * (size_t)sl.ws] = (ph.rho_n * ln_up) * kah;
-      W[7 * (size_t)sl.ws] = (ph.rho_n * dln_up) * Tn;
+      const double dlM = div_by(dkM, ph.mu_w, ph.rmu_w);
+      const double rlw = ph.rho_w * lw_up, rln = ph.rho_n * ln_up;
+      const double selw = dlw_up * (DARCY ? Tpw : Tw), seln = dln_up * Tn;
+      double U[DIM], V[DIM], G[DIM], L[DIM];
+#pragma unroll
+      for (int m = 0; m < DIM; ++m) {
+        W[(size_t)(2 + m) * sl.ws] = rlw * dT[m];
+        W[(size_t)(2 + DIM + m) * sl.ws] = rln * dT[m];
+        double w = 0.5;
+#pragma unroll
+        for (int t = 0; t < DIM - 1; ++t) w = w * (t < m ? 0.25 : 0.75);
+        U[m] = lw_up * dT[m];
+        V[m] = lwM * dT[m];
+        L[m] = ln_up * dT[m];
+        G[m] = w * dlM * ph.nid * Tc;
+      }
+      // corner j: bits 0, 1 = differs from the face's position along the other
+      // axes, then the side along K; d T / d p(q) is -dT above, +dT below
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        const int side = j >> (DIM - 1), m = (j & 1) + (DIM == 3 ? (j >> 1) & 1 : 0);
+        const int q = ((e ^ j) & 1) << O1 | (DIM == 3 ? (((e ^ j) >> 1) & 1) << O2 : 0) | side << K;
+        const bool up = (j & (NE - 1)) == 0;       // the face's own edge: its upwind end takes the k_r slope
+        double d1, d3;
+        if (DARCY) {
+          d1 = up && wa == (side == 0) ? selw : 0.0;
+        } else {
+          const double A = U[m] * dpcq[q], C = V[m] * dpcq[q];
+          d1 = side ? -A : A;
+          if (up) d1 = (wa == (side == 0) ? selw : 0.0) + d1;
+          d1 = d1 - G[m];
+          d1 = side ? d1 + C : d1 - C;
+        }
+        const double B = L[m] * dpcq[q];
+        d3 = side ? -B : B;
+        if (up) d3 = (na == (side == 0) ? seln : 0.0) + d3;
+        W[(size_t)(2 + 2 * DIM + j) * sl.ws] = ph.rho_w * d1;
+        W[(size_t)(2 + 2 * DIM + NC + j) * sl.ws] = ph.rho_n * d3;
+      }
     }
   }
-  if (WANT_J) sl.U[(size_t)K * sl.ws + wi] = (uint8_t)up;
 }
 
 template <int DIM, bool WANT_J, bool DARCY>
@@ -624,161 +663,20 @@ __global__ void __launch_bounds__(128) k_asm_faces(const __grid_constant__ Dims 
   else if (DIM == 3) faces_of_axis<DIM, DIM - 1, WANT_J, DARCY>(d, ph, in, sl, t);
 }
 
-// The faces around one vertex, edge by edge: edge (K, S) runs from the vertex
-// along axis K in direction S, and the 2^(d-1) elements around it each hold one
-// of its faces.  ce[c] is the workspace index of the element whose corner c
-// (bits x, y, z) the vertex is, or -1 outside the grid.
-
-// block of the stencil at offset 0 (the edge's own end) or S (its far end)
-// along K, and d1, d2 along the other axes in order
-template <int DIM, int K, int S>
-__device__ __forceinline__ int edge_blk(int far, int d1, int d2) {
-  const int dk = far ? S : 0;
-  const int dx = K == 0 ? dk : d1;
-  const int dy = K == 0 ? d1 : (K == 1 ? dk : d2);
-  const int dz = DIM == 3 ? (K == 2 ? dk : d2) : 0;
-  return DIM == 3 ? (dx + 1) + 3 * (dy + 1) + 9 * (dz + 1) : (dx + 1) + 3 * (dy + 1);
-}
-
-// the element of edge (K, S) on sides (s1, s2: 0 = below, 1 = above) of the
-// other axes: its bits as a corner index, and the edge's face position in it
-template <int DIM, int K, int S>
-__device__ __forceinline__ int edge_elem(int s1, int s2) {
-  const int bk = S > 0 ? 0 : 1, b1 = s1 ? 0 : 1, b2 = s2 ? 0 : 1;
-  const int x = K == 0 ? bk : b1, y = K == 0 ? b1 : (K == 1 ? bk : b2), z = DIM == 3 ? (K == 2 ? bk : b2) : 0;
-  return x | y << 1 | z << 2;
-}
-
-template <int DIM, int K, int S, int CO>
-__device__ __forceinline__ void edge_load(const double* __restrict__ W, int ws, int m, const int (&ce)[1 << DIM],
-                                          double (&v)[1 << (DIM - 1)]) {
-  constexpr int NE = 1 << (DIM - 1);
-#pragma unroll
-  for (int f = 0; f < NE; ++f) {          // f: sides (s1, s2)
-    const int s1 = f & 1, s2 = (f >> 1) & 1;
-    const int c = ce[edge_elem<DIM, K, S>(s1, s2)];
-    const int e = (s1 ? 0 : 1) | (DIM == 3 ? (s2 ? 0 : 2) : 0);   // face position in that element
-    v[f] = c >= 0 ? W[(size_t)((K * NE + e) * CO + m) * ws + c] : 0.0;
-  }
-}
-
-// adds (or subtracts) the tensor transform of the edge's faces v to the blocks
-// at its own end and to those at its far end; its factors 3 and 9 ride on the
-// accumulation's multiply-add
-// (INIT: of an accumulator that holds nothing yet, the blocks this edge is the
-// first to reach, the edges in row_diff's order, are set instead)
-template <int DIM, int K, int S, int NB, bool INIT = false>
-__device__ __forceinline__ void edge_add(const double (&v)[1 << (DIM - 1)], bool own_minus, bool far_minus,
-                                         double (&acc)[NB]) {
-  constexpr bool SET_OWN = INIT && K == 0 && S < 0, SET_FAR = INIT && K == 0;
-  double E[DIM == 3 ? 9 : 3];             // without the factors
-  if (DIM == 3) {
-#pragma unroll
-    for (int s2 = 0; s2 < 2; ++s2) {      // rows d2 = -1 and +1
-      E[6 * s2 + 0] = v[2 * s2];
-      E[6 * s2 + 1] = v[2 * s2] + v[2 * s2 + 1];
-      E[6 * s2 + 2] = v[2 * s2 + 1];
-    }
-#pragma unroll
-    for (int t = 0; t < 3; ++t) E[3 + t] = E[t] + E[6 + t];
-  } else {
-    E[0] = v[0]; E[1] = v[0] + v[1]; E[2] = v[1];
-  }
-#pragma unroll
-  for (int t = 0; t < (DIM == 3 ? 9 : 3); ++t) {
-    const int d1 = t % 3 - 1, d2 = DIM == 3 ? t / 3 - 1 : 0;
-    const double f = (d1 == 0 ? 3.0 : 1.0) * (DIM == 3 && d2 == 0 ? 3.0 : 1.0);
-    const int b0 = edge_blk<DIM, K, S>(0, d1, d2), b1 = edge_blk<DIM, K, S>(1, d1, d2);
-    acc[b0] = SET_OWN ? (own_minus ? -f : f) * E[t] : __fma_rn(own_minus ? -f : f, E[t], acc[b0]);
-    acc[b1] = SET_FAR ? (far_minus ? -f : f) * E[t] : __fma_rn(far_minus ? -f : f, E[t], acc[b1]);
-  }
-}
-
-// every edge of the vertex: own end -, far end + (alpha, beta, nu); sets acc
-template <int DIM, int NB, int CO>
-__device__ __forceinline__ void row_diff(const double* __restrict__ W, int ws, int m, const int (&ce)[1 << DIM],
-                                         double (&acc)[NB]) {
-  double v[1 << (DIM - 1)];
-  edge_load<DIM, 0, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 0, -1, NB, true>(v, true, false, acc);
-  edge_load<DIM, 0, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 0, 1, NB, true>(v, true, false, acc);
-  edge_load<DIM, 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 1, -1, NB, true>(v, true, false, acc);
-  edge_load<DIM, 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 1, 1, NB, true>(v, true, false, acc);
-  if (DIM == 3) {
-    edge_load<DIM, DIM - 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, DIM - 1, -1, NB, true>(v, true, false, acc);
-    edge_load<DIM, DIM - 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, DIM - 1, 1, NB, true>(v, true, false, acc);
-  }
-}
-
-// both ends + for the edges that leave upwards, - for those that come from below (gamma)
-template <int DIM, int NB, int CO>
-__device__ __forceinline__ void row_mean(const double* __restrict__ W, int ws, int m, const int (&ce)[1 << DIM],
-                                         double (&acc)[NB]) {
-  double v[1 << (DIM - 1)];
-  edge_load<DIM, 0, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 0, -1, NB>(v, true, true, acc);
-  edge_load<DIM, 0, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 0, 1, NB>(v, false, false, acc);
-  edge_load<DIM, 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, 1, -1, NB>(v, true, true, acc);
-  edge_load<DIM, 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, 1, 1, NB>(v, false, false, acc);
-  if (DIM == 3) {
-    edge_load<DIM, DIM - 1, -1, CO>(W, ws, m, ce, v); edge_add<DIM, DIM - 1, -1, NB>(v, true, true, acc);
-    edge_load<DIM, DIM - 1, 1, CO>(W, ws, m, ce, v);  edge_add<DIM, DIM - 1, 1, NB>(v, false, false, acc);
-  }
-}
-
-// one edge's upwind terms (delta, eta; m, upwind bit BIT) and flux (mf):
-// the vertex is the edge's lower end for S > 0 (row: -) and its upper one for
-// S < 0 (row: +); a term goes to the block of the face's upwind vertex
-template <int DIM, int K, int S, int NB, int CO, bool WANT_J>
-__device__ __forceinline__ void edge_up(const Slab& sl, const int (&ce)[1 << DIM], int m, int bit, int mf,
-                                        double (&acc)[NB], double& F) {
-  constexpr int NE = 1 << (DIM - 1);
-  double fv[NE];
-  edge_load<DIM, K, S, CO>(sl.W, sl.ws, mf, ce, fv);
-#pragma unroll
-  for (int f = 0; f < NE; ++f) F = S > 0 ? F - fv[f] : F + fv[f];
-  if (WANT_J) {
-    const int b0 = edge_blk<DIM, K, S>(0, 0, 0), b1 = edge_blk<DIM, K, S>(1, 0, 0);
-    double v[NE];
-    edge_load<DIM, K, S, CO>(sl.W, sl.ws, m, ce, v);
-    double own = 0.0, far = 0.0;
-#pragma unroll
-    for (int f = 0; f < NE; ++f) {
-      const int s1 = f & 1, s2 = (f >> 1) & 1;
-      const int c = ce[edge_elem<DIM, K, S>(s1, s2)];
-      const int e = (s1 ? 0 : 1) | (DIM == 3 ? (s2 ? 0 : 2) : 0);
-      const bool lower = c >= 0 && ((sl.U[(size_t)K * sl.ws + c] >> (2 * e + bit)) & 1);
-      const bool mine = lower == (S > 0);
-      own += mine ? v[f] : 0.0;
-      far += mine ? 0.0 : v[f];
-    }
-    acc[b0] = S > 0 ? acc[b0] - own : acc[b0] + own;
-    acc[b1] = S > 0 ? acc[b1] - far : acc[b1] + far;
-  }
-}
-
-template <int DIM, int NB, int CO, bool WANT_J>
-__device__ __forceinline__ void row_up(const Slab& sl, const int (&ce)[1 << DIM], int m, int bit, int mf,
-                                       double (&acc)[NB], double& F) {
-  edge_up<DIM, 0, -1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
-  edge_up<DIM, 0, 1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
-  edge_up<DIM, 1, -1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
-  edge_up<DIM, 1, 1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
-  if (DIM == 3) {
-    edge_up<DIM, DIM - 1, -1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
-    edge_up<DIM, DIM - 1, 1, NB, CO, WANT_J>(sl, ce, m, bit, mf, acc, F);
-  }
-}
-
 // Vertex planes [v0, v1): 32 vertices per block, one warp their water rows and
 // one their NAPL rows (so that the two halves of each 32-byte block are written
-// at about the same time; the water rows' accumulators take 182 registers, and
-// blocks of two warps let an SM hold 10 warps instead of 8).  Sources, Dirichlet p_w rows (0 =
-// p_dir - p_w: J row -e, M row 0) and the mass diagonal are applied here.
+// at about the same time; with blocks of two warps an SM holds ten of these
+// warps, whose accumulators take 108 registers).  Sources, Dirichlet p_w rows (0
+// = p_dir - p_w: J row -e, M row 0) and the mass diagonal are applied here.
+// c: the element of colour c, whose corner s = (vertex parity ^ c) the vertex is.
+// In mirrored coordinates it extends to +1 along the axes where c's bit is 0
+// and to -1 where it is 1.
 template <int DIM, bool WANT_J>
 __global__ void __launch_bounds__(64) k_asm_rows(const __grid_constant__ Dims d, const __grid_constant__ Phys ph,
-                                                  const __grid_constant__ AsmIn in, const __grid_constant__ Slab sl, int v0, int v1,
-                                                  double* __restrict__ F, double* __restrict__ J,
-                                                  double2* __restrict__ mdiag) {
-  constexpr int NC = 1 << DIM, NB = DIM == 3 ? 27 : 9, CO = WANT_J ? NCO : NCO_F;
+                                                 const __grid_constant__ AsmIn in, const __grid_constant__ Slab sl, int v0,
+                                                 int v1, double* __restrict__ F, double* __restrict__ J,
+                                                 double2* __restrict__ mdiag) {
+  constexpr int NC = 1 << DIM, NE = 1 << (DIM - 1), NB = DIM == 3 ? 27 : 9, CO = nco(DIM, WANT_J);
   const int napl = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nline = DIM == 2 ? 1 : sl.ax == 1 ? d.nz : d.ny;    // x-lines per vertex plane
   const int64_t t = (int64_t)blockIdx.x * 32 + lane;
@@ -789,80 +687,89 @@ __global__ void __launch_bounds__(64) k_asm_rows(const __grid_constant__ Dims d,
   const int j = DIM == 2 || sl.ax == 1 ? vpl : line, k = DIM == 2 ? 0 : sl.ax == 1 ? line : vpl;
   const int64_t p = ((int64_t)j + (int64_t)d.ny * k) * d.nx + vpos;
   const int cx = d.nx - 1, cy = d.ny - 1, cz = DIM == 3 ? d.nz - 1 : 1, EC = (cx + 1) / 2;
-  int ce[NC];
+  const int par = (i & 1) | (j & 1) << 1 | (DIM == 3 ? (k & 1) << 2 : 0);
+  double a0[NB], a1[NB], f = 0.0;
+  if (WANT_J) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) { a0[b] = 0.0; a1[b] = 0.0; }
+  }
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = DIM == 3 ? k - ((c >> 2) & 1) : 0;
-    const bool ok = ci >= 0 && ci < cx && cj >= 0 && cj < cy && ck >= 0 && ck < cz;
+    const int s = par ^ c;
+    const int ci = i - (s & 1), cj = j - ((s >> 1) & 1), ck = DIM == 3 ? k - ((s >> 2) & 1) : 0;
+    if (ci < 0 || ci >= cx || cj < 0 || cj >= cy || ck < 0 || ck >= cz) continue;
     const int pos = (ci & 1) ? EC + (ci >> 1) : (ci >> 1);
     const int plane = DIM == 2 || sl.ax == 1 ? cj : ck, cl = DIM == 2 ? 0 : sl.ax == 1 ? ck : cj;
-    ce[c] = ok ? (int)((uint32_t)plane % (uint32_t)sl.ring) * sl.pc + cl * cx + pos : -1;
+    const double* W = sl.W + ((uint32_t)plane % (uint32_t)sl.ring) * (uint32_t)sl.pc + cl * cx + pos;
+    double fe = 0.0;
+#pragma unroll
+    for (int kk = 0; kk < DIM; ++kk) {
+      const int o1 = kk == 0 ? 1 : 0, o2 = kk == 2 ? 1 : 2;
+      const int e = ((s >> o1) & 1) | (DIM == 3 ? ((s >> o2) & 1) << 1 : 0);
+      const double* Wf = W + (size_t)((kk * NE + e) * CO) * sl.ws;
+      const int sk = (s >> kk) & 1;              // the vertex is the face's lower (0: row -) or upper (1: row +) end
+      const double fv = Wf[(size_t)napl * sl.ws];
+      fe = fe + flip_sign(fv, sk == 0);
+      if (WANT_J) {
+        const double* Wx = Wf + (size_t)(2 + napl * DIM) * sl.ws;
+        const double* Wown = Wf + (size_t)(2 + 2 * DIM + napl * NC + sk * NE) * sl.ws;
+        const double* Wfar = Wf + (size_t)(2 + 2 * DIM + napl * NC + (1 - sk) * NE) * sl.ws;
+        double x[DIM], own[NE], far[NE];
+#pragma unroll
+        for (int m = 0; m < DIM; ++m) x[m] = Wx[(size_t)m * sl.ws];
+#pragma unroll
+        for (int r = 0; r < NE; ++r) {
+          own[r] = flip_sign(Wown[(size_t)r * sl.ws], sk == 0);
+          far[r] = flip_sign(Wfar[(size_t)r * sl.ws], sk == 0);
+        }
+#pragma unroll
+        for (int r = 0; r < NE; ++r) {
+          // corner r of the face's other axes: mirrored block offsets of its two sides
+          const int D1 = r & 1, D2 = DIM == 3 ? (r >> 1) & 1 : 0, m = D1 + D2;
+          const int u1 = D1 ? ((c >> o1) & 1 ? -1 : 1) : 0, u2 = D2 ? ((c >> o2) & 1 ? -1 : 1) : 0;
+          const int uk = (c >> kk) & 1 ? -1 : 1;
+          const int st1 = o1 == 0 ? 1 : 3, st2 = o2 == 1 ? 3 : 9, stk = kk == 0 ? 1 : kk == 1 ? 3 : 9;
+          const int bo = (DIM == 3 ? 13 : 4) + u1 * st1 + (DIM == 3 ? u2 * st2 : 0), bf = bo + uk * stk;
+          a0[bo] = a0[bo] - x[m];
+          a0[bf] = a0[bf] + x[m];
+          a1[bo] = a1[bo] + own[r];
+          a1[bf] = a1[bf] + far[r];
+        }
+      }
+    }
+    f += fe;
   }
   const bool dirv = in.dir[p] != 0;
-  double a1[NB];
-  double f = 0.0;
-  if (!napl) {
-    if (WANT_J) {
-      // (w, S_n): the beta sums times dpc, then gamma and delta
-      row_diff<DIM, NB, CO>(sl.W, sl.ws, 3, ce, a1);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        const int dx = b % 3 - 1, dy = (b / 3) % 3 - 1, dz = DIM == 3 ? b / 9 - 1 : 0;
-        const int ii = i + dx, jj = j + dy, kk = k + dz;
-        const bool ok = ii >= 0 && ii < d.nx && jj >= 0 && jj < d.ny && (DIM == 2 || (kk >= 0 && kk < d.nz));
-        a1[b] = ok ? a1[b] * in.dpc[pidx(d, ii, jj, kk)] : 0.0;
-      }
-      row_mean<DIM, NB, CO>(sl.W, sl.ws, 4, ce, a1);
-    }
-    row_up<DIM, NB, CO, WANT_J>(sl, ce, 5, 0, 0, a1, f);
-    if (WANT_J) {
-      double a0[NB];
-      row_diff<DIM, NB, CO>(sl.W, sl.ws, 2, ce, a0);
-      constexpr int C = DIM == 3 ? 13 : 4;
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        const double2 e = dirv ? make_double2(b == C ? -1.0 : 0.0, 0.0) : make_double2(a0[b], a1[b]);
-        *reinterpret_cast<double2*>(J + ((int64_t)b * d.nv + p) * 4) = e;
-      }
-    }
-    if (in.q_in) f += in.q_in[p].x;
-    if (dirv) f = in.pw_dir[p] - in.u[p].x;
-    F[2 * p] = f;
-    return;
-  }
   if (WANT_J) {
-    row_diff<DIM, NB, CO>(sl.W, sl.ws, 6, ce, a1);
-    double a3[NB];
+    constexpr int C = DIM == 3 ? 13 : 4;
+    const int fx = i & 1 ? -1 : 1, fy = j & 1 ? -3 : 3, fz = DIM == 3 ? (k & 1 ? -9 : 9) : 0;   // back from the mirror
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-      const int dx = b % 3 - 1, dy = (b / 3) % 3 - 1, dz = DIM == 3 ? b / 9 - 1 : 0;
-      const int ii = i + dx, jj = j + dy, kk = k + dz;
-      const bool ok = ii >= 0 && ii < d.nx && jj >= 0 && jj < d.ny && (DIM == 2 || (kk >= 0 && kk < d.nz));
-      a3[b] = ok ? a1[b] * in.dpc[pidx(d, ii, jj, kk)] : 0.0;
+      const int br = C + (b % 3 - 1) * fx + ((b / 3) % 3 - 1) * fy + (DIM == 3 ? (b / 9 - 1) * fz : 0);
+      double2 v = make_double2(a0[b], a1[b]);
+      if (dirv && !napl) v = make_double2(b == C ? -1.0 : 0.0, 0.0);
+      *reinterpret_cast<double2*>(J + ((int64_t)br * d.nv + p) * 4 + 2 * napl) = v;
     }
-    row_up<DIM, NB, CO, WANT_J>(sl, ce, 7, 1, 1, a3, f);
-#pragma unroll
-    for (int b = 0; b < NB; ++b)
-      *reinterpret_cast<double2*>(J + ((int64_t)b * d.nv + p) * 4 + 2) = make_double2(a1[b], a3[b]);
-    double pvol = in.phiv[p];
-    if (ph.scheme & SCHEME_SHAT_STORAGE) {
-      const double frac = DIM == 3 ? 0.125 : 0.25, se = in.Se[p], pdm = in.pdmin[p];
-      pvol = 0.0;
-      for (int c = 0; c < NC; ++c) {
-        const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = DIM == 3 ? k - ((c >> 2) & 1) : 0;
-        if (ci < 0 || ci >= cx || cj < 0 || cj >= cy || ck < 0 || ck >= cz) continue;
-        const int64_t cell = ci + (int64_t)cx * (cj + (int64_t)cy * ck);
-        double sh, dsh;
-        shat_of(ph.lam, se, in.pd[cell], pdm, sh, dsh);
-        pvol += in.phi[cell] * in.vol * frac * dsh;
+    if (napl) {
+      double pvol = in.phiv[p];
+      if (ph.scheme & SCHEME_SHAT_STORAGE) {
+        const double frac = DIM == 3 ? 0.125 : 0.25, se = in.Se[p], pdm = in.pdmin[p];
+        pvol = 0.0;
+        for (int c = 0; c < NC; ++c) {
+          const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = DIM == 3 ? k - ((c >> 2) & 1) : 0;
+          if (ci < 0 || ci >= cx || cj < 0 || cj >= cy || ck < 0 || ck >= cz) continue;
+          const int64_t cell = ci + (int64_t)cx * (cj + (int64_t)cy * ck);
+          double sh, dsh;
+          shat_of(ph.lam, se, in.pd[cell], pdm, sh, dsh);
+          pvol += in.phi[cell] * in.vol * frac * dsh;
+        }
       }
+      mdiag[p] = make_double2(dirv ? 0.0 : -ph.rho_w * pvol, ph.rho_n * pvol);
     }
-    mdiag[p] = make_double2(dirv ? 0.0 : -ph.rho_w * pvol, ph.rho_n * pvol);
-  } else {
-    row_up<DIM, NB, CO, WANT_J>(sl, ce, 7, 1, 1, a1, f);
   }
-  if (in.q_in) f += in.q_in[p].y;
-  F[2 * p + 1] = f;
+  if (in.q_in) f += napl ? in.q_in[p].y : in.q_in[p].x;
+  if (dirv && !napl) f = in.pw_dir[p] - in.u[p].x;
+  F[2 * p + napl] = f;
 }
 
 // ---------------------------------------------------------------- storage (S hat variant)
@@ -910,16 +817,15 @@ void launch_perm_scalar_to_p(const Dims& d, const double* nat, double* out, void
 }
 
 // Face workspace of one assembly: at most ASM_WS_BYTES (with J; F alone a
-// quarter of that, as its faces need a quarter of the numbers), at least two
-// cell planes.  At 257^3 a slab then holds 9 planes (50 MB each), 15 waves of
-// k_asm_faces.  Slabs go along z, or along y where two z planes exceed the
+// quarter of that), at least two cell planes.  At 257^3 the ring then holds 3
+// planes of 151 MB, and a slab of 2 is 10 waves of k_asm_faces.  Slabs go along z, or along y where two z planes exceed the
 // limit and y planes are smaller (wide, shallow boxes).
 constexpr size_t ASM_WS_BYTES = (size_t)512 << 20;
 
 struct SlabShape { int ax, planes, ring; int64_t plane; };
 
 static SlabShape slab_shape(const Dims& d, bool want_j) {
-  const size_t cell = (size_t)(d.dim << (d.dim - 1)) * (want_j ? NCO : NCO_F) * sizeof(double);
+  const size_t cell = (size_t)(d.dim << (d.dim - 1)) * nco(d.dim, want_j) * sizeof(double);
   const int64_t fit = (int64_t)((want_j ? ASM_WS_BYTES : ASM_WS_BYTES / 4) / cell);   // cells
   const int64_t zp = (int64_t)(d.nx - 1) * (d.ny - 1), yp = (int64_t)(d.nx - 1) * (d.dim == 3 ? d.nz - 1 : 1);
   SlabShape r;
@@ -933,8 +839,7 @@ static SlabShape slab_shape(const Dims& d, bool want_j) {
 
 size_t assemble_workspace(const Dims& d, bool want_j) {
   const SlabShape r = slab_shape(d, want_j);
-  const size_t cell = (size_t)(d.dim << (d.dim - 1)) * (want_j ? NCO : NCO_F) * sizeof(double);
-  return (size_t)(r.ring * r.plane) * (cell + (want_j ? d.dim : 0));
+  return (size_t)(r.ring * r.plane) * (d.dim << (d.dim - 1)) * nco(d.dim, want_j) * sizeof(double);
 }
 
 template <int DIM, bool WANT_J>
@@ -947,7 +852,6 @@ static void slabs_t(const Dims& d, const Phys& ph, const AsmIn& in, const AsmArr
   sl.pc = (int)sh.plane;
   sl.ws = (int)(sh.plane * sh.ring);
   sl.W = a.faces;
-  sl.U = reinterpret_cast<uint8_t*>(a.faces + (size_t)sl.ws * (DIM << (DIM - 1)) * (WANT_J ? NCO : NCO_F));
   // the first slab fills the ring; a later one leaves the plane below it in place
   for (int c0 = 0, v0 = 0; c0 < planes;) {
     const int c1 = c0 == 0 ? sl.ring : (c0 + sl.ring - 1 < planes ? c0 + sl.ring - 1 : planes);
@@ -974,6 +878,8 @@ cudaError_t launch_assemble(const Dims& d, const PhysParams& pp, const AsmArrays
   ph.scheme = pp.scheme;
   for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = 1.0 / pp.h[t]; }
   ph.rmu_w = 1.0 / pp.mu_w;
+  ph.rmu_n = 1.0 / pp.mu_n;
+  ph.rden = 1.0 / ph.den;
   ph.nid = -1.0 / ph.den;
   for (int t = 0; t < 3; ++t) {
     ph.Af[t] = 1.0;
@@ -981,6 +887,11 @@ cudaError_t launch_assemble(const Dims& d, const PhysParams& pp, const AsmArrays
       if (m != t) ph.Af[t] *= pp.h[m] * 0.5;
     ph.gw[t] = pp.rho_w * pp.g[t];
     ph.gn[t] = pp.rho_n * pp.g[t];
+    for (int m = 0; m < 3; ++m) {
+      double w = 1.0;
+      for (int q = 0; q < d.dim - 1; ++q) w *= q < m ? 0.25 : 0.75;
+      ph.gt[t][m] = w / pp.h[t];
+    }
   }
   const int nblk = (int)((d.nv + 255) / 256);
   RF_LAUNCH(k_vertex_state, nblk, 256, 0, s, d, ph, (const double2*)a.u, a.pdmin, a.Se, a.pn, a.pc, a.dpc,
@@ -1034,6 +945,8 @@ void launch_storage_sw(const Dims& d, const PhysParams& pp, const double* u, con
   ph.scheme = pp.scheme;
   for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = 1.0 / pp.h[t]; }
   ph.rmu_w = 1.0 / pp.mu_w;
+  ph.rmu_n = 1.0 / pp.mu_n;
+  ph.rden = 1.0 / ph.den;
   ph.nid = -1.0 / ph.den;
   for (int t = 0; t < 3; ++t) {
     ph.Af[t] = 1.0;
@@ -1041,6 +954,11 @@ void launch_storage_sw(const Dims& d, const PhysParams& pp, const double* u, con
       if (m != t) ph.Af[t] *= pp.h[m] * 0.5;
     ph.gw[t] = pp.rho_w * pp.g[t];
     ph.gn[t] = pp.rho_n * pp.g[t];
+    for (int m = 0; m < 3; ++m) {
+      double w = 1.0;
+      for (int q = 0; q < d.dim - 1; ++q) w *= q < m ? 0.25 : 0.75;
+      ph.gt[t][m] = w / pp.h[t];
+    }
   }
   RF_LAUNCH(k_storage_sw, (int)((d.nv + 255) / 256), 256, 0, s, d, ph, (const double2*)u, pdmin, phi, pd, vol, sw);
 }

@@ -1879,13 +1879,14 @@ cudaError_t launch_vcycle_tail(const TailParams& P, int kind, int nb, int csize,
 // With L, C, R the blocks of fine rows 2I - 1, 2I, 2I + 1 (missing rows are
 // zero) at offsets -1, 0, 1 along the axis, the output blocks of row I are
 //   D = -1: (L[-1] + L[0]/2 + C[-1]) / 2
-//   D =  0: C[0] + (C[-1] + C[1] + L[1] + R[-1] + (L[0] + R[0])/2) / 2
-//   D = +1: (R[1] + R[0]/2 + C[1]) / 2.
+//   D =  0: (L[0]/2 + L[1] + C[-1] + 2 C[0] + C[1] + R[-1] + R[0]/2) / 2
+//   D = +1: (C[1] + R[0]/2 + R[1]) / 2,
+// summed in this order (rows, then columns upwards).
 // The fine masks D_f are applied while reading the first stage, the coarse
 // masks D_c (and the identity of coarse Dirichlet rows) when writing the last.
 //
 // A thread makes the three blocks D of one row and one pair of other offsets:
-// 9 block loads and 12 FP64 operations per entry (the set-up is FP64-pipe-bound
+// 9 block loads and 13 FP64 operations per entry (the set-up is FP64-pipe-bound
 // on large grids).  M of the finest level is vertex-diagonal, so until the
 // stages have spread it along an axis its blocks off that axis are zero and
 // neither read nor written.  The stages run over windows of planes along the
@@ -2002,8 +2003,10 @@ __global__ void __launch_bounds__(128) k_galerkin(const __grid_constant__ GalSta
       }
     double2 o[3];
     o[0] = gal_scale(gal_add(gal_half(A[0][0], A[0][1]), A[1][0]));
-    o[1] = gal_half(A[1][1], gal_half(gal_add(gal_add(A[1][0], A[1][2]), gal_add(A[0][2], A[2][0])), gal_add(A[0][1], A[2][1])));
-    o[2] = gal_scale(gal_add(gal_half(A[2][2], A[2][1]), A[1][2]));
+    o[1] = gal_add(gal_half(A[0][2], A[0][1]), A[1][0]);
+    o[1] = make_double2(fma(2.0, A[1][1].x, o[1].x), fma(2.0, A[1][1].y, o[1].y));
+    o[1] = gal_scale(gal_half(gal_add(gal_add(o[1], A[1][2]), A[2][0]), A[2][1]));
+    o[2] = gal_scale(gal_add(gal_half(A[1][2], A[2][1]), A[2][2]));
     double m[3] = {0.0, 0.0, 0.0};
     if (has_m) {
       double B[3][3];
@@ -2018,8 +2021,8 @@ __global__ void __launch_bounds__(128) k_galerkin(const __grid_constant__ GalSta
           if (AX == 0 && h == 0 && ((mrow >> a) & 1)) B[a][e] = 0.0;
         }
       m[0] = 0.5 * (fma(0.5, B[0][1], B[0][0]) + B[1][0]);
-      m[1] = fma(0.5, fma(0.5, B[0][1] + B[2][1], (B[1][0] + B[1][2]) + (B[0][2] + B[2][0])), B[1][1]);
-      m[2] = 0.5 * (fma(0.5, B[2][1], B[2][2]) + B[1][2]);
+      m[1] = 0.5 * fma(0.5, B[2][1], ((fma(2.0, B[1][1], fma(0.5, B[0][1], B[0][2]) + B[1][0])) + B[1][2]) + B[2][0]);
+      m[2] = 0.5 * (fma(0.5, B[2][1], B[1][2]) + B[2][2]);
     }
 #pragma unroll
     for (int D = 0; D < 3; ++D) {

@@ -4,8 +4,8 @@ vertex: F, J and M over the shapes where its slabs and edges differ — one cell
 per axis, odd and even line lengths, 2D, several slabs along z, slabs along y
 (wide, shallow boxes), per-medium laws and the discretisation variants.
 
-Both kernels take the same decisions and round every face coefficient alike;
-the entries are sums of at most 24 face terms in another order, so rows agree
+Both kernels take the same decisions and round every face derivative alike;
+the entries are sums of at most 24 of them in another order, so rows agree
 to a few hundred roundings of their largest term (1e-13 of the row's largest
 entry covers it, as the terms of these states do not cancel by more than 10x).
 """
