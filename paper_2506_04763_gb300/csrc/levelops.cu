@@ -2185,7 +2185,8 @@ __global__ void __launch_bounds__(256) k_pack_dinv(Dims d, bool fine, const doub
   const double2 m = fine ? md[p] : reinterpret_cast<const double2*>(M)[(int64_t)C * d.nv + p];
   for (int j = 0; j < out.n; ++j) {
     const double a00 = -u.x, a01 = out.shift[j] * m.x - u.y, a10 = -w.x, a11 = out.shift[j] * m.y - w.y;
-    const double det = a00 * a11 - a01 * a10, r = 1.0 / det;
+    // explicit, so that the inverse does not follow the compiler's choice of which product it fuses
+    const double det = __fma_rn(a00, a11, -__dmul_rn(a01, a10)), r = 1.0 / det;
     const uint32_t e = ((uint32_t)__double2hiint(det) >> 20) & 0x7ffu;
     double q[4] = {a11, -a01, -a10, a00};
 #pragma unroll
