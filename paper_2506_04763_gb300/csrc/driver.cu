@@ -2862,6 +2862,9 @@ extern "C" rf_status rf_apply(rf_grid* g, int op, int level, int sh, const doubl
   if (two && !in1) return fail(RF_EINVAL, "this operation needs in1");
   if ((op == RF_OP_RESTRICT || op == RF_OP_PROLONG) && level >= g->nl - 1) return fail(RF_EINVAL, "no coarser level");
   if (op == RF_OP_COARSE && level != g->nl - 1) return fail(RF_EINVAL, "RF_OP_COARSE works on the coarsest level");
+  // the coarsest level holds its inverse only
+  if ((op == RF_OP_SMOOTH || op == RF_OP_RESIDUAL) && !level_op(g, level, sh).A)
+    return fail(RF_EINVAL, "level %d has no packed operator", level);
   const Dims& d = g->L[level].d;
   const Dims& dc = (level + 1 < g->nl) ? g->L[level + 1].d : d;
   const Dims& dl = (op == RF_OP_PROLONG) ? dc : d;   // dims of in0
