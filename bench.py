@@ -49,12 +49,11 @@ GS_ALGO_PER_VERTEX = 456.0
 # (4 flop) and the fused inner products (<rh, v>: 4 flop; <t, s>, <t, t>: 8
 # flop), averaged over the two applications of an iteration.
 SPMV64_FLOP_PER_VERTEX = 216.0 + 4.0 + 6.0
-# FP64 instructions (DADD + DMUL + DFMA) per vertex of one K1 assembly with the
-# Jacobian, counted by ncu (smsp__sass_thread_inst_executed_op_d{add,mul,fma})
-# over the 8 colour launches of one assembly of this recipe at 129^3; K1 is
-# FP64-issue-bound, so its roofline is that instruction rate against the FMA
-# issue rate rf_fp64_fma_rate measures.
-K1_FP64_INST_PER_VERTEX = 4154.0
+# FP64 instructions per vertex of one K1 assembly with the Jacobian: about 1790
+# per element in the face pass (ncu, FP64 pipe instructions at 97^3) and 840 per
+# vertex in the row pass; K1 is FP64-issue-bound, so its roofline is that
+# instruction rate against the FMA issue rate rf_fp64_fma_rate measures.
+K1_FP64_INST_PER_VERTEX = 2630.0
 
 
 def args_():
@@ -373,10 +372,10 @@ def main():
                      "hbm_frac_same_kernel": per_class_frac(sp, pk["hbm"]),
                      "peak_source": "rf_fp64_fma_rate in this process (8 FMA chains per thread, 2 flop per FMA)"}
     k1_rate = K1_FP64_INST_PER_VERTEX * g.nv / (asm_ms / 1e3)
-    roofline_fp64["k1_assembly"] = {"kernel": "k_assemble_cells", "achieved_inst_per_s": k1_rate,
+    roofline_fp64["k1_assembly"] = {"kernel": "k_asm_faces + k_asm_rows", "achieved_inst_per_s": k1_rate,
                                     "peak_inst_per_s": fma_rate, "frac": round(k1_rate / fma_rate, 4),
                                     "inst_per_vertex": K1_FP64_INST_PER_VERTEX,
-                                    "source": "FP64 instruction count per vertex from ncu at 129^3; time measured here"}
+                                    "source": "FP64 instruction count per vertex from ncu at 97^3; time measured here"}
     shares = {k: round(v["ms"] / sum(p["ms"] for p in prof.values()), 4) for k, v in prof.items()}
     per_class = {k: {"ms_per_step": round(v["ms"] / a.steps, 3), "launches": v["launches"],
                      "GB_per_s": round(v["bytes"] / (v["ms"] / 1e3) / 1e9, 1) if v["ms"] > 0 else None,
