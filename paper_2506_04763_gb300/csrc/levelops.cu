@@ -2350,6 +2350,7 @@ __global__ void __launch_bounds__(GJ_THREADS) k_gauss_jordan(int N, const double
       if (t == 0) { cand[lr] = gj_key(v); step[lr] = -1; }
     }
   }
+  cl.sync();   // every CTA of the cluster runs before a peer writes into its table
   int pend = -1, pend_c = 0;      // the local row waiting for its scaling, its step and reciprocal pivot
   double pend_inv = 0.0;
   bool bad = false;
