@@ -13,11 +13,10 @@
 // All of these are HBM-bandwidth kernels except the set-up ones.
 #include <cooperative_groups.h>
 #include <algorithm>
-#include <array>
-#include <map>
-#include <mutex>
 #include <type_traits>
+#include <vector>
 
+#include "cluster_plan.h"
 #include "rf_common.cuh"
 #include "rf_kernels.h"
 
@@ -1816,41 +1815,60 @@ static bool tail_cl_layout(TailParams& P, int kind, int nb, int csize, int optin
   return at <= optin;
 }
 
+// choose_cluster's view of a kernel on the current device; cfg(cs, smem, attr): its launch
+template <typename Kernel, typename Cfg>
+struct ClusterCalls {
+  Kernel kernel;
+  Cfg cfg;
+  static bool ok(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+  }
+  int device() {
+    int dev = -1;
+    return ok(cudaGetDevice(&dev)) ? dev : -1;
+  }
+  size_t smem_optin() {
+    int v = 0;
+    return ok(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device())) ? (size_t)v : 0;
+  }
+  bool allow(size_t cap) {
+    return ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) &&
+           ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
+  }
+  int clusters(int cs, size_t smem) {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t c = cfg(cs, smem, attr);
+    c.numAttrs = 1;   // the cluster's dimension
+    int n = 0;
+    return ok(cudaOccupancyMaxActiveClusters(&n, kernel, &c)) ? n : -1;
+  }
+};
+template <typename Kernel, typename Cfg, typename Smem>
+static int choose_cluster_of(Kernel kernel, int id, const std::vector<int>& sizes, Cfg cfg, Smem smem) {
+  static ClusterAnswers known;   // (one per kernel type; id tells kernels of a type apart)
+  return choose_cluster(ClusterCalls<Kernel, Cfg>{kernel, cfg}, known, id, sizes, smem);
+}
+
 // The kernel's dynamic shared-memory cap is set to the device's opt-in maximum,
 // not to this plan's size: grids of different sizes share the kernel, and each
 // launch passes its own size.
 bool tail_cl_plan(TailParams& P, int kind, int nb) {
-  P.cl_bytes = 0;
   int dev = 0, optin = 0;
+  P.cl_bytes = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  for (int csize = 16; csize >= 8; csize /= 2) {
-    if (!tail_cl_layout(P, kind, nb, csize, optin)) continue;
-    // whether such a cluster can be co-scheduled: asked once per process
-    static std::mutex mu;
-    static std::map<std::array<int, 5>, bool> asked;
-    std::lock_guard<std::mutex> lk(mu);
-    const std::array<int, 5> key{dev, kind, nb, csize, P.cl_bytes};
-    const auto it = asked.find(key);
-    const bool ok = it != asked.end() ? it->second : with_cl(kind, nb, [&](auto kernel) {
-      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
-        return false;
-      cudaLaunchAttribute attr[2];
-      cudaLaunchConfig_t cfg = tail_cl_config(csize, P.cl_bytes, nullptr, attr);
-      cfg.numAttrs = 1;
-      int n = 0;
-      return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
-    });
-    asked[key] = ok;
-    if (ok) return true;
-    cudaGetLastError();
-  }
-  P.cl_bytes = 0;
-  return false;
+  const int cs = with_cl(kind, nb, [&](auto kernel) {
+    return choose_cluster_of(
+        kernel, kind * 64 + nb, {16, 8},
+        [](int c, size_t smem, cudaLaunchAttribute* attr) { return tail_cl_config(c, (int)smem, nullptr, attr); },
+        [&](int c) { return tail_cl_layout(P, kind, nb, c, optin) ? (size_t)P.cl_bytes : ~(size_t)0; });
+  });
+  if (cs == 0) P.cl_bytes = 0;   // (else the layout is that of cs, the last size asked for)
+  return cs > 0;
 }
 
 cudaError_t launch_vcycle_cl(const TailParams& P, int kind, int nb, void* s) {
@@ -2437,42 +2455,42 @@ __global__ void __launch_bounds__(GJ_THREADS) k_gauss_jordan(int N, const double
   if (!finite) status[mat] = 1;
 }
 
-// Cluster size of k_gauss_jordan for N unknowns (0: it does not fit).  A step's
-// update takes N ceil(N / cs) multiply-adds of a CTA, its barrier and copies
-// grow with cs.  Measured for one inverse, cs = 1 / 4 / 8 / 16 (the call's 40 us
-// of launch and read-back included): N = 50 205 / 135 / 137 / 152 us, N = 90
-// 524 / 280 / 245 / 271, N = 126 1068 / 461 / 386 / 406, N = 144 1522 / 637 /
-// 523 / 488, N = 250 - / - / 1298 / 1131.
-static int gj_cluster(int N) {
-  static const int optin = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-        cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize, v) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    return v;
-  }();
-  int cs = N <= 50 ? 4 : N < 144 ? 8 : 16;
-  while (cs < GJ_MAX_CS && gj_smem(N, cs) > (size_t)optin) cs *= 2;
-  return gj_smem(N, cs) <= (size_t)optin ? cs : 0;
-}
-
-static cudaError_t launch_gauss_jordan(int N, int nmat, int cs, const double* D, const InvOut& out, int* status, void* s) {
+static cudaLaunchConfig_t gj_config(int nmat, int cs, size_t smem, void* s, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cs * nmat, 1, 1);
   cfg.blockDim = dim3(GJ_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = gj_smem(N, cs);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = (cudaStream_t)s;
-  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Cluster size of k_gauss_jordan for N unknowns (0: it does not fit).  A step's
+// update takes N ceil(N / cs) multiply-adds of a CTA, its barrier and copies
+// grow with cs.  Measured for one inverse, cs = 1 / 4 / 8 / 16 (the call's 40 us
+// of launch and read-back included): N = 50 205 / 135 / 137 / 152 us, N = 90
+// 524 / 280 / 245 / 271, N = 126 1068 / 461 / 386 / 406, N = 144 1522 / 637 /
+// 523 / 488, N = 250 - / - / 1298 / 1131.  A size that the device refuses is
+// passed over: each gives the same inverse, bit for bit.
+static int gj_cluster(int N) {
+  std::vector<int> sizes;
+  const int first = N <= 50 ? 4 : N < 144 ? 8 : GJ_MAX_CS;
+  for (int cs = first; cs <= GJ_MAX_CS; cs *= 2) sizes.push_back(cs);
+  for (int cs = first / 2; cs >= 1; cs /= 2) sizes.push_back(cs);
+  return choose_cluster_of(
+      k_gauss_jordan, 0, sizes,
+      [](int cs, size_t smem, cudaLaunchAttribute* attr) { return gj_config(1, cs, smem, nullptr, attr); },
+      [&](int cs) { return gj_smem(N, cs); });
+}
+
+static cudaError_t launch_gauss_jordan(int N, int nmat, int cs, const double* D, const InvOut& out, int* status, void* s) {
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = gj_config(nmat, cs, gj_smem(N, cs), s, attr);
   count_launch();
   return cudaLaunchKernelEx(&cfg, k_gauss_jordan, N, D, out, status);
 }
