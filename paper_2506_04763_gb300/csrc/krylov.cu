@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(BS) k_bicg_v_df(Dims d, Nbr nb, const float4* 
                                                   const double2* __restrict__ md, double shift,
                                                   const float2* __restrict__ y, const double2* __restrict__ rh,
                                                   double2* __restrict__ v, double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(y, rh);
   double acc[1] = {0.0};
   for (int64_t p = blockIdx.x * (int64_t)BS + threadIdx.x; p < d.nv; p += (int64_t)gridDim.x * BS) {
     double y0, y1;
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(BS) k_bicg_t_df(Dims d, Nbr nb, const float4* 
                                                   const double2* __restrict__ md, double shift,
                                                   const float2* __restrict__ z, const double2* __restrict__ s,
                                                   double2* __restrict__ t, double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(z, s);
   double acc[2] = {0.0, 0.0};
   for (int64_t p = blockIdx.x * (int64_t)BS + threadIdx.x; p < d.nv; p += (int64_t)gridDim.x * BS) {
     double y0, y1;
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(BS) k_bicg_v(Dims d, Nbr nb, const double* __r
                                                const double2* __restrict__ md, double shift,
                                                const XV* __restrict__ y, const double2* __restrict__ rh,
                                                double2* __restrict__ v, double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(y, rh);
   double acc[1] = {0.0};
   for (int64_t p = blockIdx.x * (int64_t)BS + threadIdx.x; p < d.nv; p += (int64_t)gridDim.x * BS) {
     double y0, y1;
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(BS) k_bicg_t(Dims d, Nbr nb, const double* __r
                                                const double2* __restrict__ md, double shift,
                                                const XV* __restrict__ z, const double2* __restrict__ s,
                                                double2* __restrict__ t, double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(z, s);
   double acc[2] = {0.0, 0.0};
   for (int64_t p = blockIdx.x * (int64_t)BS + threadIdx.x; p < d.nv; p += (int64_t)gridDim.x * BS) {
     double y0, y1;
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(BS) k_true_res(Dims d, Nbr nb, const double* _
                                                  const double2* __restrict__ md, double shift,
                                                  const double2* __restrict__ x, const double2* __restrict__ b,
                                                  double2* __restrict__ r, double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(x, b);
   double acc[1] = {0.0};
   for (int64_t p = blockIdx.x * (int64_t)BS + threadIdx.x; p < d.nv; p += (int64_t)gridDim.x * BS) {
     double y0, y1;
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(BS) k_bicg_init(int64_t nv, const double2* __r
                                                   double2* __restrict__ r, double2* __restrict__ rh,
                                                   double2* __restrict__ p, double2* __restrict__ v,
                                                   double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(b);
   double acc[1] = {0.0};
   for (int64_t q = blockIdx.x * (int64_t)BS + threadIdx.x; q < nv; q += (int64_t)gridDim.x * BS) {
     const double2 bv = b[q];
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(BS) k_bicg_init(int64_t nv, const double2* __r
 __global__ void __launch_bounds__(BS) k_bicg_restart(int64_t nv, const double2* __restrict__ r,
                                                      double2* __restrict__ rh, double2* __restrict__ p,
                                                      double2* __restrict__ v, double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(r);
   double acc[1] = {0.0};
   for (int64_t q = blockIdx.x * (int64_t)BS + threadIdx.x; q < nv; q += (int64_t)gridDim.x * BS) {
     const double2 rv = r[q];
@@ -286,7 +286,7 @@ template <typename LV>
 __global__ void __launch_bounds__(BS) k_bicg_p(int64_t nv, const double* __restrict__ scal,
                                                const double2* __restrict__ r, const double2* __restrict__ v,
                                                double2* __restrict__ p, LV* __restrict__ plo) {
-  rf_pdl_begin();
+  rf_pdl_begin(scal, r, v, p);
   const double beta = scal[S_BETA], omega = scal[S_OMEGA];
   for (int64_t q = blockIdx.x * (int64_t)BS + threadIdx.x; q < nv; q += (int64_t)gridDim.x * BS) {
     const double2 rv = r[q], vv = v[q], pv = p[q];
@@ -301,7 +301,7 @@ template <typename LV>
 __global__ void __launch_bounds__(BS) k_bicg_s(int64_t nv, const double* __restrict__ scal,
                                                const double2* __restrict__ r, const double2* __restrict__ v,
                                                double2* __restrict__ s, LV* __restrict__ slo) {
-  rf_pdl_begin();
+  rf_pdl_begin(scal, r, v);
   const double alpha = scal[S_ALPHA];
   for (int64_t q = blockIdx.x * (int64_t)BS + threadIdx.x; q < nv; q += (int64_t)gridDim.x * BS) {
     const double2 rv = r[q], vv = v[q];
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(BS) k_bicg_xr(int64_t nv, const double* __rest
                                                 const double2* __restrict__ s, const double2* __restrict__ t,
                                                 const double2* __restrict__ rh, double2* __restrict__ x,
                                                 double2* __restrict__ r, double* __restrict__ partial) {
-  rf_pdl_begin();
+  rf_pdl_begin(scal, y, z, s, t, rh, x);
   const double alpha = scal[S_ALPHA], omega = scal[S_OMEGA];
   double acc[2] = {0.0, 0.0};
   for (int64_t q = blockIdx.x * (int64_t)BS + threadIdx.x; q < nv; q += (int64_t)gridDim.x * BS) {
@@ -398,7 +398,7 @@ __device__ __forceinline__ void finalize_body(int stage, int nblk, double* __res
 
 __global__ void k_finalize(int stage, int nblk, double* __restrict__ scal, const double* __restrict__ partial,
                            double rtol) {
-  rf_pdl_begin();
+  rf_pdl_begin(scal, partial);
   finalize_body(stage, nblk, scal, partial, rtol);
 }
 

@@ -97,17 +97,32 @@ __device__ __forceinline__ uint4 ld_stream_u4(const uint4* p) {
 // Neighbour values of x: kept in L1 (neighbouring threads share them) and
 // last in line for eviction from L2.  Only values this launch does not write
 // are read this way (GS reads other colours; residual / Jacobi read an input).
+// Volatile and not .nc: the preceding launch may write x until rf_pdl_begin() has
+// waited for it, so the loads may not move ahead of that, nor is x read-only for
+// as long as the kernel runs.
 __device__ __forceinline__ float2 ld_keep(const float2* p) {
   float2 v;
-  asm("ld.global.nc.L2::cache_hint.v2.f32 {%0,%1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(l2_policy_last()));
+  asm volatile("ld.global.L2::cache_hint.v2.f32 {%0,%1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(l2_policy_last()));
   return v;
 }
 __device__ __forceinline__ double2 ld_keep(const double2* p) {
   double2 v;
-  asm("ld.global.nc.L2::cache_hint.v2.f64 {%0,%1}, [%2], %3;" : "=d"(v.x), "=d"(v.y) : "l"(p), "l"(l2_policy_last()));
+  asm volatile("ld.global.L2::cache_hint.v2.f64 {%0,%1}, [%2], %3;" : "=d"(v.x), "=d"(v.y) : "l"(p), "l"(l2_policy_last()));
   return v;
 }
 #endif
+// Values that another thread of this block has just written (behind a block
+// barrier, which the load may not cross): at L2, past this SM's L1.
+__device__ __forceinline__ float2 ld_written(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.cg.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double2 ld_written(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.cg.v2.f64 {%0,%1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+  return v;
+}
 
 // Stencil blocks that reach the other x-parity run of the vertex's own x-line
 // (dx = -1, +1 with dy = dz = 0).  In a launch that sweeps a pair of colours
@@ -120,12 +135,12 @@ __host__ __device__ constexpr bool same_line_block(int b) {
 }
 template <bool SAME, int NB, typename V>
 __device__ __forceinline__ V ld_xn(const V* p, int b) {
-  if (SAME && same_line_block<NB>(b)) return __ldcg(p);
+  if (SAME && same_line_block<NB>(b)) return ld_written(p);
   return ld_keep(p);
 }
 template <bool SAME, int NB, typename V>
 __device__ __forceinline__ V ld_xn_plain(const V* p, int b) {
-  if (SAME && same_line_block<NB>(b)) return __ldcg(p);
+  if (SAME && same_line_block<NB>(b)) return ld_written(p);
   return *p;
 }
 
@@ -414,7 +429,7 @@ template <int KIND, bool FINE, int NB, int CH>
 __global__ void __launch_bounds__(CH > 0 ? 256 : 512) k_residual(LevelOp L, const typename V2<typename Ty<KIND>::T>::t* __restrict__ b,
                                                   const typename V2<typename Ty<KIND>::T>::t* __restrict__ x,
                                                   typename V2<typename Ty<KIND>::T>::t* __restrict__ r) {
-  rf_pdl_begin();
+  rf_pdl_begin(b, x);
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= L.d.nv) return;
   residual_point<KIND, FINE, NB, CH>(L, b, x, r, p);
@@ -451,7 +466,7 @@ __global__ void __launch_bounds__(CH > 0 ? 256 : 512) k_jacobi(LevelOp L, const 
                                                 const typename V2<typename Ty<KIND>::T>::t* __restrict__ xin,
                                                 typename V2<typename Ty<KIND>::T>::t* __restrict__ xout, double omega,
                                                 int zero_x) {
-  rf_pdl_begin();
+  rf_pdl_begin(b, xin);
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= L.d.nv) return;
   jacobi_point<KIND, FINE, NB, CH>(L, b, xin, xout, omega, zero_x, p);
@@ -499,7 +514,7 @@ __global__ void __launch_bounds__(CH > 0 ? 256 : 512) k_gs_colour(LevelOp L, con
                                                    typename V2<typename Ty<KIND>::T>::t* __restrict__ x, int px, int py,
                                                    int pz, int cnt_x, int lines_y, int64_t count, uint32_t skipmask,
                                                    int reverse) {
-  rf_pdl_begin();
+  rf_pdl_begin(b, x);
   // reverse: blocks take the colour's vertices from the end (see gs_zigzag)
   const int64_t bx = reverse ? (int64_t)(gridDim.x - 1 - blockIdx.x) : (int64_t)blockIdx.x;
   int64_t t = bx * blockDim.x + threadIdx.x;
@@ -536,7 +551,7 @@ __global__ void __launch_bounds__(GS_PAIR_MAX_THREADS) k_gs_pair(LevelOp L, cons
                                                   typename V2<typename Ty<KIND>::T>::t* __restrict__ x,
                                                   int py, int pz, int lines_y, int nlines, int lpb,
                                                   uint32_t skip_first, uint32_t skip_second, int reverse) {
-  rf_pdl_begin();
+  rf_pdl_begin(b, x);
   const int bx = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
   const int l0 = bx * lpb;
   const int nl = min(lpb, nlines - l0);
@@ -618,7 +633,7 @@ __global__ void __launch_bounds__(64) k_residual_small(const __grid_constant__ L
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   RowF32<NB> R;
   if (p < L.d.nv) row_load<NB, true>(L, p, 0u, R);
-  rf_pdl_begin();
+  rf_pdl_begin(b, x);
   if (p >= L.d.nv) return;
   const float2 bv = b[p];
   float s0, s1;
@@ -632,7 +647,7 @@ __global__ void __launch_bounds__(64) k_jacobi_small(const __grid_constant__ Lev
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   RowF32<NB> R;
   if (p < L.d.nv) row_load<NB, true>(L, p, 0u, R);
-  rf_pdl_begin();
+  rf_pdl_begin(b, xin);
   if (p >= L.d.nv) return;
   const float2 bv = b[p], x0 = xin[p];
   float s0, s1;
@@ -654,7 +669,7 @@ __global__ void __launch_bounds__(GS_PAIR_MAX_THREADS) k_gs_pair_small(const __g
   const int64_t p1 = on1 ? pair_vertex(L.d, l0, v, cnt1, 1 - FPX, py, pz, lines_y) : 0;
   RowF32<NB> R;
   if (on0) row_load<NB, false>(L, p0, skip_first, R);
-  rf_pdl_begin();
+  rf_pdl_begin(b, x);
   auto update = [&](int64_t p, float2 bv, float s0, float s1) {
     const float r0 = FINE ? bv.x + s0 : bv.x - s0, r1 = FINE ? bv.y + s1 : bv.y - s1;   // as gs_vertex
     x[p] = make_float2(R.d.x * r0 + R.d.y * r1, R.d.z * r0 + R.d.w * r1);
@@ -733,7 +748,7 @@ __global__ void __launch_bounds__(64) k_residual_small64(const __grid_constant__
   const int h = (int)(t & 1);
   RowF64<NB> R;
   if (p < L.d.nv) row_load<NB, true>(L, p, h, 0u, R);
-  rf_pdl_begin();
+  rf_pdl_begin(b, x);
   if (p >= L.d.nv) return;
   const double bv = reinterpret_cast<const double*>(b)[t];
   reinterpret_cast<double*>(r)[t] = bv - row_apply<NB, FINE>(L, p, h, x, R);
@@ -746,7 +761,7 @@ __global__ void __launch_bounds__(64) k_jacobi_small64(const __grid_constant__ L
   const int h = (int)(t & 1);
   RowF64<NB> R;
   if (p < L.d.nv) row_load<NB, true>(L, p, h, 0u, R);
-  rf_pdl_begin();
+  rf_pdl_begin(b, xin);
   if (p >= L.d.nv) return;
   const double bv = reinterpret_cast<const double*>(b)[t], x0 = reinterpret_cast<const double*>(xin)[t];
   const double mine = bv - row_apply<NB, FINE>(L, p, h, xin, R), other = pair_other(mine);
@@ -760,25 +775,31 @@ __global__ void __launch_bounds__(NB == 27 ? 128 : 288) k_gs_pair_small64(const 
                                                         uint32_t skip_first, uint32_t skip_second) {
   // one line per block (longer runs in several rounds)
   const int cnt0 = FPX ? L.d.nx / 2 : (L.d.nx + 1) / 2, cnt1 = FPX ? (L.d.nx + 1) / 2 : L.d.nx / 2;
-  const int h = threadIdx.x & 1;
-  auto colour = [&](auto same, int cnt, int px, uint32_t skip, bool wait) {
-    for (int v = threadIdx.x >> 1; v < cnt || wait; v += blockDim.x >> 1) {
-      const bool on = v < cnt;
-      const int64_t p = on ? pair_vertex(L.d, blockIdx.x, v, cnt, px, py, pz, lines_y) : 0;
-      RowF64<NB> R;
-      if (on) row_load<NB, false>(L, p, h, skip, R);
-      if (wait) rf_pdl_begin();
-      wait = false;
-      if (!on) break;
-      const double bv = reinterpret_cast<const double*>(b)[2 * p + h];
-      const double s = row_sum<NB, false, decltype(same)::value>(L, p, px, x, skip, R);
-      const double mine = FINE ? bv + s : bv - s, other = pair_other(mine);   // as gs_vertex
-      reinterpret_cast<double*>(x)[2 * p + h] = h ? R.d.x * other + R.d.y * mine : R.d.x * mine + R.d.y * other;
-    }
+  const int h = threadIdx.x & 1, v0 = threadIdx.x >> 1, step = blockDim.x >> 1;
+  RowF64<NB> R;
+  auto load = [&](int v, int cnt, int px, uint32_t skip) {
+    const int64_t p = pair_vertex(L.d, blockIdx.x, v, cnt, px, py, pz, lines_y);
+    row_load<NB, false>(L, p, h, skip, R);
+    return p;
   };
-  colour(std::false_type{}, cnt0, FPX, skip_first, true);
+  auto update = [&](auto same, int64_t p, int px, uint32_t skip) {
+    const double bv = reinterpret_cast<const double*>(b)[2 * p + h];
+    const double s = row_sum<NB, false, decltype(same)::value>(L, p, px, x, skip, R);
+    const double mine = FINE ? bv + s : bv - s, other = pair_other(mine);   // as gs_vertex
+    reinterpret_cast<double*>(x)[2 * p + h] = h ? R.d.x * other + R.d.y * mine : R.d.x * mine + R.d.y * other;
+  };
+  int64_t p = v0 < cnt0 ? load(v0, cnt0, FPX, skip_first) : 0;
+  rf_pdl_begin(b, x);
+  for (int v = v0; v < cnt0;) {
+    update(std::false_type{}, p, FPX, skip_first);
+    v += step;
+    if (v < cnt0) p = load(v, cnt0, FPX, skip_first);
+  }
   __syncthreads();
-  colour(std::true_type{}, cnt1, 1 - FPX, skip_second, false);
+  for (int v = v0; v < cnt1; v += step) {
+    p = load(v, cnt1, 1 - FPX, skip_second);
+    update(std::true_type{}, p, 1 - FPX, skip_second);
+  }
 }
 
 // ----------------------------------------------------------------- transfers
@@ -837,7 +858,7 @@ __global__ void __launch_bounds__(256) k_restrict(Dims df, Dims dc, const uint8_
                                                   const uint8_t* __restrict__ dmc,
                                                   const typename V2<T>::t* __restrict__ rf,
                                                   typename V2<T>::t* __restrict__ bc) {
-  rf_pdl_begin();
+  rf_pdl_begin(rf);
   int64_t pc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (pc >= dc.nv) return;
   restrict_point<T>(df, dc, dmf, dmc, rf, bc, pc);
@@ -899,7 +920,7 @@ __global__ void __launch_bounds__(256) k_prolong(Dims df, Dims dc, const uint8_t
                                                  const uint8_t* __restrict__ dmc,
                                                  const typename V2<T>::t* __restrict__ xc,
                                                  typename V2<T>::t* __restrict__ xf) {
-  rf_pdl_begin();
+  rf_pdl_begin(xc, xf);
   int64_t pf = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (pf >= df.nv) return;
   prolong_point<T>(df, dc, dmf, dmc, xc, xf, pf);
@@ -919,7 +940,7 @@ __device__ __forceinline__ void restrict_planes_body(const Dims& df, const Dims&
                                                      const uint8_t* __restrict__ dmc,
                                                      const typename V2<T>::t* __restrict__ rf,
                                                      typename V2<T>::t* __restrict__ bc) {
-  rf_pdl_begin();
+  rf_pdl_begin(rf);
   typedef typename V2<T>::t V;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= dc.nx * dc.ny) return;
@@ -999,7 +1020,7 @@ __device__ __forceinline__ void prolong_pairs_body(const Dims& df, const Dims& d
                                                    const uint8_t* __restrict__ dmc,
                                                    const typename V2<T>::t* __restrict__ xc,
                                                    typename V2<T>::t* __restrict__ xf) {
-  rf_pdl_begin();
+  rf_pdl_begin(xc, xf);
   typedef typename V2<T>::t V;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= dc.nx * df.ny) return;
@@ -1076,7 +1097,7 @@ __global__ void __launch_bounds__(256) k_prolong_planes(Dims df, Dims dc, const 
 template <typename T>
 __device__ __forceinline__ void coarse_solve_body(int N, const double* __restrict__ Ainv, const T* __restrict__ b,
                                                   T* __restrict__ x) {
-  rf_pdl_begin();
+  rf_pdl_begin(b);
   extern __shared__ double sb[];
   for (int t = threadIdx.x; t < N; t += blockDim.x) sb[t] = (double)b[t];
   __syncthreads();
@@ -2676,7 +2697,7 @@ __global__ void k_cast_f64_f32(const double* __restrict__ in, float* __restrict_
     out[t] = (float)in[t];
 }
 __global__ void k_cast_f32_f64(const float* __restrict__ in, double* __restrict__ out, int64_t n) {
-  rf_pdl_begin();
+  rf_pdl_begin(in);
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
     out[t] = (double)in[t];
 }

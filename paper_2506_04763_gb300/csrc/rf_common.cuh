@@ -115,9 +115,17 @@ bool pdl_enabled();
 // (griddepcontrol.launch_dependents takes effect once every block of this grid
 // has issued it, i.e. when its last wave is resident, so the next grid's blocks
 // only fill SMs that this grid no longer needs, and they wait in turn).
-__device__ __forceinline__ void rf_pdl_begin() {
+// Its arguments are the kernel's pointers to data that an earlier launch of the
+// solve writes.  Through a const __restrict__ parameter the compiler takes such data
+// as constant for the whole kernel and may load it ahead of the wait; a pointer that
+// an asm statement behind the wait hands back carries no such promise.
+template <typename P>
+__device__ __forceinline__ void pdl_fresh(P& ptr) { asm volatile("" : "+l"(ptr) : : "memory"); }
+template <typename... P>
+__device__ __forceinline__ void rf_pdl_begin(P&... ptr) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  (pdl_fresh(ptr), ...);
 }
 
 // launch with the programmatic-stream-serialisation attribute where `pdl` says
