@@ -44,7 +44,7 @@ namespace rf {
 struct Phys {
   double rho_w, rho_n, mu_w, mu_n, S_wr, S_nr, lam, den;
   double h[3], g[3];
-  double rh[3], rmu_w, rmu_n, rden, nid;   // 1 / h, 1 / mu_w, 1 / mu_n, 1 / den (rounded), -1 / den
+  double rh[3], rmu_w, rmu_n, rden, nid;   // recip of h, mu_w, mu_n, den; -1 / den
   double Af[3], gw[3], gn[3]; // SCV face sizes, rho_w g, rho_n g per axis
   double gt[3][3];            // w / h by axis and number of 1/4 factors in w
   int scheme;   // SCHEME_* bits (0: the discretisation of Sec. 3)
@@ -876,10 +876,10 @@ cudaError_t launch_assemble(const Dims& d, const PhysParams& pp, const AsmArrays
   ph.S_wr = pp.S_wr; ph.S_nr = pp.S_nr; ph.lam = pp.lambda;
   ph.den = 1.0 - pp.S_wr - pp.S_nr;
   ph.scheme = pp.scheme;
-  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = 1.0 / pp.h[t]; }
-  ph.rmu_w = 1.0 / pp.mu_w;
-  ph.rmu_n = 1.0 / pp.mu_n;
-  ph.rden = 1.0 / ph.den;
+  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = recip(pp.h[t]); }
+  ph.rmu_w = recip(pp.mu_w);
+  ph.rmu_n = recip(pp.mu_n);
+  ph.rden = recip(ph.den);
   ph.nid = -1.0 / ph.den;
   for (int t = 0; t < 3; ++t) {
     ph.Af[t] = 1.0;
@@ -943,10 +943,10 @@ void launch_storage_sw(const Dims& d, const PhysParams& pp, const double* u, con
   ph.S_wr = pp.S_wr; ph.S_nr = pp.S_nr; ph.lam = pp.lambda;
   ph.den = 1.0 - pp.S_wr - pp.S_nr;
   ph.scheme = pp.scheme;
-  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = 1.0 / pp.h[t]; }
-  ph.rmu_w = 1.0 / pp.mu_w;
-  ph.rmu_n = 1.0 / pp.mu_n;
-  ph.rden = 1.0 / ph.den;
+  for (int t = 0; t < 3; ++t) { ph.h[t] = pp.h[t]; ph.g[t] = pp.g[t]; ph.rh[t] = recip(pp.h[t]); }
+  ph.rmu_w = recip(pp.mu_w);
+  ph.rmu_n = recip(pp.mu_n);
+  ph.rden = recip(ph.den);
   ph.nid = -1.0 / ph.den;
   for (int t = 0; t < 3; ++t) {
     ph.Af[t] = 1.0;

@@ -2225,23 +2225,19 @@ __global__ void __launch_bounds__(256) k_pack_dinv(Dims d, bool fine, const doub
   for (int j = 0; j < out.n; ++j) {
     const double a00 = -u.x, a01 = out.shift[j] * m.x - u.y, a10 = -w.x, a11 = out.shift[j] * m.y - w.y;
     // explicit, so that the inverse does not follow the compiler's choice of which product it fuses
-    const double det = __fma_rn(a00, a11, -__dmul_rn(a01, a10)), r = 1.0 / det;
-    const uint32_t e = ((uint32_t)__double2hiint(det) >> 20) & 0x7ffu;
+    const double det = __fma_rn(a00, a11, -__dmul_rn(a01, a10)), r = recip(det);
     double q[4] = {a11, -a01, -a10, a00};
 #pragma unroll
-    for (int t = 0; t < 4; ++t) q[t] = e - 256u < 1536u ? div_by(q[t], det, r) : q[t] / det;
+    for (int t = 0; t < 4; ++t) q[t] = div_by(q[t], det, r);
     store_block(q[0], q[1], q[2], q[3], reinterpret_cast<T*>(out.Dinv[j]) + p * 4);
   }
 }
 
 // The finest level in FP16: per vertex and entry position one FP32 scale (the
 // largest magnitude over the block row), entries J / scale rounded to nearest,
-// blocks in the paired layout of stencil_sum_f16.  The quotients take one
-// Newton step on the product with the rounded reciprocal (Markstein's
-// correction: the correctly rounded quotient for normal operands, here |J| <=
-// scale; below 2^-900 of the FP64 range both round to the same half, zero): 3
-// FP64 operations (108 divisions per vertex took 2.9 ms at 129^3; the set-up
-// there went from 11.6 to 6.2 ms with this, k_galerkin and one pack for Dinv).
+// blocks in the paired layout of stencil_sum_f16.  The quotients are div_by's (108
+// divisions per vertex took 2.9 ms at 129^3; the set-up there went from 11.6 to 6.2
+// ms with this, k_galerkin and one pack for Dinv).
 __global__ void __launch_bounds__(128) k_pack_f16(Dims d, const double* __restrict__ J, uint4* __restrict__ A,
                                                   float4* __restrict__ scale) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -2268,7 +2264,7 @@ __global__ void __launch_bounds__(128) k_pack_f16(Dims d, const double* __restri
   for (int t = 0; t < 4; ++t) {
     const double v = __longlong_as_double(mx[t]);
     sc[t] = v >= 1.17549435e-38 ? (float)v : 1.0f;
-    r[t] = 1.0 / (double)sc[t];
+    r[t] = recip((double)sc[t]);
   }
   scale[p] = make_float4(sc[0], sc[1], sc[2], sc[3]);
   const int slots = (nb + 1) & ~1;
@@ -2286,8 +2282,7 @@ __global__ void __launch_bounds__(128) k_pack_f16(Dims d, const double* __restri
       __half v[4];
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        const double s64 = (double)sc[t], y0 = e[t] * r[t];
-        v[t] = __double2half(sc[t] < INFINITY ? fma(fma(-y0, s64, e[t]), r[t], y0) : e[t] / s64);
+        v[t] = __double2half(div_by(e[t], (double)sc[t], r[t]));
       }
       hw[2 * hh] = (uint32_t)__half_as_ushort(v[0]) | (uint32_t)__half_as_ushort(v[1]) << 16;
       hw[2 * hh + 1] = (uint32_t)__half_as_ushort(v[2]) | (uint32_t)__half_as_ushort(v[3]) << 16;

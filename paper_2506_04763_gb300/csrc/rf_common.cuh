@@ -81,18 +81,26 @@ inline Nbr make_nbr(const Dims& d) {
   return r;
 }
 
-// x / h given rh = 1 / h rounded to nearest: one Newton step on x * rh, the
-// correctly rounded quotient for every h when no step under- or overflows
-// (Markstein, IBM J. Res. Dev. 34 (1990); Brisebarre, Muller, Raina, IEEE
-// Trans. Comput. 53 (2004)); 3 FP64 instructions where the general division
-// has about 10.  Outside [2^-959, 2^957] it divides; zero needs no step.
+// 1 / h for div_by; NaN where h is so close to an end of the FP64 range that its
+// reciprocal is not a full-precision number (div_by then divides)
+__host__ __device__ inline double recip(double h) {
+  const double a = h < 0.0 ? -h : h;
+  return a >= 0x1p-959 && a <= 0x1p959 ? 1.0 / h : __builtin_nan("");
+}
+
+// x / h given rh = recip(h): one Newton step on x * rh, the correctly rounded
+// quotient when no step under- or overflows (Markstein, IBM J. Res. Dev. 34 (1990);
+// Brisebarre, Muller, Raina, IEEE Trans. Comput. 53 (2004)); 3 FP64 instructions
+// where the general division has about 10.  Where x or the quotient lies outside
+// [2^-959, 2^959] it divides, except for zeros, whose product has the sign.
 __device__ __forceinline__ double div_by(double x, double h, double rh) {
-  const uint32_t e = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
   const double q = __dmul_rn(x, rh);
   const double y = __fma_rn(__fma_rn(-q, h, x), rh, q);
-  if (e - 64u < 1917u) return y;
-  if ((((uint32_t)__double2hiint(x) << 1) | (uint32_t)__double2loint(x)) == 0u) return y;
-  return __ddiv_rn(x, h);
+  const uint32_t ex = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu, eq = ((uint32_t)__double2hiint(q) >> 20) & 0x7ffu;
+  if (ex - 64u < 1919u && eq - 64u < 1919u) return y;
+  const uint32_t zx = ((uint32_t)__double2hiint(x) << 1) | (uint32_t)__double2loint(x);
+  const uint32_t zq = ((uint32_t)__double2hiint(q) << 1) | (uint32_t)__double2loint(q);
+  return (zx | zq) == 0u ? q : __ddiv_rn(x, h);
 }
 
 // halo of a padded vector (in pairs), rounded for alignment
