@@ -1,5 +1,5 @@
 // cluster_plan.h — the cluster size a kernel is launched with whose CTAs take
-// most of an SM's shared memory (k_gauss_jordan, k_vcycle_cl).  Host code only,
+// most of an SM's shared memory (k_lu_cluster, k_vcycle_cl).  Host code only,
 // the CUDA calls behind `Api`.
 //
 // Api (of one kernel, on the current device):
@@ -38,15 +38,18 @@ class ClusterAnswers {
 
 // The first of `sizes` whose CTAs' shared memory (smem(cs)) fits the device and of
 // which a cluster can run; 0: none, the caller takes a kernel without a cluster.
-// Function attributes belong to a device, so they are set at every call.
+// Function attributes belong to a device, so they are set on each one that asks,
+// before its first query.
 template <class Api, class Smem>
 int choose_cluster(Api&& api, ClusterAnswers& known, int kernel, const std::vector<int>& sizes, Smem smem) {
   const int dev = api.device();
   const size_t cap = dev < 0 ? 0 : api.smem_optin();
-  if (cap == 0 || !api.allow(cap)) return 0;
+  if (cap == 0) return 0;
   for (const int cs : sizes) {
     const size_t bytes = smem(cs);
-    if (bytes <= cap && known.fits({dev, kernel, cs, (long long)bytes}, [&] { return api.clusters(cs, bytes); })) return cs;
+    if (bytes <= cap && known.fits({dev, kernel, cs, (long long)bytes},
+                                   [&] { return api.allow(cap) ? api.clusters(cs, bytes) : -1; }))
+      return cs;
   }
   return 0;
 }

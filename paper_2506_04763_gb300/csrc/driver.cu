@@ -1113,7 +1113,7 @@ extern "C" rf_status rf_gmg_setup(rf_grid* g, const double* shifts, int nshift, 
     const Level& C = g->L[g->nl - 1];
     const int N = (int)(2 * C.d.nv);
     if (N > 4096) { drop_hierarchy(g, s); return fail(RF_EINVAL, "coarsest level too large (%d unknowns): use more levels", N); }
-    // all shifts at once: one LU per CTA, the inverse columns of every shift in one grid
+    // all shifts at once: one LU per cluster, the inverse columns of every shift in one grid
     double* D;
     int* piv;
     int* status;

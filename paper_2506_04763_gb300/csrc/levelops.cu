@@ -2322,159 +2322,174 @@ __global__ void k_dense(Dims d, Nbr nb, const double* __restrict__ J, const doub
   D[(2 * p + 1) * N + 2 * q + 1] = e3;
 }
 
-// Inverse by in-place Gauss-Jordan elimination with partial pivoting, one
-// thread-block cluster per matrix: CTA r of the cluster keeps rows r, r + cs,
-// ... in shared memory, and every step costs one cluster barrier.  Step c:
+// LU factors with partial pivoting, one thread-block cluster per matrix: CTA r of
+// the cluster keeps rows r, r + cs, ... in shared memory, and every step costs one
+// cluster barrier.  Rows are not swapped; pos and at hold the order that swapping
+// would give (the position of a row, the row at a position).  Step c:
 //   - each CTA's first warp picks its largest |A[row][c]| over rows not yet
-//     used as pivots (the candidates were left by the previous update) and
-//     puts it, its row and its reciprocal into every CTA's table;
-//   - after the barrier all take the largest (the smaller row on ties) and
-//     copy the pivot row from its owner through distributed shared memory;
-//   - every other row: l = A[row][c] / pivot, A[row][t] -= l A[pivot][t], and
-//     A[row][c] = -l; one warp per row.  The pivot row itself is scaled by its
-//     owner one step later, when no one reads it any more.
-// Rows are never swapped: with pi(c) the pivot row of step c, the inverse is
-// Ainv[c][pi(t)] = B[pi(c)][t] of the final array B.  A pivot that is zero or
-// not finite, or a non-finite entry in the result (any NaN of A ends there),
-// sets status.
-// The one-CTA LU below does its N^3 / 3 multiply-adds on one SM's FP64 pipe (2
-// per clock) with four block barriers per column: 4.5 ms + 0.78 ms for the
-// inverse columns at N = 250 (5^3 vertices), 0.40 + 0.11 ms at N = 50 (5^2).
-// Spread over a cluster: 1.1 ms at N = 250, 0.10 ms at N = 50; what is left is
-// the step's chain of barrier, table, row copy and FP64 latencies (2 of 4.4 us
-// at N = 250).
-constexpr int GJ_THREADS = 512, GJ_MAX_CS = 16;
+//     used as pivots (the candidates were left by the previous update; the
+//     earlier position on ties) and puts it and its row into every CTA's table;
+//   - after the barrier all take the largest; the first warp computes the
+//     multipliers l = A[row][c] / pivot of the CTA's rows, a lane each, while the
+//     others copy the pivot row from column c on from its owner through distributed
+//     shared memory;
+//   - every unused row: A[row][t] -= l A[pivot][t] for t > c, and l in the place of
+//     A[row][c]; one warp per row.
+// The factors go to D in the order of the positions, the rows at them to piv.  A
+// pivot that is zero or not finite, or a multiplier that is not finite (any NaN
+// of A ends in one of these), sets status.
+// Each operation is k_lu's, so are the factors, to the last bit.  (Gauss-Jordan
+// elimination in the same place needs no substitution afterwards, but its sums run
+// over whole columns one term after another: against a reference in 113 bits, on the
+// coarsest operators of 129^3, 65^3 and 161 x 97 x 65 grids, the inverse's largest error
+// was 1.1 to 5 times that of LU and substitution, whose sums are 32 lanes' partial
+// sums.)
+// The one-CTA k_lu does its N^3 / 3 multiply-adds on one SM's FP64 pipe (2 per
+// clock) with four block barriers per column: 4.5 ms at N = 250 (5^3 vertices), 0.40
+// ms at N = 50 (5^2).  Spread over a cluster: 0.68 ms and 0.09 ms, 2.7 and 1.8 us a
+// step, most of it the chain of barrier, table, reciprocal and row copy.
+constexpr int LU_THREADS = 512, LU_MAX_CS = 16;
 
-struct GjShared {
-  long long key[2][GJ_MAX_CS];   // bits of |candidate|, -1: none (as integers: no FP64-pipe comparisons)
-  double inv[2][GJ_MAX_CS];
-  int row[2][GJ_MAX_CS];
+struct LuShared {
+  unsigned long long key[2][LU_MAX_CS];   // bits of |candidate| (as integers: no FP64-pipe comparisons)
+  double val[2][LU_MAX_CS];
+  int row[2][LU_MAX_CS];
 };
 
-__host__ __device__ inline size_t gj_smem(int N, int cs) {
+__host__ __device__ inline size_t lu_smem(int N, int cs) {
   const int rows = (N + cs - 1) / cs;
-  return sizeof(GjShared) + sizeof(double) * ((size_t)rows * N + N) + sizeof(long long) * rows +
-         sizeof(int) * (size_t)(N + rows + 2);
+  return sizeof(LuShared) + sizeof(double) * ((size_t)rows * N + N + 2 * (size_t)rows) +
+         sizeof(int) * (2 * (size_t)N + rows + 2);
 }
 
-__device__ __forceinline__ long long gj_key(double v) {
-  const long long k = __double_as_longlong(fabs(v));
-  return k > 0x7ff0000000000000LL ? -1 : k;   // NaN: never a pivot
+__device__ __forceinline__ unsigned long long lu_key(double v) {
+  const unsigned long long k = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+  return k > 0x7ff0000000000000ULL ? 0 : k;   // NaN: never a pivot
 }
 
-__global__ void __launch_bounds__(GJ_THREADS) k_gauss_jordan(int N, const double* __restrict__ D, InvOut out,
-                                                             int* __restrict__ status) {
+// Whether this lane of a warp holds the largest key, the lowest position among
+// equals (positions differ)
+__device__ __forceinline__ bool lu_largest(unsigned long long k, unsigned pos) {
+  const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
+  // (every lane takes part in all three reductions)
+  const unsigned top = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned low = __reduce_max_sync(0xffffffffu, hi == top ? lo : 0u);
+  const bool mine = hi == top && lo == low;
+  const unsigned first = __reduce_min_sync(0xffffffffu, mine ? pos : ~0u);
+  return mine && pos == first;
+}
+
+__global__ void __launch_bounds__(LU_THREADS) k_lu_cluster(int N, double* __restrict__ D, int* __restrict__ piv,
+                                                           int* __restrict__ status) {
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank(), mat = blockIdx.x / cs;
   const int rows = (N + cs - 1) / cs, nloc = (N - rank + cs - 1) / cs;
-  extern __shared__ __align__(16) unsigned char gj_raw[];
-  GjShared& T = *reinterpret_cast<GjShared*>(gj_raw);
-  double* A = reinterpret_cast<double*>(gj_raw + sizeof(GjShared));   // [rows][N]
+  extern __shared__ __align__(16) unsigned char lu_raw[];
+  LuShared& T = *reinterpret_cast<LuShared*>(lu_raw);
+  double* A = reinterpret_cast<double*>(lu_raw + sizeof(LuShared));   // [rows][N]
   double* prow = A + (size_t)rows * N;
-  long long* cand = reinterpret_cast<long long*>(prow + N);           // [rows]
-  int* perm = reinterpret_cast<int*>(cand + rows);                    // [N]: pivot row of each step
-  int* step = perm + N;                                               // [rows]: step a local row was pivot of, or -1
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = GJ_THREADS >> 5;
+  double* mult = prow + N;                                            // [rows]
+  unsigned long long* cand = reinterpret_cast<unsigned long long*>(mult + rows);   // [rows]: 0 once used
+  int* pos = reinterpret_cast<int*>(cand + rows);                     // [N]
+  int* at = pos + N;                                                  // [N]
+  int* step = at + N;                                                 // [rows]: step a local row was pivot of, or -1
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = LU_THREADS >> 5;
   D += (int64_t)mat * N * N;
   for (int lr = warp; lr < nloc; lr += nw) {
     const double* src = D + (int64_t)(lr * cs + rank) * N;
     for (int t = lane; t < N; t += 32) {
       const double v = src[t];
       A[lr * N + t] = v;
-      if (t == 0) { cand[lr] = gj_key(v); step[lr] = -1; }
+      if (t == 0) { cand[lr] = lu_key(v); step[lr] = -1; }
     }
   }
+  for (int t = tid; t < N; t += LU_THREADS) { pos[t] = t; at[t] = t; }
   cl.sync();   // every CTA of the cluster runs before a peer writes into its table
-  int pend = -1, pend_c = 0;      // the local row waiting for its scaling, its step and reciprocal pivot
-  double pend_inv = 0.0;
-  bool bad = false;
+  bool bad = false, finite = true;
   for (int c = 0; c < N; ++c) {
     const int par = c & 1;
     __syncthreads();
     if (warp == 0) {
-      long long k = -1;
-      int r = N;
-      for (int lr = lane; lr < nloc; lr += 32)
-        if (cand[lr] > k) { k = cand[lr]; r = lr; }      // ascending rows: the first of equals stays
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long ok = __shfl_xor_sync(0xffffffffu, k, o);
-        const int orow = __shfl_xor_sync(0xffffffffu, r, o);
-        if (ok > k || (ok == k && orow < r)) { k = ok; r = orow; }
+      unsigned long long k = 0;
+      int r = 0;
+      unsigned p = N + lane;                             // (no candidate: key 0)
+      for (int lr = lane; lr < nloc; lr += 32) {
+        const unsigned long long kr = cand[lr];
+        const unsigned q = (unsigned)pos[lr * cs + rank];
+        if (kr > k || (kr == k && kr != 0 && q < p)) { k = kr; r = lr; p = q; }
       }
-      const double inv = k > 0 ? 1.0 / A[r * N + c] : 0.0;
+      const int src = __ffs(__ballot_sync(0xffffffffu, lu_largest(k, p))) - 1;
+      k = __shfl_sync(0xffffffffu, k, src);
+      r = __shfl_sync(0xffffffffu, r, src);
       if (lane < cs) {
-        GjShared& O = *cl.map_shared_rank(&T, lane);
+        LuShared& O = *cl.map_shared_rank(&T, lane);
         O.key[par][rank] = k;
-        O.inv[par][rank] = inv;
-        O.row[par][rank] = k >= 0 ? r * cs + rank : N;
+        O.val[par][rank] = nloc > 0 ? A[r * N + c] : 0.0;
+        O.row[par][rank] = nloc > 0 ? r * cs + rank : 0;
       }
     }
     cl.sync();
-    long long k = -1;
-    int pr = N;
-    double inv = 0.0;
-#pragma unroll
-    for (int q = 0; q < GJ_MAX_CS; ++q) {
-      if (q >= cs) break;
-      const long long kq = T.key[par][q];
-      const int rq = T.row[par][q];
-      if (kq > k || (kq == k && rq < pr)) { k = kq; pr = rq; inv = T.inv[par][q]; }
-    }
-    if (k <= 0 || k >= 0x7ff0000000000000LL) { bad = true; break; }   // the same decision in every CTA
+    const unsigned long long kq = lane < cs ? T.key[par][lane] : 0;
+    const int rq = lane < cs ? T.row[par][lane] : 0;
+    const unsigned pq = kq != 0 ? (unsigned)pos[rq] : (unsigned)(N + lane);
+    const int best = __ffs(__ballot_sync(0xffffffffu, lu_largest(kq, pq))) - 1;
+    const unsigned long long k = __shfl_sync(0xffffffffu, kq, best);
+    if (k == 0 || k >= 0x7ff0000000000000ULL) { bad = true; break; }   // the same decision in every CTA
+    const int pr = __shfl_sync(0xffffffffu, rq, best), p = (int)__shfl_sync(0xffffffffu, pq, best);
     const int owner = pr % cs, plr = pr / cs;
-    const double* src = cl.map_shared_rank(A, owner) + plr * N;
-    for (int t = tid; t < N; t += GJ_THREADS) prow[t] = src[t];
-    if (tid == 0) perm[c] = pr;
+    if (warp == 0) {
+      // (the general division leaves its fast path for a zero, of which there are many)
+      const double pv = T.val[par][best], inv = recip(pv);
+      for (int lr = lane; lr < nloc; lr += 32) {
+        const double l = div_by(A[lr * N + c], pv, inv);
+        mult[lr] = l;
+        if (step[lr] < 0 && !(rank == owner && lr == plr))
+          finite = finite && ((__double2hiint(l) & 0x7ff00000) != 0x7ff00000);
+      }
+    } else {
+      const double* src = cl.map_shared_rank(A, owner) + plr * N;
+      for (int t = c + tid - 32; t < N; t += LU_THREADS - 32) prow[t] = src[t];
+    }
     __syncthreads();
+    if (tid == 0) {                     // (read again behind the next block barrier)
+      const int q = at[c];
+      at[c] = pr;
+      at[p] = q;
+      pos[q] = p;
+      pos[pr] = c;
+    }
     for (int lr = warp; lr < nloc; lr += nw) {
       if (rank == owner && lr == plr) {
-        if (lane == 0) { cand[lr] = -1; step[lr] = c; }
+        if (lane == 0) { step[lr] = c; cand[lr] = 0; }
         continue;
       }
+      if (step[lr] >= 0) continue;
       double* a = A + lr * N;
-      if (lr == pend) {
-        for (int t = lane; t < N; t += 32) a[t] = t == pend_c ? pend_inv : a[t] * pend_inv;
-        __syncwarp();
-      }
-      const double l = a[c] * inv;
-      __syncwarp();
-      const bool used = step[lr] >= 0;
-      for (int t = lane; t < N; t += 32) {
-        const double v = t == c ? -l : fma(-l, prow[t], a[t]);
+      const double l = mult[lr];
+      if (lane == 0) a[c] = l;
+#pragma unroll 2
+      for (int t = c + 1 + lane; t < N; t += 32) {
+        const double v = __fma_rn(-l, prow[t], a[t]);
         a[t] = v;
-        if (t == c + 1) cand[lr] = used ? -1 : gj_key(v);
+        if (t == c + 1) cand[lr] = lu_key(v);
       }
     }
-    pend = rank == owner ? plr : -1;
-    pend_c = c;
-    pend_inv = inv;
   }
-  cl.sync();   // no CTA leaves, or scales its last pivot row, while its rows are read
-  if (bad) {
-    if (tid == 0) status[mat] = 1;
-    return;
-  }
-  if (pend >= 0 && warp == 0)
-    for (int t = lane; t < N; t += 32) A[pend * N + t] = t == pend_c ? pend_inv : A[pend * N + t] * pend_inv;
-  __syncthreads();
-  double* __restrict__ Ainv = out.Ainv[mat];
-  bool finite = true;
+  cl.sync();   // no CTA leaves while its rows are read
+  if (bad || !finite) status[mat] = 1;
+  if (bad) return;
   for (int lr = warp; lr < nloc; lr += nw) {
-    double* dst = Ainv + (int64_t)step[lr] * N;
-    for (int t = lane; t < N; t += 32) {
-      const double v = A[lr * N + t];
-      finite = finite && ((__double2hiint(v) & 0x7ff00000) != 0x7ff00000);
-      dst[perm[t]] = v;
-    }
+    double* dst = D + (int64_t)step[lr] * N;
+    for (int t = lane; t < N; t += 32) dst[t] = A[lr * N + t];
   }
-  if (!finite) status[mat] = 1;
+  if (rank == 0)
+    for (int t = tid; t < N; t += LU_THREADS) piv[(int64_t)mat * N + t] = at[t];
 }
 
-static cudaLaunchConfig_t gj_config(int nmat, int cs, size_t smem, void* s, cudaLaunchAttribute* attr) {
+static cudaLaunchConfig_t lu_config(int nmat, int cs, size_t smem, void* s, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cs * nmat, 1, 1);
-  cfg.blockDim = dim3(GJ_THREADS, 1, 1);
+  cfg.blockDim = dim3(LU_THREADS, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = (cudaStream_t)s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2486,29 +2501,28 @@ static cudaLaunchConfig_t gj_config(int nmat, int cs, size_t smem, void* s, cuda
   return cfg;
 }
 
-// Cluster size of k_gauss_jordan for N unknowns (0: it does not fit).  A step's
-// update takes N ceil(N / cs) multiply-adds of a CTA, its barrier and copies
-// grow with cs.  Measured for one inverse, cs = 1 / 4 / 8 / 16 (the call's 40 us
-// of launch and read-back included): N = 50 205 / 135 / 137 / 152 us, N = 90
-// 524 / 280 / 245 / 271, N = 126 1068 / 461 / 386 / 406, N = 144 1522 / 637 /
-// 523 / 488, N = 250 - / - / 1298 / 1131.  A size that the device refuses is
-// passed over: each gives the same inverse, bit for bit.
-static int gj_cluster(int N) {
+// Cluster size of k_lu_cluster for N unknowns (0: none).  A step's update takes
+// N ceil(N / cs) multiply-adds of a CTA, its barrier and copies grow with cs.
+// Measured for one inverse, cs = 4 / 8 / 16 (the call's 40 us of launch and
+// read-back included): N = 50 170 / 169 / 180 us, N = 90 329 / 303 / 315, N = 126 516 /
+// 452 / 452, N = 144 700 / 551 / 525, N = 250 1804 / 1263 / 1092.  A size that the
+// device refuses is passed over: each gives the same factors, bit for bit.
+static int lu_cluster(int N) {
   std::vector<int> sizes;
-  const int first = N <= 50 ? 4 : N < 144 ? 8 : GJ_MAX_CS;
-  for (int cs = first; cs <= GJ_MAX_CS; cs *= 2) sizes.push_back(cs);
+  const int first = N <= 50 ? 4 : N < 144 ? 8 : LU_MAX_CS;
+  for (int cs = first; cs <= LU_MAX_CS; cs *= 2) sizes.push_back(cs);
   for (int cs = first / 2; cs >= 1; cs /= 2) sizes.push_back(cs);
   return choose_cluster_of(
-      k_gauss_jordan, 0, sizes,
-      [](int cs, size_t smem, cudaLaunchAttribute* attr) { return gj_config(1, cs, smem, nullptr, attr); },
-      [&](int cs) { return gj_smem(N, cs); });
+      k_lu_cluster, 0, sizes,
+      [](int cs, size_t smem, cudaLaunchAttribute* attr) { return lu_config(1, cs, smem, nullptr, attr); },
+      [&](int cs) { return lu_smem(N, cs); });
 }
 
-static cudaError_t launch_gauss_jordan(int N, int nmat, int cs, const double* D, const InvOut& out, int* status, void* s) {
+static cudaError_t launch_lu_cluster(int N, int nmat, int cs, double* D, int* piv, int* status, void* s) {
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = gj_config(nmat, cs, gj_smem(N, cs), s, attr);
+  cudaLaunchConfig_t cfg = lu_config(nmat, cs, lu_smem(N, cs), s, attr);
   count_launch();
-  return cudaLaunchKernelEx(&cfg, k_gauss_jordan, N, D, out, status);
+  return cudaLaunchKernelEx(&cfg, k_lu_cluster, N, D, piv, status);
 }
 
 // LU with partial pivoting in one CTA (first maximal pivot on ties).  Per
@@ -2620,7 +2634,7 @@ __global__ void __launch_bounds__(128) k_lu_inverse_cols(int N, const double* __
   for (int r = 1; r < N; ++r) {
     const double* Lr = LU + (int64_t)r * N;
     double s = 0.0;
-    for (int c = lane; c < r; c += 32) s += Lr[c] * x[c];
+    for (int c = lane; c < r; c += 32) s = __fma_rn(Lr[c], x[c], s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) x[r] -= s;
@@ -2629,11 +2643,86 @@ __global__ void __launch_bounds__(128) k_lu_inverse_cols(int N, const double* __
   for (int r = N - 1; r >= 0; --r) {
     const double* Ur = LU + (int64_t)r * N;
     double s = 0.0;
-    for (int c = r + 1 + lane; c < N; c += 32) s += Ur[c] * x[c];
+    for (int c = r + 1 + lane; c < N; c += 32) s = __fma_rn(Ur[c], x[c], s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) x[r] = (x[r] - s) / Ur[r];
     __syncwarp();
+  }
+  for (int r = lane; r < N; r += 32) Ainv[(int64_t)r * N + col] = x[r];
+}
+
+// The same, of the same operations, for the factors of k_lu_cluster (N <= ~650).  A
+// row costs its chain of latencies, 2 N rows in turn with few warps in flight: the
+// rows ahead are copied to shared memory (cp.async) while one is summed, and the
+// division by a pivot is one Newton step on its reciprocal.  0.39 ms at N = 250 and
+// 0.06 ms at N = 50, where k_lu_inverse_cols takes 0.78 and 0.11 ms.
+constexpr int LU_AHEAD = 4;   // row buffers per warp
+
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+__host__ __device__ inline size_t lu_ahead_smem(int N, int warps) {
+  return sizeof(double) * ((size_t)warps * (LU_AHEAD + 1) + 2) * N;
+}
+
+__global__ void __launch_bounds__(128) k_lu_inverse_ahead(int N, const double* __restrict__ LU,
+                                                          const int* __restrict__ piv, InvOut out) {
+  LU += (int64_t)blockIdx.y * N * N;
+  piv += (int64_t)blockIdx.y * N;
+  double* __restrict__ Ainv = out.Ainv[blockIdx.y];
+  extern __shared__ double la_raw[];
+  double* diag = la_raw;                 // the pivots and their reciprocals
+  double* rdiag = diag + N;
+  for (int r = threadIdx.x; r < N; r += blockDim.x) {
+    const double d = LU[(int64_t)r * N + r];
+    diag[r] = d;
+    rdiag[r] = recip(d);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int col = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (col >= N) return;
+  double* x = rdiag + N + (int64_t)warp * (LU_AHEAD + 1) * N;
+  double* buf = x + N;                   // row r in buffer r % LU_AHEAD
+  auto ahead = [&](int r, int c0, int c1) {   // columns [c0, c1) of row r (none: an empty group)
+#pragma unroll 1
+    for (int c = c0 + lane; c < c1; c += 32) cp_async8(buf + (r & (LU_AHEAD - 1)) * N + c, LU + (int64_t)r * N + c);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto dot = [&](int r, int c0, int c1) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(LU_AHEAD - 2) : "memory");   // row r has arrived
+    __syncwarp();
+    const double* row = buf + (r & (LU_AHEAD - 1)) * N;
+    double s = 0.0;
+#pragma unroll 1
+    for (int c = c0 + lane; c < c1; c += 32) s = __fma_rn(row[c], x[c], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  };
+  for (int r = lane; r < N; r += 32) x[r] = piv[r] == col ? 1.0 : 0.0;
+#pragma unroll 1
+  for (int r = 1; r < LU_AHEAD; ++r) ahead(r, 0, r < N ? r : 0);
+#pragma unroll 1
+  for (int r = 1; r < N; ++r) {
+    const double s = dot(r, 0, r);
+    if (lane == 0) x[r] -= s;
+    __syncwarp();                        // (also: no lane reads this row's buffer any more)
+    ahead(r + LU_AHEAD - 1, 0, r + LU_AHEAD - 1 < N ? r + LU_AHEAD - 1 : 0);
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+#pragma unroll 1
+  for (int k = 0; k < LU_AHEAD - 1; ++k) ahead(N - 1 - k, N - k, N - 1 - k >= 0 ? N : N - k);
+#pragma unroll 1
+  for (int r = N - 1; r >= 0; --r) {
+    const double s = dot(r, r + 1, N);
+    if (lane == 0) x[r] = div_by(x[r] - s, diag[r], rdiag[r]);
+    __syncwarp();
+    ahead(r - LU_AHEAD + 1, r - LU_AHEAD + 2, r - LU_AHEAD + 1 >= 0 ? N : r - LU_AHEAD + 2);
   }
   for (int r = lane; r < N; r += 32) Ainv[(int64_t)r * N + col] = x[r];
 }
@@ -3572,14 +3661,29 @@ cudaError_t launch_dense_inverse_batched(int N, int nmat, double* D, double* con
   if (nmat < 1 || nmat > RF_MAXSHIFT) return cudaErrorInvalidValue;
   InvOut out;
   for (int j = 0; j < RF_MAXSHIFT; ++j) out.Ainv[j] = j < nmat ? Ainv[j] : nullptr;
-  if (const int cs = gj_cluster(N)) return launch_gauss_jordan(N, nmat, cs, D, out, status, s);
-  // beyond a cluster's shared memory (N > ~650): LU in global memory
-  const size_t lsm = sizeof(double) * 2 * (size_t)N;   // 64 KB at N = 4096
-  cudaFuncSetAttribute(k_lu, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
-  RF_LAUNCH(k_lu, nmat, 1024, lsm, s, N, D, piv, status);
+  // k_lu in global memory serves N beyond a cluster's shared memory (N > ~650),
+  // devices that run no such cluster, and comparisons (RF_LU_CLUSTER=0, read per call)
+  const char* env = getenv("RF_LU_CLUSTER");
+  const int cs = env && atoi(env) == 0 ? 0 : lu_cluster(N);
+  if (cs > 0) {
+    const cudaError_t e = launch_lu_cluster(N, nmat, cs, D, piv, status, s);
+    if (e != cudaSuccess) return e;
+  } else {
+    const size_t lsm = sizeof(double) * 2 * (size_t)N;   // 64 KB at N = 4096
+    cudaFuncSetAttribute(k_lu, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
+    RF_LAUNCH(k_lu, nmat, 1024, lsm, s, N, D, piv, status);
+  }
+  const dim3 grid((N + 3) / 4, nmat);
+  if (cs > 0) {
+    const size_t bytes = lu_ahead_smem(N, 4);            // 114 KB at N = 650
+    if (bytes > 48 * 1024)
+      cudaFuncSetAttribute(k_lu_inverse_ahead, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    RF_LAUNCH(k_lu_inverse_ahead, grid, 128, bytes, s, N, D, piv, out);
+    return cudaGetLastError();
+  }
   const size_t smem = sizeof(double) * 4 * (size_t)N;   // 4 warps per block, one x each (128 KB at N = 4096)
   cudaFuncSetAttribute(k_lu_inverse_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  RF_LAUNCH(k_lu_inverse_cols, dim3((N + 3) / 4, nmat), 128, smem, s, N, D, piv, out);
+  RF_LAUNCH(k_lu_inverse_cols, grid, 128, smem, s, N, D, piv, out);
   return cudaGetLastError();
 }
 

@@ -84,8 +84,14 @@ inline Nbr make_nbr(const Dims& d) {
 // 1 / h for div_by; NaN where h is so close to an end of the FP64 range that its
 // reciprocal is not a full-precision number (div_by then divides)
 __host__ __device__ inline double recip(double h) {
+#ifdef __CUDA_ARCH__
+  const uint32_t e = ((uint32_t)__double2hiint(h) >> 20) & 0x7ffu;   // (comparisons issue on the FP64 pipe)
+  const bool ok = e - 64u < 1919u;
+#else
   const double a = h < 0.0 ? -h : h;
-  return a >= 0x1p-959 && a <= 0x1p959 ? 1.0 / h : __builtin_nan("");
+  const bool ok = a >= 0x1p-959 && a < 0x1p960;
+#endif
+  return ok ? 1.0 / h : __builtin_nan("");
 }
 
 // x / h given rh = recip(h): one Newton step on x * rh, the correctly rounded
@@ -100,7 +106,10 @@ __device__ __forceinline__ double div_by(double x, double h, double rh) {
   if (ex - 64u < 1919u && eq - 64u < 1919u) return y;
   const uint32_t zx = ((uint32_t)__double2hiint(x) << 1) | (uint32_t)__double2loint(x);
   const uint32_t zq = ((uint32_t)__double2hiint(q) << 1) | (uint32_t)__double2loint(q);
-  return (zx | zq) == 0u ? q : __ddiv_rn(x, h);
+  if ((zx | zq) == 0u) return q;
+  double z;   // (volatile: not computed for zeros beside the product and dropped)
+  asm volatile("div.rn.f64 %0, %1, %2;" : "=d"(z) : "d"(x), "d"(h));
+  return z;
 }
 
 // halo of a padded vector (in pairs), rounded for alignment

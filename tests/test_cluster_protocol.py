@@ -60,7 +60,7 @@ def _events(body):
 
 
 def test_there_are_cluster_kernels():
-    assert {"k_vcycle_cl", "k_gauss_jordan"} <= {k for k, _ in _kernels()}
+    assert {"k_vcycle_cl", "k_lu_cluster"} <= {k for k, _ in _kernels()}
 
 
 @pytest.mark.parametrize("name,body", _kernels(), ids=[k for k, _ in _kernels()])
