@@ -118,8 +118,9 @@ struct Level {
 //     against 1.93 ms with two).
 static void default_shape(Level& Lv, int kind, int smoother) {
   const int64_t nv = Lv.d.nv;
+  const char* env = getenv("RF_SMALL_NV");   // the limit in vertices, read per set-up (0: the plain kernels on every level)
   Lv.block = 128;
-  Lv.small = nv <= 40000;
+  Lv.small = nv <= (env ? atoll(env) : 40000);
   Lv.batched = kind == STORE_F32 || (kind == STORE_F64 && nv <= (smoother == RF_SMOOTH_GS8 ? 400000 : 100000)) ||
                (kind == STORE_F16 && Lv.small);
 }
