@@ -189,19 +189,32 @@ __device__ __forceinline__ void load_block(const void* A, int64_t nv, int b, int
   unpack_block<KIND>(r, sc, a);
 }
 
-// Row sum += (a_0 x_0 + a_1 x_1) for one block row, in explicit operations, so
+// A row's sum of a_0 x_0 + a_1 x_1 over its blocks, in explicit operations, so
 // that every kernel applying a block (per-block, batched, shared-matrix) rounds
 // it identically, whatever the compiler would otherwise contract.  FP32: one
-// product, one multiply-add, one sum (a chain of one add per block).  FP64: two
-// multiply-adds, as these kernels are bound by the FP64 pipe (65^3 Jacobi: 104 us
-// a sweep with three operations per pair, 70 us with two; its 108 multiply-adds
-// per vertex take 56 us).
-__device__ __forceinline__ float blk_acc(float s, float a0, float a1, float2 x) {
-  return __fadd_rn(s, __fmaf_rn(a0, x.x, __fmul_rn(a1, x.y)));
-}
-__device__ __forceinline__ double blk_acc(double s, double a0, double a1, double2 x) {
-  return __fma_rn(a0, x.x, __fma_rn(a1, x.y, s));
-}
+// product, one multiply-add, one sum per block (a chain of one add per block).
+// FP64: a multiply-add for each of two sums, of the a_0 x_0 and of the a_1 x_1, added
+// at the end, as these kernels are bound by the FP64 pipe (65^3 Jacobi: 104 us a sweep
+// with three operations per block, 70 us with two; its 108 multiply-adds per vertex
+// take 56 us).  One sum through both products rounds twice as long a chain: its mean
+// error against 113 bits, in units of sum |a x|, is 9.2e-17 at 17^3 and 6.6e-17 at
+// 33 x 17, with two sums 6.8e-17 and 5.2e-17 (the three operations: 7.2e-17, 6.0e-17).
+template <typename T> struct RowAcc;
+template <> struct RowAcc<float> {
+  float s = 0.f;
+  __device__ __forceinline__ void add(float a0, float a1, float2 x) {
+    s = __fadd_rn(s, __fmaf_rn(a0, x.x, __fmul_rn(a1, x.y)));
+  }
+  __device__ __forceinline__ float value() const { return s; }
+};
+template <> struct RowAcc<double> {
+  double u = 0.0, v = 0.0;
+  __device__ __forceinline__ void add(double a0, double a1, double2 x) {
+    u = __fma_rn(a0, x.x, u);
+    v = __fma_rn(a1, x.y, v);
+  }
+  __device__ __forceinline__ double value() const { return __dadd_rn(u, v); }
+};
 
 // FP16 storage holds the blocks of a row in pairs, one 16-byte load per pair
 // (a warp reads 512 contiguous bytes per load, as with FP32 blocks): slot s
@@ -243,7 +256,7 @@ __device__ __forceinline__ void f16_half(const uint4& u, int h, const float4& sc
 
 // The FP16 stencil sum, slot by slot: CP pairs (2 CP blocks) and their x values
 // loaded per memory round trip, then summed.  Per-block, batched and
-// shared-matrix FP16 kernels all sum in this slot order with blk_acc.
+// shared-matrix FP16 kernels all sum in this slot order with RowAcc.
 template <int NB, int CP, bool SAME = false>
 __device__ __forceinline__ void stencil_sum_f16(const LevelOp& L, int64_t p, int par,
                                                 const float2* __restrict__ x, bool skip_centre, uint32_t skipmask,
@@ -251,7 +264,7 @@ __device__ __forceinline__ void stencil_sum_f16(const LevelOp& L, int64_t p, int
   constexpr int C = NB == 27 ? 13 : 4, NP = (NB + 1) / 2;
   const float4 sc = reinterpret_cast<const float4*>(L.scale)[p];
   const uint4* __restrict__ A = reinterpret_cast<const uint4*>(L.A);
-  float a0 = 0.f, a1 = 0.f;
+  RowAcc<float> a0, a1;
 #pragma unroll
   for (int q0 = 0; q0 < NP; q0 += CP) {
     uint4 raw[CP];
@@ -281,12 +294,13 @@ __device__ __forceinline__ void stencil_sum_f16(const LevelOp& L, int64_t p, int
         if (!use[c][h]) continue;
         float a[4];
         f16_half(raw[c], h, sc, a);
-        a0 = blk_acc(a0, a[0], a[1], xv[c][h]);
-        a1 = blk_acc(a1, a[2], a[3], xv[c][h]);
+        a0.add(a[0], a[1], xv[c][h]);
+        a1.add(a[2], a[3], xv[c][h]);
       }
     }
   }
-  s0 = a0; s1 = a1;
+  s0 = a0.value();
+  s1 = a1.value();
 }
 
 // sum over the stencil of blocks * x (centre optionally skipped)
@@ -299,7 +313,7 @@ __device__ __forceinline__ void stencil_sum(const LevelOp& L, int64_t p, int par
   constexpr int C = NB == 27 ? 13 : 4;
   float4 sc = make_float4(1.f, 1.f, 1.f, 1.f);
   if (KIND == STORE_F16) sc = reinterpret_cast<const float4*>(L.scale)[p];
-  T a0 = 0, a1 = 0;
+  RowAcc<T> a0, a1;
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     if (skip_centre && b == C) continue;
@@ -308,10 +322,11 @@ __device__ __forceinline__ void stencil_sum(const LevelOp& L, int64_t p, int par
     load_block<KIND>(L.A, L.d.nv, b, p, sc, a);
     const int off = par ? L.nb.off[1][b] : L.nb.off[0][b];
     const typename V2<T>::t xv = ld_xn_plain<SAME, NB>(x + p + off, b);
-    a0 = blk_acc(a0, a[0], a[1], xv);
-    a1 = blk_acc(a1, a[2], a[3], xv);
+    a0.add(a[0], a[1], xv);
+    a1.add(a[2], a[3], xv);
   }
-  s0 = a0; s1 = a1;
+  s0 = a0.value();
+  s1 = a1.value();
 }
 
 // stencil_sum with the loads of CH blocks (and their x values) issued before
@@ -319,7 +334,7 @@ __device__ __forceinline__ void stencil_sum(const LevelOp& L, int64_t p, int par
 // The block loads are the `volatile` streaming loads of load_raw, which the
 // compiler keeps in source order, so placing all CH of them ahead of the sums
 // is what batches them (ordinary loads get sunk back next to their uses).
-// The same blocks are summed in the same order with the same blk_acc, so the
+// The same blocks are summed in the same order with the same RowAcc, so the
 // sums equal stencil_sum's bit for bit.
 // This is what the small levels need, where a thread's chain of round trips,
 // not bandwidth, sets the time.
@@ -339,7 +354,7 @@ __device__ __forceinline__ void stencil_sum_batched(const LevelOp& L, int64_t p,
   constexpr int C = NB == 27 ? 13 : 4;
   float4 sc = make_float4(1.f, 1.f, 1.f, 1.f);
   if (KIND == STORE_F16) sc = reinterpret_cast<const float4*>(L.scale)[p];
-  T a0 = 0, a1 = 0;
+  RowAcc<T> a0, a1;
 #pragma unroll
   for (int b0 = 0; b0 < NB; b0 += CH) {
     RawBlock<KIND> raw[CH];
@@ -363,11 +378,12 @@ __device__ __forceinline__ void stencil_sum_batched(const LevelOp& L, int64_t p,
       if (skip[c]) continue;   // as in the per-block sum
       T a[4];
       unpack_block<KIND>(raw[c], sc, a);
-      a0 = blk_acc(a0, a[0], a[1], xv[c]);
-      a1 = blk_acc(a1, a[2], a[3], xv[c]);
+      a0.add(a[0], a[1], xv[c]);
+      a1.add(a[2], a[3], xv[c]);
     }
   }
-  s0 = a0; s1 = a1;
+  s0 = a0.value();
+  s1 = a1.value();
 }
 
 template <int KIND, int NB, int CH, bool SAME = false>
@@ -603,15 +619,15 @@ __device__ __forceinline__ void row_sum(const LevelOp& L, int64_t p, int par, co
     if (!CENTRE && b == (NB == 27 ? 13 : 4)) continue;
     if (!((mask >> b) & 1u)) xv[b] = ld_xn<SAME, NB>(x + p + (par ? L.nb.off[1][b] : L.nb.off[0][b]), b);
   }
-  float a0 = 0.f, a1 = 0.f;
+  RowAcc<float> a0, a1;
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     if ((!CENTRE && b == (NB == 27 ? 13 : 4)) || ((mask >> b) & 1u)) continue;
-    a0 = blk_acc(a0, R.a[b].x, R.a[b].y, xv[b]);
-    a1 = blk_acc(a1, R.a[b].z, R.a[b].w, xv[b]);
+    a0.add(R.a[b].x, R.a[b].y, xv[b]);
+    a1.add(R.a[b].z, R.a[b].w, xv[b]);
   }
-  s0 = a0;
-  s1 = a1;
+  s0 = a0.value();
+  s1 = a1.value();
 }
 // (A x)_p with A = shift*M - J on the finest level, as apply_row
 template <int NB, bool FINE>
@@ -711,7 +727,7 @@ __device__ __forceinline__ void row_load(const LevelOp& L, int64_t p, int h, uin
 template <int NB, bool CENTRE, bool SAME>
 __device__ __forceinline__ double row_sum(const LevelOp& L, int64_t p, int par, const double2* __restrict__ x, uint32_t mask,
                                           const RowF64<NB>& R) {
-  double s = 0.0;
+  RowAcc<double> s;
 #pragma unroll
   for (int b0 = 0; b0 < NB; b0 += 9) {
     double2 xv[9];
@@ -725,10 +741,10 @@ __device__ __forceinline__ double row_sum(const LevelOp& L, int64_t p, int par, 
     for (int c = 0; c < 9; ++c) {
       const int b = b0 + c;
       if ((!CENTRE && b == (NB == 27 ? 13 : 4)) || ((mask >> b) & 1u)) continue;
-      s = blk_acc(s, R.a[b].x, R.a[b].y, xv[c]);
+      s.add(R.a[b].x, R.a[b].y, xv[c]);
     }
   }
-  return s;
+  return s.value();
 }
 // row h of A x at p with A = shift*M - J on the finest level, as apply_row
 template <int NB, bool FINE>
@@ -1345,7 +1361,7 @@ __device__ __forceinline__ void cl_residual(const ClLevel& L, int lr, int p, int
   if constexpr (KIND == STORE_F64) {
     const double2* sm = reinterpret_cast<const double2*>(L.sA) + h * L.rows + lr;
     const double2* gm = reinterpret_cast<const double2*>(L.A) + (int64_t)p * 2 + h;
-    double a0 = 0.0;
+    RowAcc<double> a0;
     auto sum = [&](auto shared) {
       constexpr int CH = decltype(shared)::value ? 3 : 9;
 #pragma unroll
@@ -1359,17 +1375,17 @@ __device__ __forceinline__ void cl_residual(const ClLevel& L, int lr, int p, int
           if (!skipped(b0 + c)) xv[c] = xat(b0 + c);
 #pragma unroll
         for (int c = 0; c < CH; ++c)
-          if (!skipped(b0 + c)) a0 = blk_acc(a0, a[c].x, a[c].y, xv[c]);
+          if (!skipped(b0 + c)) a0.add(a[c].x, a[c].y, xv[c]);
       }
     };
     if (L.sA) sum(std::true_type{});
     else sum(std::false_type{});
-    const double mine = (h ? bv.y : bv.x) - a0;
+    const double mine = (h ? bv.y : bv.x) - a0.value();
     const double other = __shfl_xor_sync(3u << (threadIdx.x & 30), mine, 1);
     r0 = h ? other : mine;
     r1 = h ? mine : other;
   } else {
-    T a0 = 0, a1 = 0;
+    RowAcc<T> a0, a1;
     auto sum = [&](auto shared) {
       constexpr int CH = 9;
 #pragma unroll
@@ -1387,15 +1403,15 @@ __device__ __forceinline__ void cl_residual(const ClLevel& L, int lr, int p, int
 #pragma unroll
         for (int c = 0; c < CH; ++c)
           if (!skipped(b0 + c)) {
-            a0 = blk_acc(a0, a[c].x, a[c].y, xv[c]);
-            a1 = blk_acc(a1, a[c].z, a[c].w, xv[c]);
+            a0.add(a[c].x, a[c].y, xv[c]);
+            a1.add(a[c].z, a[c].w, xv[c]);
           }
       }
     };
     if (L.sA) sum(std::true_type{});
     else sum(std::false_type{});
-    r0 = bv.x - a0;
-    r1 = bv.y - a1;
+    r0 = bv.x - a0.value();
+    r1 = bv.y - a1.value();
   }
 }
 
@@ -2933,8 +2949,14 @@ __device__ __forceinline__ void shared_row(const LevelOp& L, const SysLevel* G, 
   constexpr int C = NB == 27 ? 13 : 4;
   float4 sc = make_float4(1.f, 1.f, 1.f, 1.f);
   if (KIND == STORE_F16) sc = reinterpret_cast<const float4*>(G[0].scale)[p];
+  RowAcc<T> c0[NS], c1[NS];
+  auto result = [&] {
 #pragma unroll
-  for (int q = 0; q < NS; ++q) { s0[q] = 0; s1[q] = 0; }
+    for (int q = 0; q < NS; ++q) {
+      s0[q] = c0[q].value();
+      s1[q] = c1[q].value();
+    }
+  };
   if constexpr (KIND == STORE_F16) {
     // pairs of slots, in the slot order of stencil_sum_f16
     const uint4* __restrict__ A = reinterpret_cast<const uint4*>(G[0].A);
@@ -2959,11 +2981,12 @@ __device__ __forceinline__ void shared_row(const LevelOp& L, const SysLevel* G, 
         for (int q = 0; q < NS; ++q) {
           if (!act[q]) continue;
           const V xv = ld_xn_plain<SAME, NB>((const V*)G[q].in1 + p + off, b);
-          s0[q] = blk_acc(s0[q], a[0], a[1], xv);
-          s1[q] = blk_acc(s1[q], a[2], a[3], xv);
+          c0[q].add(a[0], a[1], xv);
+          c1[q].add(a[2], a[3], xv);
         }
       }
     }
+    result();
     return;
   }
 #pragma unroll
@@ -2977,10 +3000,11 @@ __device__ __forceinline__ void shared_row(const LevelOp& L, const SysLevel* G, 
     for (int q = 0; q < NS; ++q) {
       if (!act[q]) continue;
       const V xv = ld_xn_plain<SAME, NB>((const V*)G[q].in1 + p + off, b);
-      s0[q] = blk_acc(s0[q], a[0], a[1], xv);
-      s1[q] = blk_acc(s1[q], a[2], a[3], xv);
+      c0[q].add(a[0], a[1], xv);
+      c1[q].add(a[2], a[3], xv);
     }
   }
+  result();
 }
 
 template <int KIND, int NB, int NS>
