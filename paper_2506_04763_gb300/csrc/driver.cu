@@ -839,6 +839,9 @@ static rf_status autotune_levels(rf_grid* g, void* s) {
       auto it = g_tune.find(key);
       if (it != g_tune.end()) { Lv.block = it->second.block; Lv.batched = it->second.batched; continue; }
     }
+    // nothing to choose on a small level: its candidates would be the same launches
+    // (the batched solves' kernels, which have a shape there, take the default)
+    if (level_shape_fixed(level_op(g, l, 0), g->gopt.smoother == RF_SMOOTH_GS8)) continue;
     cudaEvent_t e0, e1;
     CU(cudaEventCreate(&e0));
     CU(cudaEventCreate(&e1));

@@ -3391,6 +3391,11 @@ static void gs_t(const LevelOp& L, const void* b, void* x, bool forward, bool ze
   });
 }
 
+bool level_shape_fixed(const LevelOp& L, bool gs) {
+  int lpb = 1, threads = 32;
+  return L.small && L.kind != STORE_F16 && (!gs || (gs_pairs() && pair_shape(L.d.nx, lpb, threads)));
+}
+
 void launch_residual(const LevelOp& L, const void* b, const void* x, void* r, void* s) {
   switch (L.kind) {
     case STORE_F64: L.fine ? residual_t<STORE_F64, true>(L, b, x, r, s) : residual_t<STORE_F64, false>(L, b, x, r, s); break;

@@ -73,6 +73,8 @@ struct LevelOp {
 };
 
 // Vectors are T2 pointers to the first interior element of padded buffers.
+// whether L's sweeps and residuals have one shape, whatever L.block and L.batched say (the small forms)
+bool level_shape_fixed(const LevelOp& L, bool gs);
 void launch_residual(const LevelOp& L, const void* b, const void* x, void* r, void* s);
 void launch_jacobi(const LevelOp& L, const void* b, const void* xin, void* xout, double omega, bool zero_x,
                    void* s);
