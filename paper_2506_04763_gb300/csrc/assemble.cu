@@ -816,17 +816,23 @@ void launch_perm_scalar_to_p(const Dims& d, const double* nat, double* out, void
   RF_LAUNCH(k_perm_scalar_to_p, (int)((d.nv + 255) / 256), 256, 0, s, d, nat, out);
 }
 
-// Face workspace of one assembly: at most ASM_WS_BYTES (with J; F alone a
-// quarter of that), at least two cell planes.  At 257^3 the ring then holds 3
-// planes of 151 MB, and a slab of 2 is 10 waves of k_asm_faces.  Slabs go along z, or along y where two z planes exceed the
-// limit and y planes are smaller (wide, shallow boxes).
+// Face workspace of one assembly: at most ASM_WS_BYTES (with J; F alone a quarter of
+// that, or what it is given), at least two cell planes.  At 257^3 the ring then holds 3
+// planes of 151 MB, and a slab of 2 is 10 waves of k_asm_faces.  Slabs go along z, or
+// along y where two z planes exceed the limit and y planes are smaller (wide, shallow
+// boxes).  With 256 / 128 / 64 MB, J takes 3 / 10 / 23% longer at 65^3 (1.54 ms with 512)
+// and 7 / 25 / 35% at 129^3 (11.2 ms), F alone 0 / 4 / 14% and 2 / 7 / 16%.
 constexpr size_t ASM_WS_BYTES = (size_t)512 << 20;
 
 struct SlabShape { int ax, planes, ring; int64_t plane; };
 
-static SlabShape slab_shape(const Dims& d, bool want_j) {
-  const size_t cell = (size_t)(d.dim << (d.dim - 1)) * nco(d.dim, want_j) * sizeof(double);
-  const int64_t fit = (int64_t)((want_j ? ASM_WS_BYTES : ASM_WS_BYTES / 4) / cell);   // cells
+static size_t cell_bytes(const Dims& d, bool want_j) {
+  return (size_t)(d.dim << (d.dim - 1)) * nco(d.dim, want_j) * sizeof(double);
+}
+
+static SlabShape slab_shape(const Dims& d, bool want_j, size_t bytes) {
+  const size_t limit = want_j ? ASM_WS_BYTES : ASM_WS_BYTES / 4;
+  const int64_t fit = (int64_t)((bytes < limit ? bytes : limit) / cell_bytes(d, want_j));   // cells
   const int64_t zp = (int64_t)(d.nx - 1) * (d.ny - 1), yp = (int64_t)(d.nx - 1) * (d.dim == 3 ? d.nz - 1 : 1);
   SlabShape r;
   r.ax = d.dim == 3 && (2 * zp <= fit || zp <= yp) ? 2 : 1;
@@ -837,14 +843,14 @@ static SlabShape slab_shape(const Dims& d, bool want_j) {
   return r;
 }
 
-size_t assemble_workspace(const Dims& d, bool want_j) {
-  const SlabShape r = slab_shape(d, want_j);
-  return (size_t)(r.ring * r.plane) * (d.dim << (d.dim - 1)) * nco(d.dim, want_j) * sizeof(double);
+size_t assemble_workspace(const Dims& d) {
+  const SlabShape r = slab_shape(d, true, ASM_WS_BYTES);
+  return (size_t)(r.ring * r.plane) * cell_bytes(d, true);
 }
 
 template <int DIM, bool WANT_J>
 static void slabs_t(const Dims& d, const Phys& ph, const AsmIn& in, const AsmArrays& a, void* s) {
-  const SlabShape sh = slab_shape(d, WANT_J);
+  const SlabShape sh = slab_shape(d, WANT_J, a.faces_bytes);
   const int planes = sh.planes;
   Slab sl;
   sl.ax = sh.ax;

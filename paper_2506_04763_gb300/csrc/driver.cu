@@ -164,7 +164,7 @@ struct rf_grid {
   double *J = nullptr, *mdiag = nullptr;
   bool have_J = false;
   double *Se, *pn, *pc, *dpc, *krw, *dkrw, *krn, *dkrn;
-  double* faces = nullptr;      // workspace of the assembly (column grids: of F alone) and of the Galerkin products
+  double* faces = nullptr;      // workspace of the assembly and of the Galerkin products (column grids: a part of the parent's)
   size_t faces_bytes = 0;
   double *u_p = nullptr, *F_p = nullptr, *nat_a = nullptr, *nat_b = nullptr;
   // multigrid
@@ -639,7 +639,7 @@ extern "C" rf_status rf_grid_create(const rf_grid_desc* desc, const rf_fluids* f
   double** scratch[8] = {&g->Se, &g->pn, &g->pc, &g->dpc, &g->krw, &g->dkrw, &g->krn, &g->dkrn};
   for (auto p : scratch) NEED(*p = (double*)dalloc(g, sizeof(double) * nv, stream, false));
   // (a Galerkin workspace beyond GAL_WS_BYTES, of grids with very large planes, waits for the set-up)
-  g->faces_bytes = std::max(assemble_workspace(d, true), std::min(galerkin_workspace(d), GAL_WS_BYTES));
+  g->faces_bytes = std::max(assemble_workspace(d), std::min(galerkin_workspace(d), GAL_WS_BYTES));
   NEED(g->faces = (double*)dalloc(g, g->faces_bytes, stream, false));
   NEED(g->u_p = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
   NEED(g->F_p = (double*)dalloc(g, sizeof(double) * 2 * nv, stream, false));
@@ -677,7 +677,7 @@ extern "C" rf_status rf_grid_create(const rf_grid_desc* desc, const rf_fluids* f
 static rf_status assemble_p(rf_grid* g, bool want_j, void* s) {
   AsmArrays a;
   a.u = g->u_p; a.Se = g->Se; a.pn = g->pn; a.pc = g->pc; a.dpc = g->dpc; a.krw = g->krw; a.dkrw = g->dkrw;
-  a.krn = g->krn; a.dkrn = g->dkrn; a.faces = g->faces;
+  a.krn = g->krn; a.dkrn = g->dkrn; a.faces = g->faces; a.faces_bytes = g->faces_bytes;
   a.pdmin = g->pdmin; a.phiv = g->phiv; a.K = g->Kcell; a.pd = g->pd; a.phi = g->phi; a.vol = g->vol;
   a.dir = g->dir; a.pw_dir = g->pw_dir;
   a.q_in = g->q_in; a.F = g->F_p; a.J = want_j ? g->J : nullptr; a.mdiag = want_j ? g->mdiag : nullptr;
@@ -1953,7 +1953,6 @@ static rf_status column_grid(rf_grid* g, int j, void* s, rf_grid** out) {
     bool ok = true;
     double** scratch[8] = {&c->Se, &c->pn, &c->pc, &c->dpc, &c->krw, &c->dkrw, &c->krn, &c->dkrn};
     for (auto p : scratch) ok = ok && (*p = (double*)dalloc(c, sizeof(double) * nv, s, false));
-    ok = ok && (c->faces = (double*)dalloc(c, assemble_workspace(d, false), s, false));
     ok = ok && (c->u_p = (double*)dalloc(c, sizeof(double) * 2 * nv, s, false));
     ok = ok && (c->F_p = (double*)dalloc(c, sizeof(double) * 2 * nv, s, false));
     ok = ok && (c->K.x = (double2*)dvec(c, d, sizeof(double), s, false));
@@ -1991,6 +1990,11 @@ static rf_status column_grid(rf_grid* g, int j, void* s, rf_grid** out) {
   c->dir = g->dir; c->pw_dir = g->pw_dir; c->q_in = g->q_in; c->pdmin = g->pdmin; c->phiv = g->phiv;
   c->J = g->J; c->mdiag = g->mdiag; c->have_J = g->have_J;
   c->Jdf = g->Jdf; c->jdf_valid = g->jdf_valid;
+  // F of the columns 1 .. kappa - 1 is assembled at the same time, each in its own
+  // part of the parent's face workspace: the parent assembles before the columns
+  // start and after they have joined its stream (column 0 needs F(u0) only)
+  c->faces_bytes = g->faces_bytes / (RF_MAXSHIFT - 1) / sizeof(double) * sizeof(double);
+  c->faces = g->faces + (size_t)(j - 1) * (c->faces_bytes / sizeof(double));
   // a new hierarchy of the same shape (levels, storage kind, level sizes): keep
   // the column's own level vectors (their zero halos are never written) and
   // mirror the new operators

@@ -19,7 +19,8 @@ struct PhysParams {
 struct AsmArrays {
   const double* u;                 // [2nv] parity-split
   double *Se, *pn, *pc, *dpc, *krw, *dkrw, *krn, *dkrn;  // [nv] scratch
-  double* faces;                   // face workspace (assemble_workspace bytes)
+  double* faces;                   // face workspace: assemble_workspace bytes, for F alone a third of them at least
+  size_t faces_bytes;
   const double *pdmin, *phiv;      // [nv]
   const double *K, *pd, *phi;      // per cell
   double vol;                      // cell volume
@@ -40,8 +41,9 @@ void launch_perm_to_p(const Dims& d, const double* nat, double* out, void* s);
 void launch_perm_from_p(const Dims& d, const double* pl, double* nat, void* s);
 void launch_perm_bytes_to_p(const Dims& d, const uint8_t* nat, uint8_t* out, void* s);
 void launch_perm_scalar_to_p(const Dims& d, const double* nat, double* out, void* s);
-// bytes of the face workspace of an assembly (want_j: the one with J also serves F alone)
-size_t assemble_workspace(const Dims& d, bool want_j);
+// bytes of the face workspace of an assembly with J (F alone: any third of it serves, two planes of 12 (2D: 7)
+// times fewer numbers)
+size_t assemble_workspace(const Dims& d);
 cudaError_t launch_assemble(const Dims& d, const PhysParams& pp, const AsmArrays& a, bool want_j, void* s);
 // S hat storage variant: sw[p] = sum over the sub-control volumes of p of Phi |b| S_w (S hat)
 void launch_storage_sw(const Dims& d, const PhysParams& pp, const double* u, const double* pdmin,
