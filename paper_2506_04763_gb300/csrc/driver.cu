@@ -220,6 +220,9 @@ struct rf_grid {
   IterGraph* cap = nullptr;
   cudaStream_t cs = nullptr;             // internal stream for the iteration
   cudaEvent_t join_in = nullptr, join_out = nullptr;
+  cudaEvent_t f_done = nullptr;          // the last rf_assemble of F alone (f_stream: where it ran)
+  void* f_stream = nullptr;
+  bool f_pending = false;
   // LIMEX columns solved concurrently: column j > 0 runs on col[j], a grid
   // that shares this grid's operator data and hierarchy (read-only) and owns
   // its vectors, scratch, streams and graphs (refreshed after each set-up)
@@ -551,6 +554,7 @@ extern "C" void rf_grid_destroy(rf_grid* g) {
     }
   destroy_graphs(g);
   for (auto e : g->evpool) cudaEventDestroy(e);
+  if (g->f_done) cudaEventDestroy(g->f_done);
   if (g->join_in) cudaEventDestroy(g->join_in);
   if (g->join_out) cudaEventDestroy(g->join_out);
   if (g->cs) cudaStreamDestroy(g->cs);
@@ -660,6 +664,7 @@ extern "C" rf_status rf_grid_create(const rf_grid_desc* desc, const rf_fluids* f
     return fail(RF_ENOMEM, "pinned host allocation failed");
   }
   if (cudaStreamCreateWithFlags(&g->cs, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&g->f_done, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&g->join_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&g->join_out, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
@@ -693,6 +698,17 @@ extern "C" rf_status rf_assemble(rf_grid* g, const double* u, int want_jacobian,
   rf_status st = pairs_in(g, g->d, u, g->u_p, s);
   if (st) return st;
   if ((st = assemble_p(g, want_jacobian != 0, s))) return st;
+  if (!want_jacobian) {
+    // F alone leaves J and the hierarchy in place: a set-up on another stream may
+    // follow at once, and it works in the face workspace too (see rf_gmg_setup)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CU(cudaStreamIsCapturing((cudaStream_t)s, &cap));
+    if (cap == cudaStreamCaptureStatusNone) {
+      CU(cudaEventRecord(g->f_done, (cudaStream_t)s));
+      g->f_stream = s;
+      g->f_pending = true;
+    }
+  }
   if (F_out) return pairs_out(g, g->d, g->F_p, F_out, s);
   return RF_OK;
 }
@@ -1033,6 +1049,8 @@ extern "C" rf_status rf_gmg_setup(rf_grid* g, const double* shifts, int nshift, 
     drop_hierarchy(g, s);
   }
   struct ReplayEnd { rf_grid* g; ~ReplayEnd() { g->replay = -1; } } replay_end{g};
+  if (g->f_pending && g->f_stream != s) CU(cudaStreamWaitEvent((cudaStream_t)s, g->f_done, 0));
+  g->f_pending = false;
   ++g->hier_gen;
   for (int l = 0; l < RF_MAXL; ++l) g->L[l] = Level();
   for (int j = 0; j < RF_MAXSHIFT; ++j) g->Ainv[j] = nullptr;
