@@ -49,11 +49,11 @@ GS_ALGO_PER_VERTEX = 456.0
 # (4 flop) and the fused inner products (<rh, v>: 4 flop; <t, s>, <t, t>: 8
 # flop), averaged over the two applications of an iteration.
 SPMV64_FLOP_PER_VERTEX = 216.0 + 4.0 + 6.0
-# FP64 instructions per vertex of one K1 assembly with the Jacobian: about 1790
-# per element in the face pass (ncu, FP64 pipe instructions at 97^3) and 840 per
-# vertex in the row pass; K1 is FP64-issue-bound, so its roofline is that
-# instruction rate against the FMA issue rate rf_fp64_fma_rate measures.
-K1_FP64_INST_PER_VERTEX = 2630.0
+# FP64-pipe instructions per vertex of one K1 assembly with the Jacobian: 1,821
+# per element in the face pass and 806 per vertex in the row pass (ncu at 97^3);
+# K1 is FP64-issue-bound, so its roofline is that instruction rate against the
+# FMA issue rate rf_fp64_fma_rate measures.
+K1_FP64_INST_PER_VERTEX = 2605.0
 
 
 def args_():

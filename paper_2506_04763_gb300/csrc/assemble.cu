@@ -467,9 +467,9 @@ __global__ void __launch_bounds__(128) k_assemble(Dims d, Phys ph, AsmIn in, dou
 // adding its faces' 768 entries into J colour by colour (4,154 FP64 instructions
 // per vertex; on small grids 8 dependent chains of about 190 us): 257^3 150.9 ->
 // 91.0 ms (52.1 -> 25.2 ms), 65^3 2.79 -> 1.54 ms (1.00 -> 0.47), 17^3 1.57 -> 0.071
-// ms (0.60 -> 0.042), 33^2 0.224 -> 0.039 ms.  About 1790 FP64 instructions per
-// element in the first pass and 840 per vertex in the second, whose pipe is 83%
-// and 80% busy (ncu at 97^3); DRAM below 15% of its peak.  (Summing a row's faces
+// ms (0.60 -> 0.042), 33^2 0.224 -> 0.039 ms.  1,821 FP64-pipe instructions per
+// element in the first pass and 806 per vertex in the second, whose pipe is 83%
+// and 82% busy (ncu at 97^3); DRAM at 10% and 28% of its peak.  (Summing a row's faces
 // before their products with dp_c/dS_n, not to the last bit, took 63.1 ms.)
 // numbers per face: F_w, F_n, and with J the distinct dF_w/dp_w and dF_n/dp_w
 // and the 2^d dF_w/dS_n and dF_n/dS_n

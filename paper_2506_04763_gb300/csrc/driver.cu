@@ -2409,12 +2409,13 @@ static rf_status limex_finish(LimexWork& w, void* s) {
 // Batched rounds (RF_LIMEX_BATCH=1/0 forces the choice; never with the
 // double-FP32 operator).  By default a single step takes them on grids of at
 // least 1M vertices and the concurrent column threads below that, as measured
-// on GB300 for one kappa = 4 step of the lognormal-lenses recipe: 129^3 FP32
-// GMG 206 ms batched against 220 ms concurrent and 264 ms sequential, 257^3
-// 1389 ms against 1661 ms sequential, but 65^3 FP64 105 ms against 90 ms
-// concurrent (there every kernel is latency-bound, and a round lasts as long
-// as its slowest column while the threads let each column run ahead).  An
-// ensemble is always batched (its groups fill the launches).
+// on GB300 for one kappa = 4 step of the lognormal recipe, columns / rounds: 65^3 FP64
+// Jacobi 55 / 70 ms, FP32 GS 36 / 56; 97^3 FP32 GS 92 / 98, Jacobi 95 / 86, FP64
+// Jacobi 181 / 202; 129^3 FP32 GS 209 / 185, Jacobi 206 / 177; 161^3 FP32 GS 398 / 319.
+// On a small grid every kernel is latency-bound, and a round lasts as long as
+// its slowest column while the threads let each column run ahead; on a large one the
+// rounds read J once for all columns.  An ensemble is always batched (its groups
+// fill the launches).
 static bool limex_batched(const rf_limex_opts* o, int64_t nv = -1) {
   if (o->solve.outer != RF_OUTER_FP64) return false;
   const char* e = getenv("RF_LIMEX_BATCH");
@@ -2657,7 +2658,6 @@ extern "C" rf_status rf_limex_step_batched(rf_grid* const* grids, double* const*
     if (c) return fail(c, "problem %d: %s", i, t_err.c_str());
   }
   bool batched = true;
-  bool small = false;
   for (int i = 0; i < nprob; ++i) batched = batched && limex_batched(&o[i]);
   if (!batched) return limex_batched_threads(grids, u, H, nprob, o, infos, max_concurrent, stream);
   int workers = max_concurrent > 0 ? max_concurrent : (nprob < 16 ? nprob : 16);

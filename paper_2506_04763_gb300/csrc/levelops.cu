@@ -676,11 +676,12 @@ __global__ void __launch_bounds__(64) k_jacobi_small(const __grid_constant__ Lev
 template <int NB, bool FINE, int FPX>
 __global__ void __launch_bounds__(GS_PAIR_MAX_THREADS) k_gs_pair_small(const __grid_constant__ LevelOp L,
                                                                        const float2* __restrict__ b, float2* __restrict__ x,
-                                                                       int py, int pz, int lines_y, int nlines, int lpb,
+                                                                       int py, int pz, int lines_y,
                                                                        uint32_t skip_first, uint32_t skip_second) {
-  const int l0 = blockIdx.x * lpb, nl = min(lpb, nlines - l0), v = threadIdx.x;
+  // one line per block, one vertex per thread and run
+  const int l0 = blockIdx.x, v = threadIdx.x;
   const int cnt0 = FPX ? L.d.nx / 2 : (L.d.nx + 1) / 2, cnt1 = FPX ? (L.d.nx + 1) / 2 : L.d.nx / 2;
-  const bool on0 = v < nl * cnt0, on1 = v < nl * cnt1;
+  const bool on0 = v < cnt0, on1 = v < cnt1;
   const int64_t p0 = on0 ? pair_vertex(L.d, l0, v, cnt0, FPX, py, pz, lines_y) : 0;
   const int64_t p1 = on1 ? pair_vertex(L.d, l0, v, cnt1, 1 - FPX, py, pz, lines_y) : 0;
   RowF32<NB> R;
@@ -3265,7 +3266,7 @@ static void for_colours(const Dims& d, bool forward, bool zero_start, bool flip,
   }
 }
 
-// Colour pairs in one launch each (k_gs_pair) on FP32 and FP16 levels;
+// Colour pairs in one launch each (k_gs_pair) on FP32, FP16 and small FP64 levels;
 // RF_GS_PAIRS=0 launches every colour on its own.  Both give bitwise the same
 // sweep.
 static bool gs_pairs() {
@@ -3327,7 +3328,7 @@ static void gs_t(const LevelOp& L, const void* b, void* x, bool forward, bool ze
   typedef typename V2<typename Ty<KIND>::T>::t V;
   // FP64 levels take one launch per colour unless they are small: with pairs
   // the all-FP64 257^3 solve measured 3% slower (its fine smoother 6%), as the
-  // batched FP64 pair kernel needs 129 registers, one 288-thread block per SM
+  // batched FP64 pair kernel needs 131 registers, one 288-thread block per SM
   int lpb = 1, threads = 32;
   if ((KIND != STORE_F64 || L.small) && gs_pairs() && pair_shape(L.d.nx, lpb, threads)) {
     if (L.small) {       // spread over the SMs
@@ -3339,8 +3340,8 @@ static void gs_t(const LevelOp& L, const void* b, void* x, bool forward, bool ze
       const int g = (nlines + lpb - 1) / lpb;
       if (KIND == STORE_F32 && L.small) {
 #define RF_PAIR_SMALL(NBv, F)                                                                                      \
-  RF_LAUNCH_PDL((k_gs_pair_small<NBv, FINE, F>), g, threads, 0, s, L, (const float2*)b, (float2*)x, py, pz, lines_y, \
-                nlines, lpb, s1, s2)
+  RF_LAUNCH_PDL((k_gs_pair_small<NBv, FINE, F>), nlines, threads, 0, s, L, (const float2*)b, (float2*)x, py, pz, lines_y, \
+                s1, s2)
         if (L.d.nb == 27) { if (fpx) RF_PAIR_SMALL(27, 1); else RF_PAIR_SMALL(27, 0); }
         else if (fpx) RF_PAIR_SMALL(9, 1);
         else RF_PAIR_SMALL(9, 0);
