@@ -220,8 +220,7 @@ struct rf_grid {
   IterGraph* cap = nullptr;
   cudaStream_t cs = nullptr;             // internal stream for the iteration
   cudaEvent_t join_in = nullptr, join_out = nullptr;
-  cudaEvent_t f_done = nullptr;          // the last rf_assemble of F alone (f_stream: where it ran)
-  void* f_stream = nullptr;
+  cudaEvent_t f_done = nullptr;          // the last rf_assemble of F alone, while no set-up has waited for it
   bool f_pending = false;
   // LIMEX columns solved concurrently: column j > 0 runs on col[j], a grid
   // that shares this grid's operator data and hierarchy (read-only) and owns
@@ -705,7 +704,6 @@ extern "C" rf_status rf_assemble(rf_grid* g, const double* u, int want_jacobian,
     CU(cudaStreamIsCapturing((cudaStream_t)s, &cap));
     if (cap == cudaStreamCaptureStatusNone) {
       CU(cudaEventRecord(g->f_done, (cudaStream_t)s));
-      g->f_stream = s;
       g->f_pending = true;
     }
   }
@@ -1049,7 +1047,7 @@ extern "C" rf_status rf_gmg_setup(rf_grid* g, const double* shifts, int nshift, 
     drop_hierarchy(g, s);
   }
   struct ReplayEnd { rf_grid* g; ~ReplayEnd() { g->replay = -1; } } replay_end{g};
-  if (g->f_pending && g->f_stream != s) CU(cudaStreamWaitEvent((cudaStream_t)s, g->f_done, 0));
+  if (g->f_pending) CU(cudaStreamWaitEvent((cudaStream_t)s, g->f_done, 0));
   g->f_pending = false;
   ++g->hier_gen;
   for (int l = 0; l < RF_MAXL; ++l) g->L[l] = Level();

@@ -39,3 +39,29 @@ def test_residual_and_setup_on_two_streams(make, levels):
         assert torch.equal(F, want)
         assert np.array_equal(g.apply(rf.RF_OP_VCYCLE, 0, 0, b), cycle)
     g.close()
+
+
+def test_residual_can_still_be_captured():
+    import __graft_entry__ as G
+    G.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    prob = I.lognormal_box(17, 92)
+    g = rf.Grid(prob)
+    u = torch.tensor(prob["u0"], device="cuda")
+    F, want = torch.empty_like(u), torch.empty_like(u)
+    s = torch.cuda.Stream()
+    g.assemble(u, False, want)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        rf.rf_assemble(g.handle, u.data_ptr(), 0, F.data_ptr(), s.cuda_stream)
+    F.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(F, want)
+    g.assemble(u, True)
+    g.gmg_setup([0.1], rf.gmg_opts(3, "gs8", precision="fp32"))
+    x = torch.empty_like(u)
+    assert g.solve(0, F, x, rtol=1e-10)["status"] == rf.RF_OK
+    g.close()
