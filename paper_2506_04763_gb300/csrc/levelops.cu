@@ -2343,15 +2343,14 @@ __global__ void k_dense(Dims d, Nbr nb, const double* __restrict__ J, const doub
 // the cluster keeps rows r, r + cs, ... in shared memory, and every step costs one
 // cluster barrier.  Rows are not swapped; pos and at hold the order that swapping
 // would give (the position of a row, the row at a position).  Step c:
-//   - each CTA's first warp picks its largest |A[row][c]| over rows not yet
-//     used as pivots (the candidates were left by the previous update; the
-//     earlier position on ties) and puts it and its row into every CTA's table;
-//   - after the barrier all take the largest; the first warp computes the
-//     multipliers l = A[row][c] / pivot of the CTA's rows, a lane each, while the
-//     others copy the pivot row from column c on from its owner through distributed
-//     shared memory;
+//   - all take the largest of the CTAs' candidates (the earlier position on ties);
+//     the first warp computes the multipliers l = A[row][c] / pivot of the CTA's
+//     rows, a lane each, while the others copy the pivot row from column c on from its
+//     owner through distributed shared memory;
 //   - every unused row: A[row][t] -= l A[pivot][t] for t > c, and l in the place of
-//     A[row][c]; one warp per row.
+//     A[row][c]; one warp per row, but column c + 1 by the first warp, a lane per row,
+//     before its share: the CTA's largest |A[row][c+1]| then goes to every CTA's table
+//     while the other warps update the rest, and the barrier ends the step.
 // The factors go to D in the order of the positions, the rows at them to piv.  A
 // pivot that is zero or not finite, or a multiplier that is not finite (any NaN
 // of A ends in one of these), sets status.
@@ -2363,8 +2362,9 @@ __global__ void k_dense(Dims d, Nbr nb, const double* __restrict__ J, const doub
 // sums.)
 // The one-CTA k_lu does its N^3 / 3 multiply-adds on one SM's FP64 pipe (2 per
 // clock) with four block barriers per column: 4.5 ms at N = 250 (5^3 vertices), 0.40
-// ms at N = 50 (5^2).  Spread over a cluster: 0.68 ms and 0.09 ms, 2.7 and 1.8 us a
-// step, most of it the chain of barrier, table, reciprocal and row copy.
+// ms at N = 50 (5^2).  Spread over a cluster: 0.51 ms and 0.085 ms, 2.0 and 1.7 us a
+// step, most of it the chain of barrier, table, reciprocal and row copy (with the next
+// candidates chosen after the whole update 0.68 and 0.09 ms).
 constexpr int LU_THREADS = 512, LU_MAX_CS = 16;
 
 struct LuShared {
@@ -2375,7 +2375,7 @@ struct LuShared {
 
 __host__ __device__ inline size_t lu_smem(int N, int cs) {
   const int rows = (N + cs - 1) / cs;
-  return sizeof(LuShared) + sizeof(double) * ((size_t)rows * N + N + 2 * (size_t)rows) +
+  return sizeof(LuShared) + sizeof(double) * ((size_t)rows * N + N + rows) +
          sizeof(int) * (2 * (size_t)N + rows + 2);
 }
 
@@ -2406,8 +2406,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_cluster(int N, double* __rest
   double* A = reinterpret_cast<double*>(lu_raw + sizeof(LuShared));   // [rows][N]
   double* prow = A + (size_t)rows * N;
   double* mult = prow + N;                                            // [rows]
-  unsigned long long* cand = reinterpret_cast<unsigned long long*>(mult + rows);   // [rows]: 0 once used
-  int* pos = reinterpret_cast<int*>(cand + rows);                     // [N]
+  int* pos = reinterpret_cast<int*>(mult + rows);                     // [N]
   int* at = pos + N;                                                  // [N]
   int* step = at + N;                                                 // [rows]: step a local row was pivot of, or -1
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = LU_THREADS >> 5;
@@ -2417,34 +2416,43 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_cluster(int N, double* __rest
     for (int t = lane; t < N; t += 32) {
       const double v = src[t];
       A[lr * N + t] = v;
-      if (t == 0) { cand[lr] = lu_key(v); step[lr] = -1; }
+      if (t == 0) step[lr] = -1;
     }
   }
   for (int t = tid; t < N; t += LU_THREADS) { pos[t] = t; at[t] = t; }
   cl.sync();   // every CTA of the cluster runs before a peer writes into its table
   bool bad = false, finite = true;
+  // (first warp) this lane's candidate for the pivot of column c, then the warp's into
+  // every CTA's table
+  unsigned long long ck;
+  unsigned cp;
+  int crow;
+  double cval;
+  auto none = [&] { ck = 0; cp = N + lane; crow = 0; cval = 0.0; };   // (no candidate: key 0)
+  auto consider = [&](int lr, double v) {
+    const unsigned long long k = lu_key(v);
+    const unsigned q = (unsigned)pos[lr * cs + rank];
+    if (k > ck || (k == ck && k != 0 && q < cp)) { ck = k; cp = q; crow = lr; cval = v; }
+  };
+  auto publish = [&](int c) {
+    const int src = __ffs(__ballot_sync(0xffffffffu, lu_largest(ck, cp))) - 1;
+    const unsigned long long k = __shfl_sync(0xffffffffu, ck, src);
+    const int r = __shfl_sync(0xffffffffu, crow, src);
+    const double v = __shfl_sync(0xffffffffu, cval, src);
+    if (lane < cs) {
+      LuShared& O = *cl.map_shared_rank(&T, lane);
+      O.key[c & 1][rank] = k;
+      O.val[c & 1][rank] = v;
+      O.row[c & 1][rank] = nloc > 0 ? r * cs + rank : 0;
+    }
+  };
+  if (warp == 0) {
+    none();
+    for (int lr = lane; lr < nloc; lr += 32) consider(lr, A[lr * N]);
+    publish(0);
+  }
   for (int c = 0; c < N; ++c) {
     const int par = c & 1;
-    __syncthreads();
-    if (warp == 0) {
-      unsigned long long k = 0;
-      int r = 0;
-      unsigned p = N + lane;                             // (no candidate: key 0)
-      for (int lr = lane; lr < nloc; lr += 32) {
-        const unsigned long long kr = cand[lr];
-        const unsigned q = (unsigned)pos[lr * cs + rank];
-        if (kr > k || (kr == k && kr != 0 && q < p)) { k = kr; r = lr; p = q; }
-      }
-      const int src = __ffs(__ballot_sync(0xffffffffu, lu_largest(k, p))) - 1;
-      k = __shfl_sync(0xffffffffu, k, src);
-      r = __shfl_sync(0xffffffffu, r, src);
-      if (lane < cs) {
-        LuShared& O = *cl.map_shared_rank(&T, lane);
-        O.key[par][rank] = k;
-        O.val[par][rank] = nloc > 0 ? A[r * N + c] : 0.0;
-        O.row[par][rank] = nloc > 0 ? r * cs + rank : 0;
-      }
-    }
     cl.sync();
     const unsigned long long kq = lane < cs ? T.key[par][lane] : 0;
     const int rq = lane < cs ? T.row[par][lane] : 0;
@@ -2453,31 +2461,46 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_cluster(int N, double* __rest
     const unsigned long long k = __shfl_sync(0xffffffffu, kq, best);
     if (k == 0 || k >= 0x7ff0000000000000ULL) { bad = true; break; }   // the same decision in every CTA
     const int pr = __shfl_sync(0xffffffffu, rq, best), p = (int)__shfl_sync(0xffffffffu, pq, best);
-    const int owner = pr % cs, plr = pr / cs;
+    const int owner = pr % cs, plr = rank == owner ? pr / cs : -1;
     if (warp == 0) {
       // (the general division leaves its fast path for a zero, of which there are many)
       const double pv = T.val[par][best], inv = recip(pv);
       for (int lr = lane; lr < nloc; lr += 32) {
         const double l = div_by(A[lr * N + c], pv, inv);
         mult[lr] = l;
-        if (step[lr] < 0 && !(rank == owner && lr == plr))
-          finite = finite && ((__double2hiint(l) & 0x7ff00000) != 0x7ff00000);
+        if (step[lr] < 0 && lr != plr) finite = finite && ((__double2hiint(l) & 0x7ff00000) != 0x7ff00000);
       }
     } else {
-      const double* src = cl.map_shared_rank(A, owner) + plr * N;
+      const double* src = cl.map_shared_rank(A, owner) + (pr / cs) * N;
       for (int t = c + tid - 32; t < N; t += LU_THREADS - 32) prow[t] = src[t];
     }
     __syncthreads();
-    if (tid == 0) {                     // (read again behind the next block barrier)
-      const int q = at[c];
-      at[c] = pr;
-      at[p] = q;
-      pos[q] = p;
-      pos[pr] = c;
+    if (warp == 0) {
+      if (lane == 0) {                  // (the other warps read pos and at behind the next barrier)
+        const int q = at[c];
+        at[c] = pr;
+        at[p] = q;
+        pos[q] = p;
+        pos[pr] = c;
+      }
+      __syncwarp();
+      // column c + 1 of every row first: its candidates are on their way to the other
+      // CTAs while the warps update the rest
+      if (c + 1 < N) {
+        none();
+        for (int lr = lane; lr < nloc; lr += 32) {
+          if (step[lr] >= 0 || lr == plr) continue;
+          const double v = __fma_rn(-mult[lr], prow[c + 1], A[lr * N + c + 1]);
+          A[lr * N + c + 1] = v;
+          consider(lr, v);
+        }
+        __syncwarp();
+        publish(c + 1);
+      }
     }
     for (int lr = warp; lr < nloc; lr += nw) {
-      if (rank == owner && lr == plr) {
-        if (lane == 0) { step[lr] = c; cand[lr] = 0; }
+      if (lr == plr) {
+        if (lane == 0) step[lr] = c;
         continue;
       }
       if (step[lr] >= 0) continue;
@@ -2485,11 +2508,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_cluster(int N, double* __rest
       const double l = mult[lr];
       if (lane == 0) a[c] = l;
 #pragma unroll 2
-      for (int t = c + 1 + lane; t < N; t += 32) {
-        const double v = __fma_rn(-l, prow[t], a[t]);
-        a[t] = v;
-        if (t == c + 1) cand[lr] = lu_key(v);
-      }
+      for (int t = c + 2 + lane; t < N; t += 32) a[t] = __fma_rn(-l, prow[t], a[t]);
     }
   }
   cl.sync();   // no CTA leaves while its rows are read
@@ -2521,8 +2540,8 @@ static cudaLaunchConfig_t lu_config(int nmat, int cs, size_t smem, void* s, cuda
 // Cluster size of k_lu_cluster for N unknowns (0: none).  A step's update takes
 // N ceil(N / cs) multiply-adds of a CTA, its barrier and copies grow with cs.
 // Measured for one inverse, cs = 4 / 8 / 16 (the call's 40 us of launch and
-// read-back included): N = 50 170 / 169 / 180 us, N = 90 329 / 303 / 315, N = 126 516 /
-// 452 / 452, N = 144 700 / 551 / 525, N = 250 1804 / 1263 / 1092.  A size that the
+// read-back included): N = 50 166 / 166 / 169 us, N = 90 302 / 288 / 299, N = 126 437 /
+// 401 / 416, N = 144 597 / 499 / 481, N = 250 1244 / 969 / 918.  A size that the
 // device refuses is passed over: each gives the same factors, bit for bit.
 static int lu_cluster(int N) {
   std::vector<int> sizes;
